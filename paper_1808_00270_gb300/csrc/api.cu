@@ -160,13 +160,13 @@ void invalidate_graph(gld_ctx* c)
     if (c->gexec) cudaGraphExecDestroy(c->gexec);
     c->gexec = nullptr;
     c->graph_failed = false;
-    c->conv_valid_step = -1;
+    c->conv_valid_step = c->part_step = -1;
 }
 
 gld_status invalidate_noise(gld_ctx* c)
 {
     c->noise_valid = false;
-    c->conv_valid_step = -1;
+    c->conv_valid_step = c->part_step = -1;
     long long w[2] = {0, 1};  // {w_hi, w_lo}: w_hi < w_lo marks the W ring empty
     GLD_CUDA(c, cudaMemcpyAsync(&c->B.ctrl->w_hi, w, sizeof(w), cudaMemcpyHostToDevice, c->st));
     return GLD_OK;
@@ -186,7 +186,7 @@ gld_status ring_form(gld_ctx* c, bool alone, cudaStream_t s)
     c->P.wsplit = want;
     invalidate_graph(c);
     c->noise_valid = false;
-    c->conv_valid_step = -1;
+    c->conv_valid_step = c->part_step = -1;
     GLD_CUDA(c, cudaMemsetAsync(c->W, 0, sizeof(float) * (size_t)c->P.lw * 3 * c->P.n_pad, s));
     long long w[2] = {0, 1};  // {w_hi, w_lo}: empty
     GLD_CUDA(c, cudaMemcpyAsync(&c->B.ctrl->w_hi, w, sizeof(w), cudaMemcpyHostToDevice, s));
@@ -223,14 +223,41 @@ cudaError_t launch_noise(gld_ctx* c, cudaStream_t s)
     return e;
 }
 
-// The memory sums of step n: the history convolution, or its recursive form
-// when memory modes are set.
+// The convolution of step n, whose index the device holds in ctrl->step (or,
+// next, in ctrl->conv_step).  Blocks of conv_len steps start at `origin` and
+// every conv_len steps on: their first step forms the parts, the others resume
+// their sums from them (*part_step: first step of the block the parts belong
+// to); a step whose block has none streams the whole ring.  All give the same
+// bits.
+cudaError_t launch_conv(gld_ctx* c, long long n, long long origin, long long* part_step, bool next, cudaStream_t s)
+{
+    const StepParams& P = c->P;
+    int t = -1;
+    if (P.cblk) {
+        const int rel = (int)((n - origin) % c->conv_len);
+        if (rel == 0) {
+            const cudaError_t e =
+                launch_conv_pre(c->B.ring, P.hist_bf16, P.n_pad, P.m_max, next ? &c->B.ctrl->conv_step : &c->B.ctrl->step,
+                                c->coef, P.nacc, c->B.part, c->conv_G, c->conv_len, c->prm.kahan, s);
+            if (e != cudaSuccess) return e;
+            *part_step = n;
+        }
+        if (*part_step == n - rel) t = rel;
+    }
+    return next ? launch_hist_conv_next(c->B.ring, P.hist_bf16, P.n_pad, P.m_max, c->B.ctrl, c->coef, P.nacc, c->B.conv,
+                                        c->prm.kahan, s, c->B.part, t, c->conv_len)
+                : launch_hist_conv(c->B.ring, P.hist_bf16, P.n_pad, P.m_max, c->B.ctrl, 0, c->coef, P.nacc, c->B.conv,
+                                   c->prm.kahan, s, c->B.part, t, c->conv_len);
+}
+
+// The memory sums of the current step (of a noise block that has begun): the
+// history convolution, or its recursive form when memory modes are set.
 cudaError_t launch_memory(gld_ctx* c, cudaStream_t s)
 {
     if (c->P.nmodes > 0)
         return launch_modes_step(c->P, c->B.ctrl, c->B.ring, c->d_mcoef, c->d_mw, c->d_Y, c->B.conv, s);
-    return launch_hist_conv(c->B.ring, c->P.hist_bf16, c->P.n_pad, c->P.m_max, c->B.ctrl, 0, c->coef, c->P.nacc,
-                            c->B.conv, c->prm.kahan, s);
+    if (c->conv_valid_step == c->host_step) return cudaSuccess;  // formed beside the previous step
+    return launch_conv(c, c->host_step, c->block_start, &c->part_step, false, s);
 }
 
 // Rebuilds the auxiliary sums of the recursive form from the ring when the
@@ -263,36 +290,45 @@ cudaError_t launch_one_step(gld_ctx* c, cudaStream_t s)
 // capture stream right after the pair kernel: it reads only the ring the pair
 // kernel has just written, so it runs beside the rebuild, F^C, VACF and pair
 // correlation kernels and is joined before the next pair kernel.
-cudaError_t capture_fork_next(gld_ctx* c, cudaStream_t s)
+// (t: number of the step in the graph, which begins with a block of the
+// convolution).
+cudaError_t capture_fork_next(gld_ctx* c, int t, cudaStream_t s)
 {
     cudaError_t e = cudaEventRecord(c->ev_fork, s);
     if (e == cudaSuccess) e = cudaStreamWaitEvent(c->cap3, c->ev_fork, 0);
-    if (e == cudaSuccess)
-        e = launch_hist_conv_next(c->B.ring, c->P.hist_bf16, c->P.n_pad, c->P.m_max, c->B.ctrl, c->coef, c->P.nacc,
-                                  c->B.conv, c->prm.kahan, c->cap3);
+    long long part_step = c->P.cblk ? (t + 1) / c->conv_len * c->conv_len : 0;  // by an earlier step of the block
+    if (e == cudaSuccess) e = launch_conv(c, t + 1, 0, &part_step, true, c->cap3);
     if (e == cudaSuccess) e = cudaEventRecord(c->ev_join, c->cap3);
     return e;
 }
 
-cudaError_t capture_step_gated(gld_ctx* c, cudaStream_t s, bool overlap)
+// A step that is not overlapped computes its own memory sums first.
+cudaError_t capture_memory(gld_ctx* c, int t, cudaStream_t s)
 {
-    if (!overlap) return launch_one_step(c, s);
-    cudaError_t e = launch_pair_noise(c->P, c->B, c->d_zblk, c->d_bvec, s);
+    if (c->P.nmodes > 0) return launch_memory(c, s);
+    long long part_step = c->P.cblk ? t / c->conv_len * c->conv_len : 0;
+    return launch_conv(c, t, 0, &part_step, false, s);
+}
+
+cudaError_t capture_step_gated(gld_ctx* c, cudaStream_t s, bool overlap, int t)
+{
+    cudaError_t e = overlap ? cudaSuccess : capture_memory(c, t, s);
+    if (e == cudaSuccess) e = launch_pair_noise(c->P, c->B, c->d_zblk, c->d_bvec, s);
     if (e == cudaSuccess) e = launch_pair_force_integrate(c->P, c->B, s);
-    if (e == cudaSuccess) e = capture_fork_next(c, s);
+    if (overlap && e == cudaSuccess) e = capture_fork_next(c, t, s);
     if (e == cudaSuccess) e = launch_rebuild(c->P, c->B, s);
     if (e == cudaSuccess) e = launch_cforce(c->P, c->B, 1, s);
     if (e == cudaSuccess) e = launch_pcorr(c->P, c->B, s);
-    if (e == cudaSuccess) e = cudaStreamWaitEvent(s, c->ev_join, 0);
+    if (overlap && e == cudaSuccess) e = cudaStreamWaitEvent(s, c->ev_join, 0);
     return e;
 }
 
-cudaError_t capture_step_conditional(gld_ctx* c, cudaStream_t s, bool overlap)
+cudaError_t capture_step_conditional(gld_ctx* c, cudaStream_t s, bool overlap, int t)
 {
-    cudaError_t e = overlap ? cudaSuccess : launch_memory(c, s);
+    cudaError_t e = overlap ? cudaSuccess : capture_memory(c, t, s);
     if (e == cudaSuccess) e = launch_pair_noise(c->P, c->B, c->d_zblk, c->d_bvec, s);
     if (e == cudaSuccess) e = launch_pair_force_integrate(c->P, c->B, s);
-    if (overlap && e == cudaSuccess) e = capture_fork_next(c, s);
+    if (overlap && e == cudaSuccess) e = capture_fork_next(c, t, s);
     cudaStreamCaptureStatus cs;
     cudaGraph_t g = nullptr;
     const cudaGraphNode_t* deps = nullptr;
@@ -570,7 +606,7 @@ bool capture_graph_mode(gld_ctx* c, bool conditional)
     if (ok) {
         cudaError_t e = launch_noise(c, c->cap);
         for (int t = 0; t < c->P.T && e == cudaSuccess; ++t)
-            e = conditional ? capture_step_conditional(c, c->cap, overlap) : capture_step_gated(c, c->cap, overlap);
+            e = conditional ? capture_step_conditional(c, c->cap, overlap, t) : capture_step_gated(c, c->cap, overlap, t);
         const cudaError_t e2 = cudaStreamEndCapture(c->cap, &g);
         ok = e == cudaSuccess && e2 == cudaSuccess && g != nullptr;
     }
@@ -719,6 +755,10 @@ size_t ctx_bytes_needed(const gld_params* p, int Q, int Qs, int nr, int num_sms)
         8 * (size_t)(1 + 2 * kMaxQ) * P.m_max, 4 * np, 4 * (size_t)std::max(nt, 1) * nrr};
     size_t total = 0;
     for (size_t b : sizes) total += b == 0 ? 256 : (b + 255) & ~(size_t)255;
+    int G = 0, len = 0;
+    size_t part = 0;
+    if (1 + nt <= kMaxAcc && conv_block_shape(P.hist_bf16, P.n_pad, P.m_max, 1 + nt, p->kahan, &G, &len, &part) == cudaSuccess)
+        total += (part + 255) & ~(size_t)255;
     return total;
 }
 
@@ -927,6 +967,9 @@ gld_status gld_set_kernels(gld_ctx* c, const double* Ks, int32_t Q, const double
     c->fptab = nullptr;
     c->B.fptab = nullptr;
     kry_release(c);
+    dfree(c, c->B.part);
+    c->B.part = nullptr;
+    c->P.cblk = 0;
     const int M = c->P.m_max;
     std::vector<double> in((size_t)(1 + 2 * kMaxQ) * M, 0.0);
     std::memcpy(in.data(), Ks, sizeof(double) * M);
@@ -1008,6 +1051,15 @@ gld_status gld_set_kernels(gld_ctx* c, const double* Ks, int32_t Q, const double
             const double sm = in[(size_t)a * P.m_max + m];  // rows: K^s, g_1..g_Q, gs_1..gs_Qs
             c->wts[(size_t)a * P.m_max + m] = conv == GLD_KDISCRETE ? sm : (m == 0 ? 0.5 : 1.0) * dt * sm;
         }
+    // Parts of a block of steps for the convolution; a context without room for
+    // them streams the whole ring in every step instead.
+    size_t part_bytes = 0;
+    GLD_CUDA(c, conv_block_shape(P.hist_bf16, P.n_pad, P.m_max, P.nacc, c->prm.kahan, &c->conv_G, &c->conv_len, &part_bytes));
+    if (part_bytes) {
+        c->B.part = (float*)dalloc(c, part_bytes);
+        if (!c->B.part) cudaGetLastError();
+        P.cblk = c->B.part ? 1 : 0;
+    }
     P.nmodes = 0;  // new kernels: back to the ring convolution until modes are set again
     P.pn_deg = 0;  // and to the self-kernel noise until the pair noise is set again
     P.perp = 0;    // and to parallel components only
@@ -1029,11 +1081,14 @@ gld_status gld_step(gld_ctx* c, int64_t nsteps)
         if (!c->noise_valid || c->host_step >= c->noise_end) {
             if (c->prm.use_graphs && nsteps >= T && capture_graph(c)) {
                 // the overlapped graph starts from the projections of its first step
-                if (c->overlap_graph && c->conv_valid_step != c->host_step) GLD_CUDA(c, launch_memory(c, c->st));
-                GLD_CUDA(c, cudaGraphLaunch(c->gexec, c->st));
+                // (and the parts of their block)
                 c->block_start = c->host_step;
+                if (c->P.cblk && c->part_step != c->host_step) c->conv_valid_step = -1;
+                if (c->overlap_graph) GLD_CUDA(c, launch_memory(c, c->st));
+                GLD_CUDA(c, cudaGraphLaunch(c->gexec, c->st));
                 c->host_step += T;
                 c->conv_valid_step = c->overlap_graph ? c->host_step : -1;
+                c->part_step = c->overlap_graph && c->P.cblk ? c->host_step : -1;
                 c->noise_end = c->host_step;
                 c->noise_valid = true;
                 c->last_fr_row = T - 1;
@@ -1137,7 +1192,7 @@ gld_status gld_get_array(gld_ctx* c, int32_t which, double* out)
 
 gld_status gld_set_array(gld_ctx* c, int32_t which, const double* in)
 {
-    if (c) c->conv_valid_step = -1;
+    if (c) c->conv_valid_step = c->part_step = -1;
     if (!c || !in) return GLD_E_INVAL;
     GLD_TRY(sync_and_check(c));
     const StepParams& P = c->P;
@@ -1286,7 +1341,7 @@ gld_status gld_profile_steps(gld_ctx* c, int64_t nsteps, double* ms, int64_t* la
     GLD_TRY(ring_form(c, true, c->st));
     GLD_TRY(refresh_modes(c));
     GLD_TRY(sync_and_check(c));
-    c->conv_valid_step = -1;  // the eager steps below leave no next-step projections
+    c->conv_valid_step = c->part_step = -1;  // the eager steps below leave no next-step projections
     const int T = c->P.T;
     const int64_t blocks = (nsteps + T - 1) / T;
     // Per noise block: a short delay kernel lets the host enqueue the whole
@@ -2293,7 +2348,7 @@ gld_status batch_plan(gld_batch* b, int schedule)
 {
     const auto& ms = b->members;
     std::vector<SysDesc> desc(ms.size());
-    std::vector<Tile> pair, part, cell, vacf, conv, fir, cf;
+    std::vector<Tile> pair, part, cell, vacf, conv, fir, cf, pre;
     BatchPlan& P = b->plan;
     P = BatchPlan{};
     P.pair_fast = 1;
@@ -2330,6 +2385,8 @@ gld_status batch_plan(gld_batch* b, int schedule)
         for (int k = 0; k < d.nb_cell; ++k) cell.push_back(Tile{(int)m, k, d.nb_cell, 0});
         for (int k = 0; k < d.nb_vacf; ++k) vacf.push_back(Tile{(int)m, k, d.nb_vacf, 0});
         for (int k = 0; k < d.nb_fir; ++k) fir.push_back(Tile{(int)m, k, d.nb_fir, 0});
+        const int npre = c->P.cblk ? batch_pre_tiles(c->P.n_pad) : 0;
+        for (int k = 0; k < npre; ++k) pre.push_back(Tile{(int)m, k, npre, 0});
         P.max_H = std::max(P.max_H, c->P.H);
         P.max_n = std::max(P.max_n, c->P.n);
         P.max_ntaps = std::max(P.max_ntaps, d.ntaps);
@@ -2351,7 +2408,7 @@ gld_status batch_plan(gld_batch* b, int schedule)
     };
     const size_t o_pair = append(pair, &P.n_pair), o_part = append(part, &P.n_part), o_cell = append(cell, &P.n_cell),
                  o_vacf = append(vacf, &P.n_vacf), o_conv = append(conv, &P.n_conv), o_fir = append(fir, &P.n_fir),
-                 o_cf = append(cf, &P.n_cf);
+                 o_cf = append(cf, &P.n_cf), o_pre = append(pre, &P.n_pre);
     b->snap = desc;
     // One upload of descriptors and tiles through pinned staging, ordered on
     // the batch's stream after the blocks already queued (which keep reading
@@ -2395,6 +2452,7 @@ gld_status batch_plan(gld_batch* b, int schedule)
     P.conv = t0 + o_conv;
     P.fir = t0 + o_fir;
     P.cf = t0 + o_cf;
+    P.pre = t0 + o_pre;
     return GLD_OK;
 }
 
@@ -2402,7 +2460,7 @@ cudaError_t batch_launch_block(gld_batch* b, cudaStream_t s)
 {
     cudaError_t e = launch_batch_noise(b->plan, s);
     for (int t = 0; t < kMaxNoiseBlock && e == cudaSuccess; ++t) {
-        e = launch_batch_conv(b->plan, s);
+        e = launch_batch_conv(b->plan, t, s);
         if (e == cudaSuccess) e = launch_batch_particles(b->plan, s);
     }
     return e;
@@ -2421,8 +2479,9 @@ gld_status batch_autotune(gld_batch* b)
     for (int sc = 0; sc < 4; ++sc) {
         GLD_TRY(batch_plan(b, sc));
         float ms = 0.f;
-        bool ok = launch_batch_conv(b->plan, b->st) == cudaSuccess && cudaEventRecord(e0, b->st) == cudaSuccess;
-        for (int r = 0; r < 5 && ok; ++r) ok = launch_batch_conv(b->plan, b->st) == cudaSuccess;
+        // (step 0 of a block forms its parts; step 1 is what most steps launch)
+        bool ok = launch_batch_conv(b->plan, 0, b->st) == cudaSuccess && cudaEventRecord(e0, b->st) == cudaSuccess;
+        for (int r = 0; r < 5 && ok; ++r) ok = launch_batch_conv(b->plan, 1, b->st) == cudaSuccess;
         ok = ok && cudaEventRecord(e1, b->st) == cudaSuccess && cudaEventSynchronize(e1) == cudaSuccess &&
              cudaEventElapsedTime(&ms, e0, e1) == cudaSuccess;
         if (!ok) {
@@ -2548,7 +2607,7 @@ gld_status gld_batch_step(gld_batch* b, int64_t nsteps)
         const cudaError_t e = b->gexec ? cudaGraphLaunch(b->gexec, b->st) : batch_launch_block(b, b->st);
         if (e != cudaSuccess) return bfail(b, GLD_E_CUDA, std::string("gld_batch_step: ") + cudaGetErrorString(e));
         for (gld_ctx* c : b->members) {
-            c->conv_valid_step = -1;
+            c->conv_valid_step = c->part_step = -1;
             c->block_start = c->host_step;
             c->host_step += kMaxNoiseBlock;
             c->noise_end = c->host_step;

@@ -99,6 +99,8 @@ struct StepParams {
     // the white-noise ring holds the FP16 split of each value (the form the
     // tensor-core filter multiplies) instead of FP32
     int wsplit;
+    // the convolution resumes its sums from parts formed for blocks of steps
+    int cblk;
 };
 
 // ---------------------------------------------------------------- Philox --

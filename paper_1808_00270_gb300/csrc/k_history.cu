@@ -23,241 +23,11 @@
 // end (measured: 768 CTAs on 760 resident slots cost +50 % at 262144
 // particles).  Only when the columns exceed one full wave does the grid
 // become persistent, each thread taking columns q, q + grid, ...
-#include <algorithm>
-#include <map>
-#include <mutex>
-#include <tuple>
-#include <type_traits>
-
-#include <cuda_bf16.h>
-
-#include "launch.h"
+#include "history.cuh"
 
 namespace gld {
 
 namespace {
-
-constexpr int kThreads = 256;     // largest block; the launch picks 64 .. 256
-constexpr int kUnroll = 8;         // loads issued together per thread
-
-template <bool KAHAN>
-__device__ __forceinline__ void acc1(float& s, float& comp, float c, float v)
-{
-    if (KAHAN) {
-        const float y = fmaf(c, v, -comp);
-        const float t = s + y;
-        comp = (t - s) - y;
-        s = t;
-    } else {
-        s = fmaf(c, v, s);
-    }
-}
-
-template <int NACC>
-__device__ __forceinline__ void stage_coefs(float* cs, const float* __restrict__ coef, int M, int H,
-                                            long long n)
-{
-    int r0 = (int)((n - 1) % H);  // slot s holds m = ((n - 1 - s) mod H) + 1
-    if (r0 < 0) r0 += H;
-    for (int s = threadIdx.x; s < H; s += blockDim.x) {
-        const int r = r0 - s;
-        const int m = (r < 0 ? r + H : r) + 1;
-#pragma unroll
-        for (int a = 0; a < NACC; ++a) cs[s * NACC + a] = __ldg(coef + a * M + m);
-    }
-    __syncthreads();
-}
-
-__device__ __forceinline__ float bf_lo(uint32_t w) { return __uint_as_float(w << 16); }
-__device__ __forceinline__ float bf_hi(uint32_t w) { return __uint_as_float(w & 0xffff0000u); }
-
-template <bool BF16>
-struct Col {
-    using V = typename std::conditional<BF16, uint4, float4>::type;
-    static constexpr int W = BF16 ? 8 : 4;  // values per 16-byte column
-};
-
-template <bool BF16>
-__device__ __forceinline__ void unpack(const typename Col<BF16>::V v, float (&x)[Col<BF16>::W])
-{
-    if constexpr (BF16) {
-        x[0] = bf_lo(v.x); x[1] = bf_hi(v.x); x[2] = bf_lo(v.y); x[3] = bf_hi(v.y);
-        x[4] = bf_lo(v.z); x[5] = bf_hi(v.z); x[6] = bf_lo(v.w); x[7] = bf_hi(v.w);
-    } else {
-        x[0] = v.x; x[1] = v.y; x[2] = v.z; x[3] = v.w;
-    }
-}
-
-// One 16-byte column per thread over all slots, one wave (the common case;
-// the lean form keeps the register count at 44 for two FP32 accumulators).
-// Two FP32 accumulators fit in 40 registers: 6 CTAs of 256 threads per SM,
-// enough for one wave of the 262144-particle suspension (768 CTAs).
-template <int NACC, bool KAHAN, bool BF16>
-__global__ void __launch_bounds__(kThreads, (NACC * Col<BF16>::W * (KAHAN ? 2 : 1) <= 8) ? 6 : 1)
-    hist_conv_col(const typename Col<BF16>::V* __restrict__ ring, long long cols, int H,
-                  const float* __restrict__ coef, int M, const long long* __restrict__ nstep, long long step,
-                  float* __restrict__ out)
-{
-    using V = typename Col<BF16>::V;
-    constexpr int VW = Col<BF16>::W;
-    extern __shared__ float cs[];
-    const long long n = nstep ? *nstep : step;
-    stage_coefs<NACC>(cs, coef, M, H, n);
-    const long long q = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (q >= cols) return;
-    float acc[NACC][VW];
-    float cmp[KAHAN ? NACC : 1][VW];
-#pragma unroll
-    for (int a = 0; a < NACC; ++a)
-#pragma unroll
-        for (int e = 0; e < VW; ++e) acc[a][e] = 0.f;
-#pragma unroll
-    for (int a = 0; a < (KAHAN ? NACC : 1); ++a)
-#pragma unroll
-        for (int e = 0; e < VW; ++e) cmp[a][e] = 0.f;
-    const V* p = ring + q;
-    int s = 0;
-    for (; s + kUnroll <= H; s += kUnroll) {
-        V v[kUnroll];
-#pragma unroll
-        for (int u = 0; u < kUnroll; ++u) v[u] = __ldcs(p + (long long)(s + u) * cols);
-#pragma unroll
-        for (int u = 0; u < kUnroll; ++u) {
-            float x[VW];
-            unpack<BF16>(v[u], x);
-#pragma unroll
-            for (int a = 0; a < NACC; ++a) {
-                const float cf = cs[(s + u) * NACC + a];
-#pragma unroll
-                for (int e = 0; e < VW; ++e) acc1<KAHAN>(acc[a][e], cmp[KAHAN ? a : 0][e], cf, x[e]);
-            }
-        }
-    }
-    for (; s < H; ++s) {
-        float x[VW];
-        unpack<BF16>(__ldcs(p + (long long)s * cols), x);
-#pragma unroll
-        for (int a = 0; a < NACC; ++a) {
-            const float cf = cs[s * NACC + a];
-#pragma unroll
-            for (int e = 0; e < VW; ++e) acc1<KAHAN>(acc[a][e], cmp[KAHAN ? a : 0][e], cf, x[e]);
-        }
-    }
-    float4* o = (float4*)out;
-    const long long cols4 = cols * (VW / 4);
-#pragma unroll
-    for (int a = 0; a < NACC; ++a)
-#pragma unroll
-        for (int h = 0; h < VW / 4; ++h) {
-            float r[4];
-#pragma unroll
-            for (int e = 0; e < 4; ++e) r[e] = KAHAN ? acc[a][4 * h + e] - cmp[KAHAN ? a : 0][4 * h + e] : acc[a][4 * h + e];
-            o[a * cols4 + q * (VW / 4) + h] = make_float4(r[0], r[1], r[2], r[3]);
-        }
-}
-
-// One 16-byte column (4 FP32 or 8 BF16 values) per thread and slot group.
-// The G threads of a column split its slots into G contiguous ranges and are
-// combined in shared memory in a fixed order.  Loads run as a rolling
-// pipeline: a register is refilled with the slot kUnroll ahead as soon as it
-// is consumed, so kUnroll loads per thread stay in flight.
-template <int NACC, bool KAHAN, bool BF16>
-__global__ void __launch_bounds__(kThreads)
-    hist_conv(const typename Col<BF16>::V* __restrict__ ring, long long cols, int H, const float* __restrict__ coef,
-              int M, const long long* __restrict__ nstep, long long step, float* __restrict__ out, int G)
-{
-    using V = typename Col<BF16>::V;
-    constexpr int VW = Col<BF16>::W;
-    extern __shared__ float cs[];
-    __shared__ float4 red[kThreads * (BF16 ? 2 : 1)];
-    const long long n = nstep ? *nstep : step;
-    stage_coefs<NACC>(cs, coef, M, H, n);
-    const int per = blockDim.x / G;  // columns per block
-    const int g = threadIdx.x / per, c = threadIdx.x - g * per;
-    const int s_lo = (int)((long long)g * H / G), s_hi = (int)((long long)(g + 1) * H / G);
-    for (long long qb = (long long)blockIdx.x * per; qb < cols; qb += (long long)gridDim.x * per) {
-        const long long q = qb + c;
-        float acc[NACC][VW];
-        float cmp[KAHAN ? NACC : 1][VW];
-#pragma unroll
-        for (int a = 0; a < NACC; ++a)
-#pragma unroll
-            for (int e = 0; e < VW; ++e) acc[a][e] = 0.f;
-#pragma unroll
-        for (int a = 0; a < (KAHAN ? NACC : 1); ++a)
-#pragma unroll
-            for (int e = 0; e < VW; ++e) cmp[a][e] = 0.f;
-        if (q < cols) {
-            const V* p = ring + q;
-            int s = s_lo;
-            for (; s + kUnroll <= s_hi; s += kUnroll) {
-                V v[kUnroll];
-#pragma unroll
-                for (int u = 0; u < kUnroll; ++u) v[u] = __ldcs(p + (long long)(s + u) * cols);
-#pragma unroll
-                for (int u = 0; u < kUnroll; ++u) {
-                    float x[VW];
-                    unpack<BF16>(v[u], x);
-#pragma unroll
-                    for (int a = 0; a < NACC; ++a) {
-                        const float cf = cs[(s + u) * NACC + a];
-#pragma unroll
-                        for (int e = 0; e < VW; ++e) acc1<KAHAN>(acc[a][e], cmp[KAHAN ? a : 0][e], cf, x[e]);
-                    }
-                }
-            }
-            for (; s < s_hi; ++s) {
-                float x[VW];
-                unpack<BF16>(__ldcs(p + (long long)s * cols), x);
-#pragma unroll
-                for (int a = 0; a < NACC; ++a) {
-                    const float cf = cs[s * NACC + a];
-#pragma unroll
-                    for (int e = 0; e < VW; ++e) acc1<KAHAN>(acc[a][e], cmp[KAHAN ? a : 0][e], cf, x[e]);
-                }
-            }
-            if constexpr (KAHAN) {
-#pragma unroll
-                for (int a = 0; a < NACC; ++a)
-#pragma unroll
-                    for (int e = 0; e < VW; ++e) acc[a][e] -= cmp[a][e];  // compensated value
-            }
-        }
-        float4* o = (float4*)out;
-        const long long cols4 = cols * (VW / 4);  // float4 per accumulator row
-        if (G == 1) {
-            if (q < cols)
-#pragma unroll
-                for (int a = 0; a < NACC; ++a)
-#pragma unroll
-                    for (int h = 0; h < VW / 4; ++h)
-                        o[a * cols4 + q * (VW / 4) + h] =
-                            make_float4(acc[a][4 * h], acc[a][4 * h + 1], acc[a][4 * h + 2], acc[a][4 * h + 3]);
-        } else {
-            // fixed-order combine of the G slot ranges, one accumulator at a time
-#pragma unroll
-            for (int a = 0; a < NACC; ++a) {
-#pragma unroll
-                for (int h = 0; h < VW / 4; ++h)
-                    red[threadIdx.x * (VW / 4) + h] =
-                        make_float4(acc[a][4 * h], acc[a][4 * h + 1], acc[a][4 * h + 2], acc[a][4 * h + 3]);
-                __syncthreads();
-                if (g == 0 && q < cols) {
-#pragma unroll
-                    for (int h = 0; h < VW / 4; ++h) {
-                        float4 t = red[c * (VW / 4) + h];
-                        for (int gg = 1; gg < G; ++gg) {
-                            const float4 y = red[(gg * per + c) * (VW / 4) + h];
-                            t.x += y.x; t.y += y.y; t.z += y.z; t.w += y.w;
-                        }
-                        o[a * cols4 + q * (VW / 4) + h] = t;
-                    }
-                }
-                __syncthreads();
-            }
-        }
-    }
-}
 
 // Launch shape (see the header).  Registers are allocated per warp, so small
 // blocks can use every warp slot the registers allow (44 registers: 42 warps
@@ -285,54 +55,12 @@ cudaError_t one_wave_block(K kern, long long items, size_t smem, int* block, lon
     return cudaSuccess;
 }
 
-// A launch decision, cached per (device, columns, slots) for each
-// instantiation: the occupancy queries cost far more host time than a launch.
-struct Shape {
-    int kind;  // 0: one column per thread, 1: general kernel
-    int block, G;
-    unsigned grid;
-};
-
-template <int NACC, bool KAHAN, bool BF16>
-cudaError_t choose_shape(long long cols, int H, size_t smem, Shape* out);
-
-template <int NACC, bool KAHAN, bool BF16>
-cudaError_t launch_tb(const void* ring, int n_pad, int M, const long long* nstep, long long step, const float* coef,
-                      float* out, cudaStream_t st)
-{
-    using V = typename Col<BF16>::V;
-    static std::mutex mu;
-    static std::map<std::tuple<int, long long, int>, Shape> cache;
-    const int H = M - 1;
-    const size_t smem = sizeof(float) * (size_t)H * NACC;
-    const long long cols = 3LL * n_pad / Col<BF16>::W;
-    int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e != cudaSuccess) return e;
-    Shape sh{};
-    {
-        std::lock_guard<std::mutex> lock(mu);
-        auto it = cache.find({dev, cols, H});
-        if (it != cache.end()) {
-            sh = it->second;
-        } else {
-            if ((e = choose_shape<NACC, KAHAN, BF16>(cols, H, smem, &sh)) != cudaSuccess) return e;
-            cache[{dev, cols, H}] = sh;
-        }
-    }
-    if (sh.kind == 0)
-        hist_conv_col<NACC, KAHAN, BF16><<<sh.grid, sh.block, smem, st>>>((const V*)ring, cols, H, coef, M, nstep, step,
-                                                                          out);
-    else
-        hist_conv<NACC, KAHAN, BF16><<<sh.grid, sh.block, smem, st>>>((const V*)ring, cols, H, coef, M, nstep, step,
-                                                                      out, sh.G);
-    return cudaGetLastError();
-}
-
 template <int NACC, bool KAHAN, bool BF16>
 cudaError_t choose_shape(long long cols, int H, size_t smem, Shape* out)
 {
-    auto kc = hist_conv_col<NACC, KAHAN, BF16>;
+    // (the kernels without parts decide: the split of a column's slots, and so
+    // the order of its sum, does not depend on whether the step is in a block)
+    auto kc = hist_conv_col<NACC, KAHAN, BF16, false>;
     auto kg = hist_conv<NACC, KAHAN, BF16>;
     if (smem > 48 * 1024) {
         cudaFuncSetAttribute(kc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
@@ -372,147 +100,100 @@ cudaError_t choose_shape(long long cols, int H, size_t smem, Shape* out)
     return cudaSuccess;
 }
 
+template <int NACC, bool KAHAN, bool BF16>
+cudaError_t shape_of(int n_pad, int M, Shape* out)
+{
+    static std::mutex mu;
+    static std::map<std::tuple<int, long long, int>, Shape> cache;
+    const int H = M - 1;
+    const long long cols = 3LL * n_pad / Col<BF16>::W;
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    std::lock_guard<std::mutex> lock(mu);
+    auto it = cache.find({dev, cols, H});
+    if (it == cache.end()) {
+        Shape sh{};
+        if ((e = choose_shape<NACC, KAHAN, BF16>(cols, H, sizeof(float) * (size_t)H * NACC, &sh)) != cudaSuccess)
+            return e;
+        it = cache.emplace(std::make_tuple(dev, cols, H), sh).first;
+    }
+    *out = it->second;
+    return cudaSuccess;
+}
+
+template <int NACC, bool KAHAN, bool BF16>
+cudaError_t launch_tb(const void* ring, int n_pad, int M, const long long* nstep, long long step, const float* coef,
+                      float* out, const BlockPos& bp, cudaStream_t st)
+{
+    Shape sh{};
+    const cudaError_t e = shape_of<NACC, KAHAN, BF16>(n_pad, M, &sh);
+    if (e != cudaSuccess) return e;
+    if (bp.t >= 0) return launch_hist_conv_part(sh, NACC, KAHAN, ring, BF16, n_pad, M, nstep, step, coef, out, bp, st);
+    using V = typename Col<BF16>::V;
+    const int H = M - 1;
+    const size_t smem = sizeof(float) * (size_t)H * NACC;
+    const long long cols = 3LL * n_pad / Col<BF16>::W;
+    if (sh.kind == 0)
+        hist_conv_col<NACC, KAHAN, BF16, false><<<sh.grid, sh.block, smem, st>>>((const V*)ring, cols, H, coef, M, nstep,
+                                                                                 step, out, bp);
+    else
+        hist_conv<NACC, KAHAN, BF16><<<sh.grid, sh.block, smem, st>>>((const V*)ring, cols, H, coef, M, nstep, step, out,
+                                                                      sh.G);
+    return cudaGetLastError();
+}
+
 template <int NACC, bool KAHAN>
 cudaError_t launch_t(const void* ring, int bf16, int n_pad, int M, const long long* nstep, long long step,
-                     const float* coef, float* out, cudaStream_t st)
+                     const float* coef, float* out, const BlockPos& bp, cudaStream_t st)
 {
-    return bf16 ? launch_tb<NACC, KAHAN, true>(ring, n_pad, M, nstep, step, coef, out, st)
-                : launch_tb<NACC, KAHAN, false>(ring, n_pad, M, nstep, step, coef, out, st);
+    return bf16 ? launch_tb<NACC, KAHAN, true>(ring, n_pad, M, nstep, step, coef, out, bp, st)
+                : launch_tb<NACC, KAHAN, false>(ring, n_pad, M, nstep, step, coef, out, bp, st);
 }
 
-template <bool KAHAN>
-cudaError_t dispatch(int nacc, const void* ring, int bf16, int n_pad, int M, const long long* nstep,
-                     long long step, const float* coef, float* out, cudaStream_t st)
+cudaError_t dispatch(int nacc, int kahan, const void* ring, int bf16, int n_pad, int M, const long long* nstep,
+                     long long step, const float* coef, float* out, const BlockPos& bp, cudaStream_t st)
 {
-    switch (nacc) {
-    case 1: return launch_t<1, KAHAN>(ring, bf16, n_pad, M, nstep, step, coef, out, st);
-    case 2: return launch_t<2, KAHAN>(ring, bf16, n_pad, M, nstep, step, coef, out, st);
-    case 3: return launch_t<3, KAHAN>(ring, bf16, n_pad, M, nstep, step, coef, out, st);
-    case 4: return launch_t<4, KAHAN>(ring, bf16, n_pad, M, nstep, step, coef, out, st);
-    case 5: return launch_t<5, KAHAN>(ring, bf16, n_pad, M, nstep, step, coef, out, st);
-    case 6: return launch_t<6, KAHAN>(ring, bf16, n_pad, M, nstep, step, coef, out, st);
-    case 7: return launch_t<7, KAHAN>(ring, bf16, n_pad, M, nstep, step, coef, out, st);
-    case 8: return launch_t<8, KAHAN>(ring, bf16, n_pad, M, nstep, step, coef, out, st);
-    case 9: return launch_t<9, KAHAN>(ring, bf16, n_pad, M, nstep, step, coef, out, st);
-    default: return cudaErrorInvalidValue;
-    }
-}
-
-// Batch convolution: tile (member, 256-column block); the member's
-// coefficients are staged for its own step and memory length.
-template <int NACC, bool KAHAN, bool BF16>
-__global__ void __launch_bounds__(kBatchConvCols)
-    b_conv(const SysDesc* __restrict__ D, const Tile* __restrict__ tiles)
-{
-    using V = typename Col<BF16>::V;
-    constexpr int VW = Col<BF16>::W;
-    extern __shared__ float cs[];
-    const Tile t = tiles[blockIdx.x];
-    const SysDesc& d = D[t.m];
-    const int H = d.P.H, M = d.P.m_max;
-    stage_coefs<NACC>(cs, d.coef, M, H, d.B.ctrl->step);
-    const long long cols = 3LL * d.P.n_pad / VW;
-    // columns b*bd + tid, then strided by the member's tiles in this schedule
-    for (long long q = (long long)t.b * blockDim.x + threadIdx.x; q < cols; q += (long long)t.nb * blockDim.x) {
-    const V* p = (const V*)d.B.ring + q;
-    float acc[NACC][VW];
-    float cmp[KAHAN ? NACC : 1][VW];
-#pragma unroll
-    for (int a = 0; a < NACC; ++a)
-#pragma unroll
-        for (int e = 0; e < VW; ++e) acc[a][e] = 0.f;
-#pragma unroll
-    for (int a = 0; a < (KAHAN ? NACC : 1); ++a)
-#pragma unroll
-        for (int e = 0; e < VW; ++e) cmp[a][e] = 0.f;
-    int s = 0;
-    for (; s + kUnroll <= H; s += kUnroll) {
-        V v[kUnroll];
-#pragma unroll
-        for (int u = 0; u < kUnroll; ++u) v[u] = __ldcs(p + (long long)(s + u) * cols);
-#pragma unroll
-        for (int u = 0; u < kUnroll; ++u) {
-            float x[VW];
-            unpack<BF16>(v[u], x);
-#pragma unroll
-            for (int a = 0; a < NACC; ++a) {
-                const float cf = cs[(s + u) * NACC + a];
-#pragma unroll
-                for (int e = 0; e < VW; ++e) acc1<KAHAN>(acc[a][e], cmp[KAHAN ? a : 0][e], cf, x[e]);
-            }
-        }
-    }
-    for (; s < H; ++s) {
-        float x[VW];
-        unpack<BF16>(__ldcs(p + (long long)s * cols), x);
-#pragma unroll
-        for (int a = 0; a < NACC; ++a) {
-            const float cf = cs[s * NACC + a];
-#pragma unroll
-            for (int e = 0; e < VW; ++e) acc1<KAHAN>(acc[a][e], cmp[KAHAN ? a : 0][e], cf, x[e]);
-        }
-    }
-    float4* o = (float4*)d.B.conv;
-    const long long cols4 = cols * (VW / 4);
-#pragma unroll
-    for (int a = 0; a < NACC; ++a)
-#pragma unroll
-        for (int h = 0; h < VW / 4; ++h) {
-            float r[4];
-#pragma unroll
-            for (int e = 0; e < 4; ++e)
-                r[e] = KAHAN ? acc[a][4 * h + e] - cmp[KAHAN ? a : 0][4 * h + e] : acc[a][4 * h + e];
-            o[a * cols4 + q * (VW / 4) + h] = make_float4(r[0], r[1], r[2], r[3]);
-        }
-    }
-}
-
-template <int NACC, bool KAHAN>
-cudaError_t launch_b_conv_t(const BatchPlan& bp, cudaStream_t st)
-{
-    const size_t smem = sizeof(float) * (size_t)bp.max_H * NACC;
-    auto k = bp.bf16 ? b_conv<NACC, KAHAN, true> : b_conv<NACC, KAHAN, false>;
-    if (smem > 48 * 1024) cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    k<<<bp.n_conv, bp.conv_block, smem, st>>>(bp.desc, bp.conv);
-    return cudaGetLastError();
+    return by_nacc(nacc, kahan != 0, [&](auto na, auto ka) {
+        return launch_t<decltype(na)::value, decltype(ka)::value>(ring, bf16, n_pad, M, nstep, step, coef, out, bp, st);
+    });
 }
 
 }  // namespace
 
-cudaError_t launch_batch_conv(const BatchPlan& bp, cudaStream_t st)
+cudaError_t conv_block_shape(int bf16, int n_pad, int m_max, int nacc, int kahan, int* G, int* len, size_t* bytes)
 {
-    if (!bp.n_conv) return cudaSuccess;
-    const bool k = bp.kahan != 0;
-    switch (bp.nacc) {
-    case 1: return k ? launch_b_conv_t<1, true>(bp, st) : launch_b_conv_t<1, false>(bp, st);
-    case 2: return k ? launch_b_conv_t<2, true>(bp, st) : launch_b_conv_t<2, false>(bp, st);
-    case 3: return k ? launch_b_conv_t<3, true>(bp, st) : launch_b_conv_t<3, false>(bp, st);
-    case 4: return k ? launch_b_conv_t<4, true>(bp, st) : launch_b_conv_t<4, false>(bp, st);
-    case 5: return k ? launch_b_conv_t<5, true>(bp, st) : launch_b_conv_t<5, false>(bp, st);
-    case 6: return k ? launch_b_conv_t<6, true>(bp, st) : launch_b_conv_t<6, false>(bp, st);
-    case 7: return k ? launch_b_conv_t<7, true>(bp, st) : launch_b_conv_t<7, false>(bp, st);
-    case 8: return k ? launch_b_conv_t<8, true>(bp, st) : launch_b_conv_t<8, false>(bp, st);
-    case 9: return k ? launch_b_conv_t<9, true>(bp, st) : launch_b_conv_t<9, false>(bp, st);
-    default: return cudaErrorInvalidValue;
-    }
+    *G = *len = 0;
+    *bytes = 0;
+    if (m_max - 1 < kMinBlockedSlots) return cudaSuccess;
+    Shape sh{};
+    const cudaError_t e = by_nacc(nacc, kahan != 0, [&](auto na, auto ka) {
+        return bf16 ? shape_of<decltype(na)::value, decltype(ka)::value, true>(n_pad, m_max, &sh)
+                    : shape_of<decltype(na)::value, decltype(ka)::value, false>(n_pad, m_max, &sh);
+    });
+    if (e != cudaSuccess) return e;
+    *G = sh.G;
+    *len = pre_len(kahan, sh.G);
+    const int rows = std::max(sh.G * *len, pre_len(kahan, 1));  // alone, and in a batch (one range)
+    *bytes = sizeof(float) * (size_t)rows * nacc * (kahan ? 2 : 1) * 3 * n_pad;
+    return cudaSuccess;
 }
 
 cudaError_t launch_hist_conv(const void* ring, int bf16, int n_pad, int m_max, const Ctrl* ctrl,
                              long long step, const float* coef, int nacc, float* out, int kahan,
-                             cudaStream_t st)
+                             cudaStream_t st, const float* part, int t, int len)
 {
     if (m_max < 2 || n_pad <= 0 || n_pad % 32 != 0 || nacc < 1 || nacc > kMaxAcc) return cudaErrorInvalidValue;
     const long long* nstep = ctrl ? &ctrl->step : nullptr;
-    return kahan ? dispatch<true>(nacc, ring, bf16, n_pad, m_max, nstep, step, coef, out, st)
-                 : dispatch<false>(nacc, ring, bf16, n_pad, m_max, nstep, step, coef, out, st);
+    return dispatch(nacc, kahan, ring, bf16, n_pad, m_max, nstep, step, coef, out, BlockPos{part, t, len}, st);
 }
 
 cudaError_t launch_hist_conv_next(const void* ring, int bf16, int n_pad, int m_max, const Ctrl* ctrl,
-                                  const float* coef, int nacc, float* out, int kahan, cudaStream_t st)
+                                  const float* coef, int nacc, float* out, int kahan, cudaStream_t st,
+                                  const float* part, int t, int len)
 {
     if (m_max < 2 || n_pad <= 0 || n_pad % 32 != 0 || nacc < 1 || nacc > kMaxAcc || !ctrl) return cudaErrorInvalidValue;
-    return kahan ? dispatch<true>(nacc, ring, bf16, n_pad, m_max, &ctrl->conv_step, 0, coef, out, st)
-                 : dispatch<false>(nacc, ring, bf16, n_pad, m_max, &ctrl->conv_step, 0, coef, out, st);
+    return dispatch(nacc, kahan, ring, bf16, n_pad, m_max, &ctrl->conv_step, 0, coef, out, BlockPos{part, t, len}, st);
 }
 
 }  // namespace gld

@@ -11,16 +11,27 @@
 namespace gld {
 
 // History convolution (k_history.cu).  ctrl != nullptr: the step is read on
-// the device; otherwise `step` is used.
+// the device; otherwise `step` is used.  t >= 0: the step is number t of a
+// block of len steps whose parts launch_conv_pre has formed.
 cudaError_t launch_hist_conv(const void* ring, int bf16, int n_pad, int m_max, const Ctrl* ctrl,
                              long long step, const float* coef, int nacc, float* out, int kahan,
-                             cudaStream_t st);
+                             cudaStream_t st, const float* part = nullptr, int t = -1, int len = 0);
 
 // The convolution of the step after the current one (its index read from
 // ctrl->conv_step, written by the pair kernel), so that it can run beside the
 // current step's F^C and VACF kernels.
 cudaError_t launch_hist_conv_next(const void* ring, int bf16, int n_pad, int m_max, const Ctrl* ctrl,
-                                  const float* coef, int nacc, float* out, int kahan, cudaStream_t st);
+                                  const float* coef, int nacc, float* out, int kahan, cudaStream_t st,
+                                  const float* part = nullptr, int t = -1, int len = 0);
+
+// Blocks of steps: the split G of a column's slots, the steps of a block and
+// the bytes of its parts (G = 0: the memory is too short for blocks), and the
+// parts of the block that starts at step *nstep (device memory).
+constexpr int kMinBlockedSlots = 32;
+cudaError_t conv_block_shape(int bf16, int n_pad, int m_max, int nacc, int kahan, int* G, int* len, size_t* bytes);
+cudaError_t launch_conv_pre(const void* ring, int bf16, int n_pad, int m_max, const long long* nstep, const float* coef,
+                            int nacc, float* part, int G, int len, int kahan, cudaStream_t st);
+int batch_pre_tiles(int n_pad);
 
 // Particle kernels (k_particles.cu).
 struct ParticleBuffers {
@@ -30,6 +41,7 @@ struct ParticleBuffers {
     float4 *vel, *vhalf, *fc, *fd, *disp, *disp_build;
     int *nbr, *nbr_cnt, *perm;   // neighbour lists [maxnb][n_pad] in build order
     void* ring;
+    float* part;          // parts of a block of steps (StepParams::cblk) or null
     float* conv;
     float* frblock;
     const float* ftab;
@@ -157,14 +169,15 @@ struct Tile {
 };
 struct BatchPlan {
     const SysDesc* desc;
-    const Tile *pair, *part, *cell, *vacf, *conv, *fir, *cf;
-    int n_pair, n_part, n_cell, n_vacf, n_conv, n_fir, n_cf;
+    const Tile *pair, *part, *cell, *vacf, *conv, *fir, *cf, *pre;
+    int n_pair, n_part, n_cell, n_vacf, n_conv, n_fir, n_cf, n_pre;
     int max_H, max_n, max_ntaps, nacc, bf16, kahan, vacf_no;
     int conv_block;  // threads per convolution tile (128 or 256)
     int pair_fast;   // every member has one pair term and no self-difference term
     int pn_kmax;     // the largest Chebyshev degree of the members' pair noise (0: none)
 };
-cudaError_t launch_batch_conv(const BatchPlan& bp, cudaStream_t st);      // k_history.cu
+// step: number of the step in its 64-step block
+cudaError_t launch_batch_conv(const BatchPlan& bp, int step, cudaStream_t st);  // k_history.cu
 cudaError_t launch_batch_particles(const BatchPlan& bp, cudaStream_t st); // k_particles.cu
 cudaError_t launch_batch_noise(const BatchPlan& bp, cudaStream_t st);     // k_noise.cu
 // Block sizes of the tile schedules.
