@@ -159,6 +159,7 @@ void invalidate_graph(gld_ctx* c)
 {
     if (c->gexec) cudaGraphExecDestroy(c->gexec);
     c->gexec = nullptr;
+    c->cluster_graph = false;
     c->graph_failed = false;
     c->conv_valid_step = c->part_step = -1;
 }
@@ -589,6 +590,91 @@ gld_status pair_noise_krylov(gld_ctx* c, cudaStream_t st)
     return GLD_OK;
 }
 
+// What the kernels that take whole systems need of a context.
+SysDesc make_desc(const gld_ctx* c)
+{
+    SysDesc d{};
+    d.P = c->P;
+    d.B = c->B;
+    d.coef = c->coef;
+    d.W = c->W;
+    d.taps = c->P.pn_deg > 0 ? c->d_pntaps : c->Acp;  // row 0 of the pair-noise filters
+    d.ntaps = fir_taps_len(c->P.H);
+    d.pntaps = c->d_pntaps;
+    d.zblk = c->d_zblk;
+    d.bvec = c->d_bvec;
+    d.pn_la = c->la;
+    d.k0 = (uint32_t)c->prm.seed;
+    d.k1 = (uint32_t)(c->prm.seed >> 32);
+    d.int2ext = c->d_int2ext;
+    return d;
+}
+
+// Small systems: steps of a noise block in one kernel (k_cluster.cu), unless
+// the launches of the gated graph were asked for (use_graphs = 2).
+bool steps_in_cluster(const gld_ctx* c) { return c->prm.use_graphs != 2 && cluster_ok(c->P, c->prm.kahan); }
+
+// A noise block and its 64 steps as a graph of three kernels.
+bool capture_cluster_graph(gld_ctx* c)
+{
+    if (c->gexec && c->cluster_graph) return true;
+    if (c->graph_failed) return false;
+    invalidate_graph(c);
+    cudaGraph_t g = nullptr;
+    bool ok = cudaStreamBeginCapture(c->cap, cudaStreamCaptureModeThreadLocal) == cudaSuccess;
+    if (ok) {
+        cudaError_t e = launch_noise(c, c->cap);
+        if (e == cudaSuccess)
+            e = launch_steps_cluster(make_desc(c), c->P.T, 0, c->conv_G, c->conv_len, c->cap);
+        const cudaError_t e2 = cudaStreamEndCapture(c->cap, &g);
+        ok = e == cudaSuccess && e2 == cudaSuccess && g != nullptr;
+    }
+    if (ok) ok = cudaGraphInstantiate(&c->gexec, g, 0) == cudaSuccess;
+    if (g) cudaGraphDestroy(g);
+    if (!ok) {
+        c->gexec = nullptr;
+        c->graph_failed = true;
+        cudaGetLastError();
+    }
+    c->cluster_graph = ok;
+    c->graph_mode = ok ? 1 : c->graph_mode;
+    return ok;
+}
+
+gld_status step_cluster(gld_ctx* c, int64_t nsteps)
+{
+    const int T = c->P.T, len = c->P.cblk ? c->conv_len : 1;
+    while (nsteps > 0) {
+        const long long first = c->host_step;
+        // the first step's number in its block of the convolution: blocks go on
+        // from the one whose parts are there, or start here
+        const int rel0 = c->part_step >= 0 && first - c->part_step < len ? (int)(first - c->part_step) : 0;
+        int64_t k = T;
+        if (!c->noise_valid || first >= c->noise_end) {
+            c->block_start = first;
+            c->noise_end = first + T;
+            if (c->prm.use_graphs && nsteps >= T && rel0 == 0 && capture_cluster_graph(c)) {
+                GLD_CUDA(c, cudaGraphLaunch(c->gexec, c->st));
+            } else {
+                GLD_CUDA(c, launch_noise(c, c->st));
+                k = std::min<int64_t>(nsteps, T);
+                GLD_CUDA(c, launch_steps_cluster(make_desc(c), (int)k, rel0, c->conv_G, c->conv_len, c->st));
+            }
+            c->noise_valid = true;
+        } else {
+            k = std::min<int64_t>(nsteps, c->noise_end - first);
+            GLD_CUDA(c, launch_steps_cluster(make_desc(c), (int)k, rel0, c->conv_G, c->conv_len, c->st));
+        }
+        c->host_step += k;
+        nsteps -= k;
+        c->last_fr_row = c->host_step - 1 - c->block_start;
+        c->conv_valid_step = -1;
+        const long long origin = first - rel0;
+        c->part_step = c->P.cblk ? c->host_step - 1 - (c->host_step - 1 - origin) % len : -1;
+    }
+    return GLD_OK;
+}
+
 bool capture_graph_mode(gld_ctx* c, bool conditional)
 {
     // the overlapped form needs an idempotent convolution (not the recursive
@@ -620,12 +706,20 @@ bool capture_graph_mode(gld_ctx* c, bool conditional)
     return ok;
 }
 
+// Particles from which the rebuild goes into a conditional node: the node costs
+// about 7 us per step, the gated kernels that find nothing to do less than that
+// below (32768: 40.4 against 32.8 us per step, 131072: 98.8 against 92.9,
+// 262144: 185.5 against 185.7).
+constexpr int kConditionalMinN = 262144;
+
 bool capture_graph(gld_ctx* c)
 {
+    if (c->gexec && c->cluster_graph) invalidate_graph(c);  // the system left the cluster path
     if (c->gexec) return true;
     if (c->graph_failed || c->P.pn_kry) return false;  // the Lanczos noise decides on the host every step
-    // conditional rebuild first; the gated kernels are the fallback
-    if (c->prm.use_graphs != 2 && capture_graph_mode(c, true)) {
+    // conditional rebuild for large systems; the gated kernels otherwise, and
+    // as the fallback
+    if (c->prm.use_graphs != 2 && c->P.n >= kConditionalMinN && capture_graph_mode(c, true)) {
         c->graph_mode = 2;
         return true;
     }
@@ -1077,6 +1171,7 @@ gld_status gld_step(gld_ctx* c, int64_t nsteps)
     const int T = c->P.T;
     if (nsteps > 0) GLD_TRY(ring_form(c, true, c->st));
     if (nsteps > 0) GLD_TRY(refresh_modes(c));
+    if (steps_in_cluster(c)) return step_cluster(c, nsteps);
     while (nsteps > 0) {
         if (!c->noise_valid || c->host_step >= c->noise_end) {
             if (c->prm.use_graphs && nsteps >= T && capture_graph(c)) {
@@ -1396,7 +1491,7 @@ gld_status gld_profile_steps(gld_ctx* c, int64_t nsteps, double* ms, int64_t* la
             }
             acc[fam[q]] += t;
             const int pd = c->P.pn_deg;
-            cnt[fam[q]] += fam[q] == GLD_PROF_CELL     ? 4
+            cnt[fam[q]] += fam[q] == GLD_PROF_CELL     ? (rebuild_in_cluster(c->P) ? 1 : 4)
                            : fam[q] == GLD_PROF_NOISE  ? 2 + pd
                            : fam[q] == GLD_PROF_PNOISE ? pd
                                                        : 1;
@@ -2357,21 +2452,9 @@ gld_status batch_plan(gld_batch* b, int schedule)
     for (size_t m = 0; m < ms.size(); ++m) {
         gld_ctx* c = ms[m];
         SysDesc& d = desc[m];
-        d.P = c->P;
+        d = make_desc(c);
         d.P.wsplit = 0;  // the batched filter reads the FP32 ring
-        d.B = c->B;
-        d.coef = c->coef;
-        d.W = c->W;
-        d.taps = c->P.pn_deg > 0 ? c->d_pntaps : c->Acp;  // row 0 of the pair-noise filters
-        d.ntaps = fir_taps_len(c->P.H);
-        d.pntaps = c->d_pntaps;
-        d.zblk = c->d_zblk;
-        d.bvec = c->d_bvec;
-        d.pn_la = c->la;
         P.pn_kmax = std::max(P.pn_kmax, c->P.pn_deg);
-        d.k0 = (uint32_t)c->prm.seed;
-        d.k1 = (uint32_t)(c->prm.seed >> 32);
-        d.int2ext = c->d_int2ext;
         d.nb_pair = (c->P.n + pair_per_block - 1) / pair_per_block;
         d.nb_part = (c->P.n + kBatchPartBlock - 1) / kBatchPartBlock;
         d.nb_cf = (int)(((long long)c->P.n * kBatchCforceLanes + kBatchCforceBlock - 1) / kBatchCforceBlock);

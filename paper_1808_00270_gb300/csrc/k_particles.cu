@@ -1441,6 +1441,7 @@ cudaError_t launch_cell_build(const StepParams& P, const ParticleBuffers& B, con
 
 cudaError_t launch_rebuild(const StepParams& P, const ParticleBuffers& B, cudaStream_t st)
 {
+    if (rebuild_in_cluster(P)) return launch_rebuild_cluster(P, B, st);
     cudaError_t e = launch_cell_build(P, B, B.pos_next, &B.ctrl->rebuild, st);
     if (e != cudaSuccess) return e;
     nbr_build<<<(P.n + kThreads - 1) / kThreads, kThreads, 0, st>>>(P, B.ctrl, B.pos_sorted, B.cell_start, B.nbr,

@@ -180,6 +180,20 @@ struct BatchPlan {
 cudaError_t launch_batch_conv(const BatchPlan& bp, int step, cudaStream_t st);  // k_history.cu
 cudaError_t launch_batch_particles(const BatchPlan& bp, cudaStream_t st); // k_particles.cu
 cudaError_t launch_batch_noise(const BatchPlan& bp, cudaStream_t st);     // k_noise.cu
+// Whole steps of small systems (k_cluster.cu): whether a system's features and
+// size allow it; a system alone for nsteps steps of its noise block (rel0:
+// number of the first step in its block of the convolution, > 0: that block's
+// parts are formed; G and len as conv_block_shape).
+constexpr int kClusterMaxN = 4096;
+bool cluster_ok(const StepParams& P, int kahan);
+cudaError_t launch_steps_cluster(const SysDesc& d, int nsteps, int rel0, int G, int len, cudaStream_t st);
+
+// The list build of launch_rebuild by one cluster (gated on ctrl->rebuild), for
+// systems where that is faster than the four kernels.
+constexpr int kClusterRebuildMaxN = 12288;
+bool rebuild_in_cluster(const StepParams& P);
+cudaError_t launch_rebuild_cluster(const StepParams& P, const ParticleBuffers& B, cudaStream_t st);
+
 // Block sizes of the tile schedules.
 constexpr int kBatchPairLanes = 1;    // lanes per particle of the one-term pair kernel
 constexpr int kBatchCforceLanes = 1;  // lanes per particle of the F^C kernel
