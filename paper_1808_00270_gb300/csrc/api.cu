@@ -2443,10 +2443,11 @@ gld_status batch_plan(gld_batch* b, int schedule)
 {
     const auto& ms = b->members;
     std::vector<SysDesc> desc(ms.size());
-    std::vector<Tile> pair, part, cell, vacf, conv, fir, cf, pre;
+    std::vector<Tile> pair, part, cell, vacf, conv, fir, cf, pre, nbr;
     BatchPlan& P = b->plan;
     P = BatchPlan{};
     P.pair_fast = 1;
+    for (const gld_ctx* c : ms) P.max_nb = std::max(P.max_nb, c->P.maxnb);
     for (const gld_ctx* c : ms) P.pair_fast &= (c->P.Q == 1 && c->P.Qs == 0 && !c->P.perp) ? 1 : 0;
     const int pair_per_block = P.pair_fast ? kBatchPairBlock / kBatchPairLanes : kBatchPairBlock;
     for (size_t m = 0; m < ms.size(); ++m) {
@@ -2468,6 +2469,8 @@ gld_status batch_plan(gld_batch* b, int schedule)
         for (int k = 0; k < d.nb_cell; ++k) cell.push_back(Tile{(int)m, k, d.nb_cell, 0});
         for (int k = 0; k < d.nb_vacf; ++k) vacf.push_back(Tile{(int)m, k, d.nb_vacf, 0});
         for (int k = 0; k < d.nb_fir; ++k) fir.push_back(Tile{(int)m, k, d.nb_fir, 0});
+        const int nnbr = batch_nbr_tiles(c->P.n);
+        for (int k = 0; k < nnbr; ++k) nbr.push_back(Tile{(int)m, k, nnbr, 0});
         const int npre = c->P.cblk ? batch_pre_tiles(c->P.n_pad) : 0;
         for (int k = 0; k < npre; ++k) pre.push_back(Tile{(int)m, k, npre, 0});
         P.max_H = std::max(P.max_H, c->P.H);
@@ -2491,7 +2494,7 @@ gld_status batch_plan(gld_batch* b, int schedule)
     };
     const size_t o_pair = append(pair, &P.n_pair), o_part = append(part, &P.n_part), o_cell = append(cell, &P.n_cell),
                  o_vacf = append(vacf, &P.n_vacf), o_conv = append(conv, &P.n_conv), o_fir = append(fir, &P.n_fir),
-                 o_cf = append(cf, &P.n_cf), o_pre = append(pre, &P.n_pre);
+                 o_cf = append(cf, &P.n_cf), o_pre = append(pre, &P.n_pre), o_nbr = append(nbr, &P.n_nbr);
     b->snap = desc;
     // One upload of descriptors and tiles through pinned staging, ordered on
     // the batch's stream after the blocks already queued (which keep reading
@@ -2536,6 +2539,7 @@ gld_status batch_plan(gld_batch* b, int schedule)
     P.fir = t0 + o_fir;
     P.cf = t0 + o_cf;
     P.pre = t0 + o_pre;
+    P.nbr = t0 + o_nbr;
     return GLD_OK;
 }
 

@@ -475,6 +475,110 @@ __global__ void __launch_bounds__(kThreads) nbr_build(const StepParams P, Ctrl* 
     nbr_build_body(P, ctrl, pos_sorted, cell_start, nbr, nbr_cnt, perm, disp, disp_build, blockIdx.x, gridDim.x);
 }
 
+// The same lists (capacity at most kNbrSortCap) with kNbrLanes lanes per
+// particle.  The walk above is one chain of some 60 dependent loads per thread
+// and a serial sort: 40 to 109 us whatever the size.  Cells hold their
+// particles in the order of the scan, so a row of three cells along x is one
+// range of pos_sorted (two at the box's faces): the lanes share the nine rows,
+// read four candidates at a time, collect ids in shared memory, and write each
+// to the place of its rank among the particle's ids.  Particles are taken in
+// cell order, so the groups of a warp read the same cells.
+constexpr int kNbrLanes = 4;
+constexpr int kNbrGroups = kThreads / kNbrLanes;  // particles per block
+
+__device__ __forceinline__ void nbr_lanes_body(const StepParams& P, Ctrl* ctrl, const float4* __restrict__ pos_sorted,
+                                               const int* __restrict__ cell_start, int* __restrict__ nbr,
+                                               int* __restrict__ nbr_cnt, int* __restrict__ perm,
+                                               const float4* __restrict__ disp, float4* __restrict__ disp_build, int blk)
+{
+    if (ctrl->rebuild == 0) return;
+    extern __shared__ int lists[];  // [kNbrGroups][maxnb]
+    __shared__ int lcnt[kNbrGroups];
+    constexpr int L = kNbrLanes, R = (9 + L - 1) / L;
+    const int lane = threadIdx.x & (L - 1), grp = threadIdx.x / L, k = blk * kNbrGroups + grp;
+    const unsigned gmask = ((1u << L) - 1u) << ((threadIdx.x & 31) & ~(L - 1));
+    if (blk == 0 && threadIdx.x == 0) ctrl->rebuilds += 1;
+    if (k >= P.n) return;  // uniform over the lanes of a particle
+    const float4 pi = pos_sorted[k];
+    const int id = __float_as_int(pi.w), nc = P.nc;
+    int* list = lists + grp * P.maxnb;
+    if (lane == 0) lcnt[grp] = 0;
+    __syncwarp(gmask);
+    auto test = [&](const float4 pj) {
+        const int jd = __float_as_int(pj.w);
+        const float dx = min_image(pi.x, pj.x, P.box, P.half_box);
+        const float dy = min_image(pi.y, pj.y, P.box, P.half_box);
+        const float dz = min_image(pi.z, pj.z, P.box, P.half_box);
+        if (jd != id && dist2(dx, dy, dz) < P.rl2) {
+            const int c = atomicAdd(lcnt + grp, 1);
+            if (c < P.maxnb) list[c] = jd;
+        }
+    };
+    if (nc == 1) {
+        for (int q = lane; q < P.n; q += L) test(__ldg(pos_sorted + q));
+    } else {
+        const int cx = cell_coord(pi.x, P.inv_cell, nc), cy = cell_coord(pi.y, P.inv_cell, nc),
+                  cz = cell_coord(pi.z, P.inv_cell, nc);
+        const int xa = max(cx - 1, 0), xb = min(cx + 1, nc - 1);  // the row inside the box
+        const int xw = cx == 0 ? nc - 1 : cx == nc - 1 ? 0 : -1;  // the cell across a face
+        int b0[R], n0[R], b1[R], n1[R];
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            const int o = lane + r * L;
+            int z = cz + o / 3 - 1, y = cy + o % 3 - 1;
+            z = z < 0 ? z + nc : (z >= nc ? z - nc : z);
+            y = y < 0 ? y + nc : (y >= nc ? y - nc : y);
+            const int base = (z * nc + y) * nc;
+            b0[r] = n0[r] = b1[r] = n1[r] = 0;
+            if (o < 9) {
+                b0[r] = __ldg(cell_start + base + xa);
+                n0[r] = __ldg(cell_start + base + xb + 1) - b0[r];
+                if (xw >= 0) {
+                    b1[r] = __ldg(cell_start + base + xw);
+                    n1[r] = __ldg(cell_start + base + xw + 1) - b1[r];
+                }
+            }
+        }
+#pragma unroll
+        for (int r = 0; r < R; ++r)
+            for (int q = 0; q < n0[r] + n1[r]; q += 4) {
+                float4 pj[4];
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    const int c = q + u < n0[r] + n1[r] ? q + u : q;
+                    pj[u] = __ldg(pos_sorted + (c < n0[r] ? b0[r] + c : b1[r] + c - n0[r]));
+                }
+#pragma unroll
+                for (int u = 0; u < 4; ++u)
+                    if (q + u < n0[r] + n1[r]) test(pj[u]);
+            }
+    }
+    __syncwarp(gmask);
+    int c = lcnt[grp];
+    if (c > P.maxnb) {
+        if (lane == 0) atomicOr(&ctrl->err, kErrNbrOverflow);
+        c = P.maxnb;
+    }
+    for (int s = lane; s < c; s += L) {
+        const int v = list[s];
+        int r = 0;
+        for (int q = 0; q < c; ++q) r += list[q] < v;
+        nbr[(size_t)r * P.n_pad + id] = v;
+    }
+    if (lane == 0) {
+        nbr_cnt[id] = c;
+        perm[k] = id;
+        disp_build[id] = disp[id];
+    }
+}
+
+__global__ void __launch_bounds__(kThreads) nbr_lanes(const StepParams P, Ctrl* ctrl, const float4* __restrict__ pos_sorted,
+              const int* __restrict__ cell_start, int* __restrict__ nbr, int* __restrict__ nbr_cnt,
+              int* __restrict__ perm, const float4* __restrict__ disp, float4* __restrict__ disp_build)
+{
+    nbr_lanes_body(P, ctrl, pos_sorted, cell_start, nbr, nbr_cnt, perm, disp, disp_build, blockIdx.x);
+}
+
 // ---- velocity autocorrelation ------------------------------------------------
 constexpr int kVacfMaxOrigins = 32;  // origins in flight (vacf_len / vacf_stride)
 constexpr int kVacfGroup = 4;        // origins per block row of the VACF grid
@@ -1055,6 +1159,14 @@ __global__ void __launch_bounds__(kThreads) b_nbr_build(const SysDesc* __restric
                    d.nb_part);
 }
 
+__global__ void __launch_bounds__(kThreads) b_nbr_lanes(const SysDesc* __restrict__ D, const Tile* __restrict__ tiles)
+{
+    const Tile t = tiles[blockIdx.x];
+    const SysDesc& d = D[t.m];
+    const ParticleBuffers& B = d.B;
+    nbr_lanes_body(d.P, B.ctrl, B.pos_sorted, B.cell_start, B.nbr, B.nbr_cnt, B.perm, B.disp, B.disp_build, t.b);
+}
+
 __global__ void __launch_bounds__(kThreads) b_cforce(const SysDesc* __restrict__ D, const Tile* __restrict__ tiles)
 {
     const Tile t = tiles[blockIdx.x];
@@ -1378,6 +1490,14 @@ __global__ void lz_final(const double* __restrict__ ab, double lo, double hi, in
     if (check && (tmin < lo || tmax > hi)) atomicOr(&ctrl->err, kErrPnBound);
 }
 
+template <class K, class... A>
+cudaError_t launch_nbr_lanes(K kern, int blocks, int maxnb, cudaStream_t st, const A&... args)
+{
+    const size_t smem = sizeof(int) * (size_t)kNbrGroups * maxnb;  // at most 32 KB
+    kern<<<(unsigned)blocks, kThreads, smem, st>>>(args...);
+    return cudaGetLastError();
+}
+
 }  // namespace
 
 cudaError_t launch_batch_particles(const BatchPlan& bp, cudaStream_t st)
@@ -1392,7 +1512,14 @@ cudaError_t launch_batch_particles(const BatchPlan& bp, cudaStream_t st)
     if (bp.n_part) b_cell_assign<<<bp.n_part, kThreads, 0, st>>>(bp.desc, bp.part);
     if (bp.n_cell) b_cell_scan<<<bp.n_cell, kCellThreads, 0, st>>>(bp.desc, bp.cell);
     if (bp.n_cell) b_cell_fill<<<bp.n_cell, kCellThreads, 0, st>>>(bp.desc, bp.cell);
-    if (bp.n_part) b_nbr_build<<<bp.n_part, kThreads, 0, st>>>(bp.desc, bp.part);
+    if (bp.n_part) {
+        if (bp.max_nb <= kNbrSortCap) {
+            const cudaError_t e = launch_nbr_lanes(b_nbr_lanes, bp.n_nbr, bp.max_nb, st, bp.desc, bp.nbr);
+            if (e != cudaSuccess) return e;
+        } else {
+            b_nbr_build<<<bp.n_part, kThreads, 0, st>>>(bp.desc, bp.part);
+        }
+    }
     if (bp.n_cf) b_cforce<<<bp.n_cf, kBatchCforceBlock, 0, st>>>(bp.desc, bp.cf);
     if (bp.n_vacf) {
         const dim3 g((unsigned)bp.n_vacf, (unsigned)((bp.vacf_no + kVacfGroup - 1) / kVacfGroup));
@@ -1444,6 +1571,9 @@ cudaError_t launch_rebuild(const StepParams& P, const ParticleBuffers& B, cudaSt
     if (rebuild_in_cluster(P)) return launch_rebuild_cluster(P, B, st);
     cudaError_t e = launch_cell_build(P, B, B.pos_next, &B.ctrl->rebuild, st);
     if (e != cudaSuccess) return e;
+    if (P.maxnb <= kNbrSortCap)
+        return launch_nbr_lanes(nbr_lanes, (P.n + kNbrGroups - 1) / kNbrGroups, P.maxnb, st, P, B.ctrl, B.pos_sorted,
+                                B.cell_start, B.nbr, B.nbr_cnt, B.perm, B.disp, B.disp_build);
     nbr_build<<<(P.n + kThreads - 1) / kThreads, kThreads, 0, st>>>(P, B.ctrl, B.pos_sorted, B.cell_start, B.nbr,
                                                                      B.nbr_cnt, B.perm, B.disp, B.disp_build);
     return cudaGetLastError();
@@ -1512,6 +1642,8 @@ cudaError_t launch_pair_noise(const StepParams& P, const ParticleBuffers& B, con
     }
     return cudaSuccess;
 }
+
+int batch_nbr_tiles(int n) { return (n + kNbrGroups - 1) / kNbrGroups; }
 
 int pn_spectrum_blocks(const StepParams& P) { return (int)((P.n_pad + kThreads - 1) / kThreads); }
 

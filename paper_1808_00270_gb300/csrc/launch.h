@@ -32,6 +32,7 @@ cudaError_t conv_block_shape(int bf16, int n_pad, int m_max, int nacc, int kahan
 cudaError_t launch_conv_pre(const void* ring, int bf16, int n_pad, int m_max, const long long* nstep, const float* coef,
                             int nacc, float* part, int G, int len, int kahan, cudaStream_t st);
 int batch_pre_tiles(int n_pad);
+int batch_nbr_tiles(int n);  // tiles of the list build (k_particles.cu)
 
 // Particle kernels (k_particles.cu).
 struct ParticleBuffers {
@@ -169,10 +170,11 @@ struct Tile {
 };
 struct BatchPlan {
     const SysDesc* desc;
-    const Tile *pair, *part, *cell, *vacf, *conv, *fir, *cf, *pre;
-    int n_pair, n_part, n_cell, n_vacf, n_conv, n_fir, n_cf, n_pre;
+    const Tile *pair, *part, *cell, *vacf, *conv, *fir, *cf, *pre, *nbr;
+    int n_pair, n_part, n_cell, n_vacf, n_conv, n_fir, n_cf, n_pre, n_nbr;
     int max_H, max_n, max_ntaps, nacc, bf16, kahan, vacf_no;
     int conv_block;  // threads per convolution tile (128 or 256)
+    int max_nb;      // the longest list capacity
     int pair_fast;   // every member has one pair term and no self-difference term
     int pn_kmax;     // the largest Chebyshev degree of the members' pair noise (0: none)
 };
