@@ -157,8 +157,11 @@ gld_status sync_and_check(gld_ctx* c)
 
 void invalidate_graph(gld_ctx* c)
 {
-    if (c->gexec) cudaGraphExecDestroy(c->gexec);
-    c->gexec = nullptr;
+    for (cudaGraphExec_t* g : {&c->gexec, &c->gseg}) {
+        if (*g) cudaGraphExecDestroy(*g);
+        *g = nullptr;
+    }
+    c->eager_steps = 0;
     c->cluster_graph = false;
     c->graph_failed = false;
     c->conv_valid_step = c->part_step = -1;
@@ -641,41 +644,49 @@ bool capture_cluster_graph(gld_ctx* c)
     return ok;
 }
 
-gld_status step_cluster(gld_ctx* c, int64_t nsteps)
+// k steps of one noise block, which begins with them when boundary.
+gld_status step_cluster(gld_ctx* c, int64_t k, bool boundary)
 {
     const int T = c->P.T, len = c->P.cblk ? c->conv_len : 1;
-    while (nsteps > 0) {
-        const long long first = c->host_step;
-        // the first step's number in its block of the convolution: blocks go on
-        // from the one whose parts are there, or start here
-        const int rel0 = c->part_step >= 0 && first - c->part_step < len ? (int)(first - c->part_step) : 0;
-        int64_t k = T;
-        if (!c->noise_valid || first >= c->noise_end) {
-            c->block_start = first;
-            c->noise_end = first + T;
-            if (c->prm.use_graphs && nsteps >= T && rel0 == 0 && capture_cluster_graph(c)) {
-                GLD_CUDA(c, cudaGraphLaunch(c->gexec, c->st));
-            } else {
-                GLD_CUDA(c, launch_noise(c, c->st));
-                k = std::min<int64_t>(nsteps, T);
-                GLD_CUDA(c, launch_steps_cluster(make_desc(c), (int)k, rel0, c->conv_G, c->conv_len, c->st));
-            }
-            c->noise_valid = true;
-        } else {
-            k = std::min<int64_t>(nsteps, c->noise_end - first);
-            GLD_CUDA(c, launch_steps_cluster(make_desc(c), (int)k, rel0, c->conv_G, c->conv_len, c->st));
-        }
-        c->host_step += k;
-        nsteps -= k;
-        c->last_fr_row = c->host_step - 1 - c->block_start;
-        c->conv_valid_step = -1;
-        const long long origin = first - rel0;
-        c->part_step = c->P.cblk ? c->host_step - 1 - (c->host_step - 1 - origin) % len : -1;
+    const long long first = c->host_step;
+    // the first step's number in its block of the convolution: blocks go on
+    // from the one whose parts are there, or start here
+    const int rel0 = c->part_step >= 0 && first - c->part_step < len ? (int)(first - c->part_step) : 0;
+    if (boundary) {
+        c->block_start = first;
+        c->noise_end = first + T;
     }
+    if (boundary && c->prm.use_graphs && k == T && rel0 == 0 && c->P.n <= kClusterBlockMaxN && capture_cluster_graph(c)) {
+        GLD_CUDA(c, cudaGraphLaunch(c->gexec, c->st));
+    } else {
+        if (boundary) GLD_CUDA(c, launch_noise(c, c->st));
+        GLD_CUDA(c, launch_steps_cluster(make_desc(c), (int)k, rel0, c->conv_G, c->conv_len, c->st));
+    }
+    c->noise_valid = true;
+    c->host_step += k;
+    c->last_fr_row = c->host_step - 1 - c->block_start;
+    c->conv_valid_step = -1;
+    const long long origin = first - rel0;
+    c->part_step = c->P.cblk ? c->host_step - 1 - (c->host_step - 1 - origin) % len : -1;
     return GLD_OK;
 }
 
-bool capture_graph_mode(gld_ctx* c, bool conditional)
+// Replays a captured graph of `steps` steps from a block of the convolution's
+// first step (a noise block has begun, or begins in it).  An overlapped graph
+// starts from its first step's memory sums and the parts of their block.
+gld_status replay(gld_ctx* c, cudaGraphExec_t g, int steps)
+{
+    if (c->P.cblk && c->part_step != c->host_step) c->conv_valid_step = -1;
+    if (c->overlap_graph) GLD_CUDA(c, launch_memory(c, c->st));
+    GLD_CUDA(c, cudaGraphLaunch(g, c->st));
+    c->host_step += steps;
+    c->conv_valid_step = c->overlap_graph ? c->host_step : -1;
+    c->part_step = c->overlap_graph && c->P.cblk ? c->host_step : -1;
+    return GLD_OK;
+}
+
+// Captures `steps` steps (with a noise block before them) into *exec.
+bool capture_graph_mode(gld_ctx* c, bool conditional, int steps, bool noise, cudaGraphExec_t* exec)
 {
     // the overlapped form needs an idempotent convolution (not the recursive
     // memory form, whose kernel advances its auxiliary sums)
@@ -690,20 +701,21 @@ bool capture_graph_mode(gld_ctx* c, bool conditional)
     cudaGraph_t g = nullptr;
     bool ok = cudaStreamBeginCapture(c->cap, cudaStreamCaptureModeThreadLocal) == cudaSuccess;
     if (ok) {
-        cudaError_t e = launch_noise(c, c->cap);
-        for (int t = 0; t < c->P.T && e == cudaSuccess; ++t)
+        cudaError_t e = noise ? launch_noise(c, c->cap) : cudaSuccess;
+        for (int t = 0; t < steps && e == cudaSuccess; ++t)
             e = conditional ? capture_step_conditional(c, c->cap, overlap, t) : capture_step_gated(c, c->cap, overlap, t);
         const cudaError_t e2 = cudaStreamEndCapture(c->cap, &g);
         ok = e == cudaSuccess && e2 == cudaSuccess && g != nullptr;
     }
-    if (ok) ok = cudaGraphInstantiate(&c->gexec, g, 0) == cudaSuccess;
+    if (ok) ok = cudaGraphInstantiate(exec, g, 0) == cudaSuccess;
     if (g) cudaGraphDestroy(g);
     if (!ok) {
-        c->gexec = nullptr;
+        *exec = nullptr;
         cudaGetLastError();
+        return false;
     }
-    c->overlap_graph = ok && overlap;
-    return ok;
+    c->overlap_graph = overlap;
+    return true;
 }
 
 // Particles from which the rebuild goes into a conditional node: the node costs
@@ -712,6 +724,25 @@ bool capture_graph_mode(gld_ctx* c, bool conditional)
 // 262144: 185.5 against 185.7).
 constexpr int kConditionalMinN = 262144;
 
+// Steps of a piece of a noise block that is replayed as a graph: a block of the
+// convolution.  A program that steps by fewer than 64 otherwise launches every
+// kernel by itself (37 us per step at 10000 particles where a graph takes 20);
+// the piece is captured once some 64 steps went that way.
+int segment_steps(const gld_ctx* c) { return c->P.cblk ? c->conv_len : 8; }
+
+bool capture_segment(gld_ctx* c)
+{
+    if (c->gseg) return true;
+    if (c->graph_failed || c->P.pn_kry || c->eager_steps < c->P.T) return false;
+    const bool conditional = c->prm.use_graphs != 2 && c->P.n >= kConditionalMinN;
+    if (!capture_graph_mode(c, conditional, segment_steps(c), false, &c->gseg)) {
+        c->graph_failed = true;
+        return false;
+    }
+    if (c->graph_mode == 0) c->graph_mode = conditional ? 2 : 1;
+    return true;
+}
+
 bool capture_graph(gld_ctx* c)
 {
     if (c->gexec && c->cluster_graph) invalidate_graph(c);  // the system left the cluster path
@@ -719,11 +750,12 @@ bool capture_graph(gld_ctx* c)
     if (c->graph_failed || c->P.pn_kry) return false;  // the Lanczos noise decides on the host every step
     // conditional rebuild for large systems; the gated kernels otherwise, and
     // as the fallback
-    if (c->prm.use_graphs != 2 && c->P.n >= kConditionalMinN && capture_graph_mode(c, true)) {
+    if (c->prm.use_graphs != 2 && c->P.n >= kConditionalMinN &&
+        capture_graph_mode(c, true, c->P.T, true, &c->gexec)) {
         c->graph_mode = 2;
         return true;
     }
-    if (capture_graph_mode(c, false)) {
+    if (capture_graph_mode(c, false, c->P.T, true, &c->gexec)) {
         c->graph_mode = 1;
         return true;
     }
@@ -1171,36 +1203,46 @@ gld_status gld_step(gld_ctx* c, int64_t nsteps)
     const int T = c->P.T;
     if (nsteps > 0) GLD_TRY(ring_form(c, true, c->st));
     if (nsteps > 0) GLD_TRY(refresh_modes(c));
-    if (steps_in_cluster(c)) return step_cluster(c, nsteps);
+    const bool cluster = steps_in_cluster(c);
     while (nsteps > 0) {
-        if (!c->noise_valid || c->host_step >= c->noise_end) {
-            if (c->prm.use_graphs && nsteps >= T && capture_graph(c)) {
-                // the overlapped graph starts from the projections of its first step
-                // (and the parts of their block)
-                c->block_start = c->host_step;
-                if (c->P.cblk && c->part_step != c->host_step) c->conv_valid_step = -1;
-                if (c->overlap_graph) GLD_CUDA(c, launch_memory(c, c->st));
-                GLD_CUDA(c, cudaGraphLaunch(c->gexec, c->st));
-                c->host_step += T;
-                c->conv_valid_step = c->overlap_graph ? c->host_step : -1;
-                c->part_step = c->overlap_graph && c->P.cblk ? c->host_step : -1;
-                c->noise_end = c->host_step;
-                c->noise_valid = true;
-                c->last_fr_row = T - 1;
-                nsteps -= T;
-                continue;
-            }
+        const bool boundary = !c->noise_valid || c->host_step >= c->noise_end;
+        // a whole noise block: the graph of the step kernels, but for the
+        // smallest systems
+        if (boundary && c->prm.use_graphs && nsteps >= T && !(cluster && c->P.n <= kClusterBlockMaxN) && capture_graph(c)) {
+            c->block_start = c->host_step;
+            GLD_TRY(replay(c, c->gexec, T));
+            c->noise_end = c->host_step;
+            c->noise_valid = true;
+            c->last_fr_row = T - 1;
+            nsteps -= T;
+            continue;
+        }
+        if (cluster) {
+            const int64_t k = boundary ? std::min<int64_t>(nsteps, T) : std::min<int64_t>(nsteps, c->noise_end - c->host_step);
+            GLD_TRY(step_cluster(c, k, boundary));
+            nsteps -= k;
+            continue;
+        }
+        if (boundary) {
             GLD_CUDA(c, launch_noise(c, c->st));
             c->block_start = c->host_step;
             c->noise_end = c->host_step + T;
             c->noise_valid = true;
             if (c->P.pn_kry && c->kry.window) GLD_TRY(pair_noise_krylov(c, c->st));  // the block's rows at once
         }
+        const int seg = segment_steps(c);
+        if (c->prm.use_graphs && nsteps >= seg && (c->host_step - c->block_start) % seg == 0 && capture_segment(c)) {
+            GLD_TRY(replay(c, c->gseg, seg));
+            c->last_fr_row = c->host_step - 1 - c->block_start;
+            nsteps -= seg;
+            continue;
+        }
         if (c->P.pn_kry && !c->kry.window) GLD_TRY(pair_noise_krylov(c, c->st));
         GLD_CUDA(c, launch_one_step(c, c->st));
         c->conv_valid_step = -1;
         c->last_fr_row = c->host_step - c->block_start;
         ++c->host_step;
+        ++c->eager_steps;
         --nsteps;
     }
     return GLD_OK;

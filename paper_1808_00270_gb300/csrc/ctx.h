@@ -24,6 +24,8 @@ struct gld_ctx {
     cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
     bool overlap_graph = false;  // the graph computes each step's successor convolution
     long long conv_valid_step = -1;  // the step whose projections `conv` already holds
+    cudaGraphExec_t gseg = nullptr;  // a piece of a noise block (without the noise)
+    long long eager_steps = 0;       // steps launched kernel by kernel since the graphs were dropped
     bool cluster_graph = false;      // gexec holds a noise block and its steps in one kernel
     int conv_G = 0, conv_len = 0;    // split of a column's slots; steps of a block of the convolution
     long long part_step = -1;        // first step of the block whose parts B.part holds

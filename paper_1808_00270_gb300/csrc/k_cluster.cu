@@ -27,6 +27,7 @@
 #include <cuda_bf16.h>
 
 #include "history.cuh"
+#include "neighbours.cuh"
 
 namespace gld {
 
@@ -39,30 +40,10 @@ __device__ __forceinline__ void cluster_barrier()
     asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
-// Plain loads (L1 / L2, not the read-only path) of data written by other CTAs.
-__device__ __forceinline__ float4 ld4(const float4* p)
-{
-    float4 v;
-    asm volatile("ld.global.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(p) : "memory");
-    return v;
-}
-__device__ __forceinline__ float ld1(const float* p)
-{
-    float v;
-    asm volatile("ld.global.f32 %0, [%1];" : "=f"(v) : "l"(p) : "memory");
-    return v;
-}
-__device__ __forceinline__ int ldi(const int* p)
-{
-    int v;
-    asm volatile("ld.global.s32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
-    return v;
-}
-
-__device__ __forceinline__ float cl_dot3(float ax, float ay, float az, float bx, float by, float bz)
-{
-    return fmaf(ax, bx, fmaf(ay, by, az * bz));
-}
+// Data written by other CTAs: plain loads.
+__device__ __forceinline__ float4 ld4(const float4* p) { return LdPlain::f4(p); }
+__device__ __forceinline__ float ld1(const float* p) { return LdPlain::f1(p); }
+__device__ __forceinline__ int ldi(const int* p) { return LdPlain::i1(p); }
 
 struct ClSched {  // the VACF's view of a step (vacf_schedule in k_particles.cu)
     int on, nact, slot0, origin, lag0, buf, pending;
@@ -503,9 +484,7 @@ __device__ __forceinline__ void cl_conv(const StepParams& P, const ParticleBuffe
 }
 
 // Steps of one system.  NACC 1: self kernel only; 2: one separable pair term.
-// L lanes share a particle: lane l of a round takes the E list entries from
-// l E on, so a list of up to L E entries costs one chain of loads; their terms
-// are then added in list order by every lane (shuffles), as one thread would.
+// L lanes share a particle (neighbours.cuh).
 // The convolution's blocks have G ranges and len steps; rel0 is the number of
 // the first step in its block (> 0: the block's parts are formed).
 template <int NACC, bool BF16, int L>
@@ -524,8 +503,8 @@ __device__ __forceinline__ void cl_steps(const SysDesc& d, int nsteps, int rel0,
         cs[x] = m >= 1 && m <= H ? __ldg(d.coef + (size_t)a * M + m) : 0.f;
     }
     int* lists = (int*)(cs + NACC * ncs);  // [kClThreads / L][maxnb]
-    const int lane = tid & (L - 1), grp = tid / L;
-    const unsigned gmask = (L == 32 ? 0xffffffffu : ((1u << L) - 1u)) << ((tid & 31) & ~(L - 1));
+    const Lanes<L> ln;
+    const int lane = ln.lane, grp = tid / L;
     const int pstride = ncta * (kClThreads / L), p0 = rank * (kClThreads / L) + grp;
     const int iters = (n + pstride - 1) / pstride;
     const int cthreads = ncta * kClThreads, g0 = rank * kClThreads + tid;
@@ -587,64 +566,10 @@ __device__ __forceinline__ void cl_steps(const SysDesc& d, int nsteps, int rel0,
             }
             float f0x = 0.f, f0y = 0.f, f0z = 0.f, fhx = 0.f, fhy = 0.f, fhz = 0.f;
             if (NACC > 1) {
-                const float* pj0 = B.conv + S;
-                const int* nb = B.nbr + i;
-                int jn[E];  // entries past the list: any earlier particle index, masked below
-#pragma unroll
-                for (int u = 0; u < E; ++u) jn[u] = lane * E + u < P.maxnb ? ldi(nb + (size_t)(lane * E + u) * np) : i;
-                const int cnt = ldi(B.nbr_cnt + i);
-                for (int s = 0; s < cnt; s += L * E) {
-                    int j[E];
-                    float4 pj[E], vj[E];
-                    float qx[E], qy[E], qz[E];
-#pragma unroll
-                    for (int u = 0; u < E; ++u) j[u] = s + lane * E + u < cnt ? jn[u] : i;
-#pragma unroll
-                    for (int u = 0; u < E; ++u) {
-                        pj[u] = ld4(cur + j[u]);
-                        vj[u] = ld4(B.vel + j[u]);
-                        qx[u] = ld1(pj0 + j[u]);
-                        qy[u] = ld1(pj0 + np + j[u]);
-                        qz[u] = ld1(pj0 + 2 * np + j[u]);
-                    }
-#pragma unroll
-                    for (int u = 0; u < E; ++u) {
-                        const int e = s + L * E + lane * E + u;
-                        jn[u] = e < cnt ? ldi(nb + (size_t)e * np) : i;
-                    }
-                    float inst[E], hist[E], ex[E], ey[E], ez[E];
-#pragma unroll
-                    for (int u = 0; u < E; ++u) {
-                        const float dx = min_image_fma(pi.x, pj[u].x, P.box, P.inv_box);
-                        const float dy = min_image_fma(pi.y, pj[u].y, P.box, P.inv_box);
-                        const float dz = min_image_fma(pi.z, pj[u].z, P.box, P.inv_box);
-                        const float r2 = dist2(dx, dy, dz);
-                        inst[u] = hist[u] = ex[u] = ey[u] = ez[u] = 0.f;  // adds exactly nothing
-                        if (j[u] != i && r2 < P.rc2) {
-                            const float inv_r = rsqrtf(r2);
-                            const float r = r2 * inv_r;
-                            ex[u] = dx * inv_r;
-                            ey[u] = dy * inv_r;
-                            ez[u] = dz * inv_r;
-                            const float x = fmaxf(r, P.rc_min) * P.inv_dr;
-                            const float evj = cl_dot3(ex[u], ey[u], ez[u], vj[u].x, vj[u].y, vj[u].z);
-                            const float fq = table_at(B.ftab, P.nr, x);
-                            const float epj = cl_dot3(ex[u], ey[u], ez[u], qx[u], qy[u], qz[u]);
-                            inst[u] = fmaf(fq * g00, evj, 0.f);
-                            hist[u] = fmaf(fq, epj, 0.f);
-                        }
-                    }
-                    const int left = min(L, (cnt - s + E - 1) / E);
-                    for (int l = 0; l < left; ++l)
-#pragma unroll
-                        for (int u = 0; u < E; ++u) {
-                            const float in = __shfl_sync(gmask, inst[u], l, L), hi = __shfl_sync(gmask, hist[u], l, L);
-                            const float x = __shfl_sync(gmask, ex[u], l, L), y = __shfl_sync(gmask, ey[u], l, L),
-                                        z = __shfl_sync(gmask, ez[u], l, L);
-                            f0x = fmaf(-in, x, f0x); f0y = fmaf(-in, y, f0y); f0z = fmaf(-in, z, f0z);
-                            fhx = fmaf(-hi, x, fhx); fhy = fmaf(-hi, y, fhy); fhz = fmaf(-hi, z, fhz);
-                        }
-                }
+                float f0[3] = {0.f, 0.f, 0.f}, fh[3] = {0.f, 0.f, 0.f};
+                pair_sums<LdPlain, L, E>(P, ln, cur, B.vel, B.conv + S, B.nbr + i, B.nbr_cnt + i, i, pi, B.ftab, g00, f0, fh);
+                f0x = f0[0]; f0y = f0[1]; f0z = f0[2];
+                fhx = fh[0]; fhy = fh[1]; fhz = fh[2];
             }
             if (lane != 0) continue;
             const float fdx = fmaf(fhx - sx[0], P.inv_dt, f0x);
@@ -694,50 +619,9 @@ __device__ __forceinline__ void cl_steps(const SysDesc& d, int nsteps, int rel0,
             const float4 pi = ld4(nxt + i);
             float4 vh;
             if (lane == 0) vh = ld4(B.vhalf + i);
-            const int* nb = B.nbr + i;
-            int jn[E];
-#pragma unroll
-            for (int u = 0; u < E; ++u) jn[u] = lane * E + u < P.maxnb ? ldi(nb + (size_t)(lane * E + u) * np) : i;
-            const int cnt = ldi(B.nbr_cnt + i);
-            float fx = 0.f, fy = 0.f, fz = 0.f;
-            for (int s = 0; s < cnt; s += L * E) {
-                int j[E];
-                float4 pj[E];
-#pragma unroll
-                for (int u = 0; u < E; ++u) j[u] = s + lane * E + u < cnt ? jn[u] : i;
-#pragma unroll
-                for (int u = 0; u < E; ++u) pj[u] = ld4(nxt + j[u]);
-#pragma unroll
-                for (int u = 0; u < E; ++u) {
-                    const int e = s + L * E + lane * E + u;
-                    jn[u] = e < cnt ? ldi(nb + (size_t)e * np) : i;
-                }
-                float sc[E], dx[E], dy[E], dz[E];
-#pragma unroll
-                for (int u = 0; u < E; ++u) {
-                    dx[u] = min_image_fma(pi.x, pj[u].x, P.box, P.inv_box);
-                    dy[u] = min_image_fma(pi.y, pj[u].y, P.box, P.inv_box);
-                    dz[u] = min_image_fma(pi.z, pj[u].z, P.box, P.inv_box);
-                    const float r2 = dist2(dx[u], dy[u], dz[u]);
-                    if (j[u] != i && r2 < P.rc2) {
-                        const float inv_r = rsqrtf(r2);
-                        const float r = r2 * inv_r;
-                        sc[u] = (P.fc_nr > 0 ? table_at(B.fctab, P.fc_nr, r * P.fc_inv_dr)
-                                             : P.fc_mag * (1.0f - r * P.inv_rc)) * inv_r;
-                    } else {
-                        sc[u] = dx[u] = dy[u] = dz[u] = 0.f;  // adds exactly nothing
-                    }
-                }
-                const int left = min(L, (cnt - s + E - 1) / E);
-                for (int l = 0; l < left; ++l)
-#pragma unroll
-                    for (int u = 0; u < E; ++u) {
-                        const float k = __shfl_sync(gmask, sc[u], l, L);
-                        fx = fmaf(k, __shfl_sync(gmask, dx[u], l, L), fx);
-                        fy = fmaf(k, __shfl_sync(gmask, dy[u], l, L), fy);
-                        fz = fmaf(k, __shfl_sync(gmask, dz[u], l, L), fz);
-                    }
-            }
+            float f[3] = {0.f, 0.f, 0.f};
+            cforce_sums<LdPlain, L, E>(P, ln, nxt, B.nbr + i, B.nbr_cnt + i, i, pi, B.fctab, f);
+            const float fx = f[0], fy = f[1], fz = f[2];
             if (lane != 0) continue;
             B.fc[i] = make_float4(fx, fy, fz, 0.f);
             B.vel[i] = make_float4(fmaf(P.vf_fc, fx, vh.x), fmaf(P.vf_fc, fy, vh.y), fmaf(P.vf_fc, fz, vh.z), 0.f);

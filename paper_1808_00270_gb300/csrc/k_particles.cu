@@ -27,6 +27,7 @@
 #include <cuda_bf16.h>
 
 #include "launch.h"
+#include "neighbours.cuh"
 
 namespace gld {
 
@@ -38,6 +39,7 @@ constexpr int kPairBatch = 4;                 // list entries per round of the o
 constexpr int kCforceLanes = kBatchCforceLanes;  // lanes per particle in the F^C kernel
 constexpr int kCellThreads = kBatchCellChunk;
 constexpr int kThreads = kBatchPartBlock;
+constexpr int kLanesMaxN = 22528;  // particles up to which the neighbour kernels take several lanes each
 constexpr int kNbrSortCap = 128;  // list entries sorted by id at each build
 static_assert(kBatchVacfBlock == kThreads, "vacf blocks share the particle block size");
 
@@ -80,6 +82,70 @@ __device__ __forceinline__ void vacf_schedule(const StepParams& P, Ctrl* __restr
     ctrl->vacf_lag0 = lag0;
 }
 
+// The rest of a particle's pair step from its neighbour sums: F^D, R_{n+1}, the
+// displacement into the ring, the velocity part known now, the rebuild request.
+__device__ __forceinline__ void pair_finish(const StepParams& P, Ctrl* __restrict__ ctrl, long long n, int id,
+                                            const float4 pi, const float4 vi, float f0x, float f0y, float f0z, float fhx,
+                                            float fhy, float fhz, const float4* __restrict__ fc,
+                                            const float* __restrict__ conv, const float* __restrict__ frblock,
+                                            void* __restrict__ ring, float4* __restrict__ pos_next,
+                                            float4* __restrict__ vhalf, float4* __restrict__ fd_out,
+                                            float4* __restrict__ disp, const float4* __restrict__ disp_build)
+{
+    unsigned* err = &ctrl->err;
+    const long long np = P.n_pad;
+    // F^D = -sum_j (K^p_0 V_j + dK^s_0 V_i) - (1/dt) (S_i + sum_j ...)
+    const float sx = conv[id], sy = conv[np + id], sz = conv[2 * np + id];
+    const float fdx = fmaf(fhx - sx, P.inv_dt, f0x);
+    const float fdy = fmaf(fhy - sy, P.inv_dt, f0y);
+    const float fdz = fmaf(fhz - sz, P.inv_dt, f0z);
+    const long long row = n - ctrl->noise_n0;
+    float frx = 0.f, fry = 0.f, frz = 0.f;
+    if (row >= 0 && row < P.T) {
+        const float* fr = frblock + (size_t)row * 3 * np + id;
+        frx = fr[0];
+        fry = fr[np];
+        frz = fr[2 * np];
+    } else if (id == 0) {
+        atomicOr(err, kErrNoise);  // the host scheduled a step outside the noise block
+    }
+    const float4 fci = fc[id];
+    // Eq. GLD_integrator, position: dR = b dt V + b dt^2/(2M) (F^C + F^D + F^R)
+    const float dRx = fmaf(P.pos_f, fci.x + fdx + frx, P.pos_v * vi.x);
+    const float dRy = fmaf(P.pos_f, fci.y + fdy + fry, P.pos_v * vi.y);
+    const float dRz = fmaf(P.pos_f, fci.z + fdz + frz, P.pos_v * vi.z);
+    const long long slot = ctrl->hslot;  // n mod H
+    if (P.hist_bf16) {
+        __nv_bfloat16* h = (__nv_bfloat16*)ring + (size_t)slot * 3 * np + id;
+        h[0] = __float2bfloat16_rn(dRx);
+        h[np] = __float2bfloat16_rn(dRy);
+        h[2 * np] = __float2bfloat16_rn(dRz);
+    } else {
+        float* h = (float*)ring + (size_t)slot * 3 * np + id;
+        h[0] = dRx;
+        h[np] = dRy;
+        h[2 * np] = dRz;
+    }
+    pos_next[id] = make_float4(wrap_box(__fadd_rn(pi.x, dRx), P.box), wrap_box(__fadd_rn(pi.y, dRy), P.box),
+                               wrap_box(__fadd_rn(pi.z, dRz), P.box), 0.f);
+    // velocity part known now: a V + a dt/(2M) F^C_n + b dt/M (F^D + F^R)
+    vhalf[id] = make_float4(fmaf(P.vh_f, fdx + frx, fmaf(P.vh_fc, fci.x, P.vh_v * vi.x)),
+                            fmaf(P.vh_f, fdy + fry, fmaf(P.vh_fc, fci.y, P.vh_v * vi.y)),
+                            fmaf(P.vh_f, fdz + frz, fmaf(P.vh_fc, fci.z, P.vh_v * vi.z)), 0.f);
+    fd_out[id] = make_float4(fdx, fdy, fdz, 0.f);
+    const float4 d = disp[id];
+    const float4 dn = make_float4(d.x + dRx, d.y + dRy, d.z + dRz, 0.f);
+    disp[id] = dn;
+    // Verlet criterion: a particle moved more than half the skin since the build.
+    const float4 db = disp_build[id];
+    const float mx = dn.x - db.x, my = dn.y - db.y, mz = dn.z - db.z;
+    if (mx * mx + my * my + mz * mz > P.trig2) atomicOr(&ctrl->rebuild, 1);
+    if (!(isfinite(dRx) && isfinite(dRy) && isfinite(dRz))) {
+        atomicOr(err, kErrNonFinite);
+        atomicOr(&ctrl->rebuild, 1);
+    }
+}
+
 // FAST: exactly one separable pair term and no self-difference term.
 template <bool FAST>
 __device__ __forceinline__ void pair_force_integrate_body(const StepParams& P, Ctrl* __restrict__ ctrl, const float4* __restrict__ pos,
@@ -91,7 +157,6 @@ __device__ __forceinline__ void pair_force_integrate_body(const StepParams& P, C
                          float4* __restrict__ vhalf, float4* __restrict__ fd_out, float4* __restrict__ disp,
                          const float4* __restrict__ disp_build, int blk, int nblk)
 {
-    unsigned* err = &ctrl->err;
     // FAST: kPairLanes consecutive lanes share a particle and split its list
     constexpr int LANES = FAST ? kPairLanes : 1;
     const int k = (blk * blockDim.x + threadIdx.x) / LANES;
@@ -241,56 +306,8 @@ __device__ __forceinline__ void pair_force_integrate_body(const StepParams& P, C
             }
         });
     }
-    // F^D = -sum_j (K^p_0 V_j + dK^s_0 V_i) - (1/dt) (S_i + sum_j ...)
-    const float sx = conv[id], sy = conv[np + id], sz = conv[2 * np + id];
-    const float fdx = fmaf(fhx - sx, P.inv_dt, f0x);
-    const float fdy = fmaf(fhy - sy, P.inv_dt, f0y);
-    const float fdz = fmaf(fhz - sz, P.inv_dt, f0z);
-    const long long row = n - ctrl->noise_n0;
-    float frx = 0.f, fry = 0.f, frz = 0.f;
-    if (row >= 0 && row < P.T) {
-        const float* fr = frblock + (size_t)row * 3 * np + id;
-        frx = fr[0];
-        fry = fr[np];
-        frz = fr[2 * np];
-    } else if (k == 0) {
-        atomicOr(err, kErrNoise);  // the host scheduled a step outside the noise block
-    }
-    const float4 fci = fc[id];
-    // Eq. GLD_integrator, position: dR = b dt V + b dt^2/(2M) (F^C + F^D + F^R)
-    const float dRx = fmaf(P.pos_f, fci.x + fdx + frx, P.pos_v * vi.x);
-    const float dRy = fmaf(P.pos_f, fci.y + fdy + fry, P.pos_v * vi.y);
-    const float dRz = fmaf(P.pos_f, fci.z + fdz + frz, P.pos_v * vi.z);
-    const long long slot = ctrl->hslot;  // n mod H
-    if (P.hist_bf16) {
-        __nv_bfloat16* h = (__nv_bfloat16*)ring + (size_t)slot * 3 * np + id;
-        h[0] = __float2bfloat16_rn(dRx);
-        h[np] = __float2bfloat16_rn(dRy);
-        h[2 * np] = __float2bfloat16_rn(dRz);
-    } else {
-        float* h = (float*)ring + (size_t)slot * 3 * np + id;
-        h[0] = dRx;
-        h[np] = dRy;
-        h[2 * np] = dRz;
-    }
-    pos_next[id] = make_float4(wrap_box(__fadd_rn(pi.x, dRx), P.box), wrap_box(__fadd_rn(pi.y, dRy), P.box),
-                               wrap_box(__fadd_rn(pi.z, dRz), P.box), 0.f);
-    // velocity part known now: a V + a dt/(2M) F^C_n + b dt/M (F^D + F^R)
-    vhalf[id] = make_float4(fmaf(P.vh_f, fdx + frx, fmaf(P.vh_fc, fci.x, P.vh_v * vi.x)),
-                            fmaf(P.vh_f, fdy + fry, fmaf(P.vh_fc, fci.y, P.vh_v * vi.y)),
-                            fmaf(P.vh_f, fdz + frz, fmaf(P.vh_fc, fci.z, P.vh_v * vi.z)), 0.f);
-    fd_out[id] = make_float4(fdx, fdy, fdz, 0.f);
-    const float4 d = disp[id];
-    const float4 dn = make_float4(d.x + dRx, d.y + dRy, d.z + dRz, 0.f);
-    disp[id] = dn;
-    // Verlet criterion: a particle moved more than half the skin since the build.
-    const float4 db = disp_build[id];
-    const float mx = dn.x - db.x, my = dn.y - db.y, mz = dn.z - db.z;
-    if (mx * mx + my * my + mz * mz > P.trig2) atomicOr(&ctrl->rebuild, 1);
-    if (!(isfinite(dRx) && isfinite(dRy) && isfinite(dRz))) {
-        atomicOr(err, kErrNonFinite);
-        atomicOr(&ctrl->rebuild, 1);
-    }
+    pair_finish(P, ctrl, n, id, pi, vi, f0x, f0y, f0z, fhx, fhy, fhz, fc, conv, frblock, ring, pos_next, vhalf, fd_out,
+                disp, disp_build);
 }
 
 template <bool FAST>
@@ -304,6 +321,46 @@ __global__ void __launch_bounds__(kPairThreads) pair_force_integrate(const StepP
                          const float4* __restrict__ disp_build)
 {
     pair_force_integrate_body<FAST>(P, ctrl, pos, perm, nbr, nbr_cnt, vel, fc, conv, frblock, ftab, fptab, g0, ring, pos_next, vhalf, fd_out, disp, disp_build, blockIdx.x, gridDim.x);
+}
+
+// The same with L lanes per particle (neighbours.cuh), for systems too small to
+// fill the chip with one.
+template <bool FAST, int L>
+__global__ void __launch_bounds__(kThreads) pair_lanes(const StepParams P, Ctrl* __restrict__ ctrl, const float4* __restrict__ pos,
+                         const int* __restrict__ nbr, const int* __restrict__ nbr_cnt,
+                         const float4* __restrict__ vel, const float4* __restrict__ fc, const float* __restrict__ conv,
+                         const float* __restrict__ frblock, const float* __restrict__ ftab,
+                         const float* __restrict__ fptab,
+                         const float* __restrict__ g0, void* __restrict__ ring, float4* __restrict__ pos_next,
+                         float4* __restrict__ vhalf, float4* __restrict__ fd_out, float4* __restrict__ disp,
+                         const float4* __restrict__ disp_build)
+{
+    const Lanes<L> ln;
+    const int id = (int)((blockIdx.x * blockDim.x + threadIdx.x) / L);
+    if (id >= P.n) return;  // uniform over the lanes of a particle
+    const long long n = ctrl->step;
+    const size_t np = P.n_pad;
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        ctrl->conv_step = n + 1;
+        if (P.vacf_len > 0) vacf_schedule(P, ctrl, n + 1);
+    }
+    const float4 pi = pos[id], vi = vel[id];
+    float f0[3] = {0.f, 0.f, 0.f}, fh[3] = {0.f, 0.f, 0.f};
+    if constexpr (FAST) {
+        pair_sums<LdConst, L, (L >= 8 ? 2 : 4)>(P, ln, pos, vel, conv + 3 * np, nbr + id, nbr_cnt + id, id, pi, ftab,
+                                                __ldg(g0), f0, fh);
+    } else if (P.Q + P.Qs > 0) {
+        float ps[kMaxQ][3];
+#pragma unroll
+        for (int q = 0; q < kMaxQ; ++q)
+#pragma unroll
+            for (int c = 0; c < 3; ++c) ps[q][c] = q < P.Qs ? conv[(size_t)(1 + P.Q + q) * 3 * np + c * np + id] : 0.f;
+        pair_sums_general<LdConst, L>(P, ln, pos, vel, conv, nbr + id, nbr_cnt + id, id, pi, vi, ps, ftab, fptab, g0, f0,
+                                      fh);
+    }
+    if (ln.lane == 0)
+        pair_finish(P, ctrl, n, id, pi, vi, f0[0], f0[1], f0[2], fh[0], fh[1], fh[2], fc, conv, frblock, ring, pos_next,
+                    vhalf, fd_out, disp, disp_build);
 }
 
 // ---- cell list --------------------------------------------------------------
@@ -618,23 +675,26 @@ __device__ __forceinline__ void vacf_fold(const StepParams& P, const float* __re
     __shared__ float sh[kThreads / 32][2];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const float* base = partial + (size_t)buf * P.n_os * nblk;
+    // the first kThreads threads of the block (there may be more); its barriers
+    // are joined by all
+    const bool act = threadIdx.x < kThreads;
     for (int q = first; q < nact; q += step) {
         float hi = 0.f, lo = 0.f;
-        for (int b = threadIdx.x; b < nblk; b += blockDim.x)
+        for (int b = threadIdx.x; act && b < nblk; b += kThreads)
             df_add(hi, lo, __ldcg(base + (size_t)q * nblk + b), 0.f);
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) {
             const float h2 = __shfl_xor_sync(0xffffffffu, hi, o), l2 = __shfl_xor_sync(0xffffffffu, lo, o);
             df_add(hi, lo, h2, l2);
         }
-        if (lane == 0) {
+        if (act && lane == 0) {
             sh[warp][0] = hi;
             sh[warp][1] = lo;
         }
         __syncthreads();
         if (threadIdx.x == 0) {
             float h = 0.f, l = 0.f;
-            for (int w = 0; w < (int)(blockDim.x >> 5); ++w) df_add(h, l, sh[w][0], sh[w][1]);
+            for (int w = 0; w < kThreads / 32; ++w) df_add(h, l, sh[w][0], sh[w][1]);
             const int lg = lag0 + q * P.vacf_stride;  // < vacf_len for q < nact
             csum[lg] += (double)h + (double)l;
             ccnt[lg] += 1;
@@ -692,6 +752,61 @@ __device__ __forceinline__ void cforce_vacf(const StepParams& P, Ctrl* __restric
         __syncthreads();
     }
     if (is_origin && valid) vorig[(size_t)slot0 * P.n + i] = v;
+}
+
+// The same from the velocities of the block's 256 particles in shared memory,
+// in a block of 256 L threads: the first 256 take the particles, all threads
+// join the barriers (the fold runs on all of them for its own origins).
+template <int L>
+__device__ __forceinline__ void cforce_vacf(const StepParams& P, Ctrl* __restrict__ ctrl, const float4* vsh, int blk,
+                                            int nblk, float4* __restrict__ vorig, float* __restrict__ partial,
+                                            double* __restrict__ csum, long long* __restrict__ ccnt,
+                                            long long* __restrict__ norig)
+{
+    const bool act = threadIdx.x < kThreads;
+    if (ctrl->pv_nact > 0)  // uniform over the block
+        vacf_fold(P, partial, csum, ccnt, ctrl->pv_buf, ctrl->pv_nact, ctrl->pv_lag0, nblk, blk, nblk);
+    if (!ctrl->vacf_on) return;  // uniform over the grid
+    const int n_act = ctrl->vacf_nact;
+    const bool is_origin = ctrl->vacf_origin != 0;
+    const int slot0 = ctrl->vacf_slot0;  // slot of age j: (slot0 - j) mod n_os
+    if (blk == 0 && threadIdx.x == 0) {
+        ctrl->vacf_pending = 1;
+        if (is_origin) *norig += 1;
+    }
+    // groups of 256 threads take the origins 4 g .. 4 g + 3 in turn
+    __shared__ float wsum[kThreads * L / 32][kVacfGroup];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, g = threadIdx.x / kThreads, p = threadIdx.x % kThreads;
+    const int i = blk * kThreads + p;
+    const bool valid = i < P.n;
+    const float4 v = valid ? vsh[p] : make_float4(0.f, 0.f, 0.f, 0.f);
+    float* out = partial + (size_t)ctrl->vacf_buf * P.n_os * nblk;
+    for (int b0 = 0; b0 < n_act; b0 += kVacfGroup * L) {
+        const int q0 = b0 + kVacfGroup * g;
+        float4 w[kVacfGroup];
+#pragma unroll
+        for (int q = 0; q < kVacfGroup; ++q) {
+            const int j = q0 + q;
+            const int sl = slot0 - j < 0 ? slot0 - j + P.n_os : slot0 - j;
+            // the origin of age 0 on an origin step is V_{n+1} itself
+            const bool use = valid && j < n_act && !(j == 0 && is_origin);
+            w[q] = use ? __ldcs(vorig + (size_t)sl * P.n + i) : v;
+        }
+#pragma unroll
+        for (int q = 0; q < kVacfGroup; ++q) {
+            const float d = (valid && q0 + q < n_act) ? fmaf(v.x, w[q].x, fmaf(v.y, w[q].y, v.z * w[q].z)) : 0.f;
+            const float sq = warp_sum_f(d);
+            if (lane == 0) wsum[warp][q] = sq;
+        }
+        __syncthreads();
+        if (p < kVacfGroup && q0 + p < n_act) {
+            float sb = 0.f;
+            for (int w2 = 0; w2 < kThreads / 32; ++w2) sb += wsum[(kThreads / 32) * g + w2][p];
+            out[(size_t)(q0 + p) * nblk + blk] = sb;
+        }
+        __syncthreads();
+    }
+    if (is_origin && valid && act) vorig[(size_t)slot0 * P.n + i] = v;
 }
 
 // ---- conservative force and velocity finish --------------------------------
@@ -791,6 +906,50 @@ __global__ void __launch_bounds__(kThreads) cforce(const StepParams P, Ctrl* __r
 {
     cforce_body<STEP, VACF>(P, ctrl, pos_next, pos, perm, nbr, nbr_cnt, vhalf, vel, fc, fctab, blockIdx.x, gridDim.x,
                             vorig, vpartial, csum, ccnt, norig);
+}
+
+// The step form with L lanes per particle; with the VACF, blocks of 256
+// particles (its blocks), whose new velocities meet in shared memory.
+template <int L, bool VACF>
+__global__ void __launch_bounds__(kThreads * L) cforce_lanes(const StepParams P, Ctrl* __restrict__ ctrl,
+           const float4* __restrict__ pos_next, float4* __restrict__ pos, const int* __restrict__ nbr,
+           const int* __restrict__ nbr_cnt, const float4* __restrict__ vhalf, float4* __restrict__ vel,
+           float4* __restrict__ fc, const float* __restrict__ fctab, float4* __restrict__ vorig,
+           float* __restrict__ vpartial, double* __restrict__ csum, long long* __restrict__ ccnt,
+           long long* __restrict__ norig)
+{
+    __shared__ float4 vsh[VACF ? kThreads : 1];
+    const Lanes<L> ln;
+    const int grp = threadIdx.x / L, id = (int)(blockIdx.x * blockDim.x / L) + grp;
+    if (blockIdx.x == 0 && threadIdx.x == 0) ctrl->rebuild = 0;  // the lists are current for R_{n+1}
+    if (id < P.n) {  // uniform over the lanes of a particle
+        const float4 pi = pos_next[id];
+        float4 vh;
+        if (ln.lane == 0) vh = vhalf[id];
+        float f[3] = {0.f, 0.f, 0.f};
+        cforce_sums<LdConst, L, (L >= 8 ? 2 : 4)>(P, ln, pos_next, nbr + id, nbr_cnt + id, id, pi, fctab, f);
+        if (ln.lane == 0) {
+            pos[id] = pi;
+            fc[id] = make_float4(f[0], f[1], f[2], 0.f);
+            const float4 v = make_float4(fmaf(P.vf_fc, f[0], vh.x), fmaf(P.vf_fc, f[1], vh.y), fmaf(P.vf_fc, f[2], vh.z), 0.f);
+            vel[id] = v;
+            if (VACF) vsh[grp] = v;
+        }
+    }
+    if constexpr (VACF) {
+        __syncthreads();
+        cforce_vacf<L>(P, ctrl, vsh, (int)blockIdx.x, (int)gridDim.x, vorig, vpartial, csum, ccnt, norig);
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        __threadfence();
+        if (atomicAdd(&ctrl->done_cforce, 1u) == gridDim.x - 1) {
+            ctrl->step += 1;
+            ctrl->hslot = ctrl->hslot + 1 == P.H ? 0 : ctrl->hslot + 1;
+            ctrl->done_cforce = 0u;
+            __threadfence();
+        }
+    }
 }
 
 // Block (x, y) of the grid (gx <= 256 = blockDim) takes the particles
@@ -1277,6 +1436,46 @@ __device__ __forceinline__ void pn_stage_body(const StepParams& P, Ctrl* __restr
     if (S.last && !P.pn_iv && rowsum > P.pn_lambda) atomicOr(&ctrl->err, kErrPnBound);
 }
 
+template <int L>
+__global__ void __launch_bounds__(kThreads)
+    pn_stage_lanes(const StepParams P, Ctrl* __restrict__ ctrl, const float4* __restrict__ pos, const int* __restrict__ nbr,
+                   const int* __restrict__ nbr_cnt, const float* __restrict__ ftab, const float* __restrict__ fptab,
+                   const PnStage S)
+{
+    const Lanes<L> ln;
+    const int id = (int)((blockIdx.x * blockDim.x + threadIdx.x) / L);
+    if (id >= P.n) return;  // uniform over the lanes of a particle
+    const size_t np = P.n_pad;
+    const long long row = ctrl->step - ctrl->noise_n0;
+    if (row < 0 || row >= P.T) {
+        if (id == 0 && ln.lane == 0) atomicOr(&ctrl->err, kErrNoise);
+        return;
+    }
+    const size_t roff = (size_t)row * 3 * np;
+    const float* b1 = S.b1 + (S.b1_rows ? roff : 0);
+    const float* b2 = S.b2 ? S.b2 + (S.b2_rows ? roff : 0) : nullptr;
+    float* out = S.out + (S.out_rows ? roff : 0);
+    const float* z = S.z + roff;
+    const float bi[3] = {b1[id], b1[np + id], b1[2 * np + id]};
+    float zi[3] = {0.f, 0.f, 0.f}, b2i[3] = {0.f, 0.f, 0.f};
+    if (ln.lane == 0)
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            zi[c] = z[c * np + id];
+            if (b2) b2i[c] = b2[c * np + id];
+        }
+    float m[3] = {0.f, 0.f, 0.f}, rowsum = 0.f;
+    pn_sums<LdConst, L, 2>(P, ln, pos, nbr + id, nbr_cnt + id, id, pos[id], ftab, fptab, b1, bi, m, rowsum);
+    if (ln.lane != 0) return;
+    const float c = (S.last ? 1.0f : 2.0f) * P.pn_inv_lambda;
+#pragma unroll
+    for (int x = 0; x < 3; ++x) {
+        if (P.pn_cen != 0.f) m[x] = fmaf(-P.pn_cen, bi[x], m[x]);  // the interval [cen - rho, cen + rho]: (M - cen) b1
+        out[x * np + id] = fmaf(c, m[x], zi[x]) - b2i[x];
+    }
+    if (S.last && !P.pn_iv && rowsum > P.pn_lambda) atomicOr(&ctrl->err, kErrPnBound);
+}
+
 // Clenshaw stage k of a degree-K evaluation: b_K = Z_K (read in place), b_k
 // for K > k >= 1 in bvec[k % 3], the last stage writes F over the Z_0 row.
 __host__ __device__ __forceinline__ PnStage pn_stage_args(const StepParams& P, const float* frblock, const float* zblk,
@@ -1540,10 +1739,42 @@ cudaError_t launch_delay(unsigned long long ns, cudaStream_t st)
     return cudaGetLastError();
 }
 
+namespace {
+
+// Lanes per particle of the neighbour kernels of a system alone: eight while
+// they are at most about 1000 threads per SM.  Pair kernel, us (events) with
+// eight / one: 8.4 / 12.2 at 4096 particles, 9.7 / 12.2 at 10007, general form
+// 20.5 / 32.8 at 20000; with four / one 12.6 / 10.8 at 32768, with two / one
+// 19.7 / 16.7 at 65536: the shuffled additions cost more than they hide.
+int lanes_for(int n) { return n <= kLanesMaxN ? 8 : 1; }
+
+template <bool FAST, int L>
+cudaError_t pair_lanes_launch(const StepParams& P, const ParticleBuffers& B, cudaStream_t st)
+{
+    pair_lanes<FAST, L><<<(unsigned)(((long long)P.n * L + kThreads - 1) / kThreads), kThreads, 0, st>>>(
+        P, B.ctrl, B.pos, B.nbr, B.nbr_cnt, B.vel, B.fc, B.conv, B.frblock, B.ftab, B.fptab, B.g0, B.ring, B.pos_next,
+        B.vhalf, B.fd, B.disp, B.disp_build);
+    return cudaGetLastError();
+}
+
+template <int L>
+cudaError_t cforce_lanes_launch(const StepParams& P, const ParticleBuffers& B, bool vac, cudaStream_t st)
+{
+    auto k = vac ? cforce_lanes<L, true> : cforce_lanes<L, false>;
+    const int block = vac ? kThreads * L : kThreads;  // without the VACF, smaller blocks spread over more SMs
+    k<<<(unsigned)((P.n + block / L - 1) / (block / L)), block, 0, st>>>(
+        P, B.ctrl, B.pos_next, B.pos, B.nbr, B.nbr_cnt, B.vhalf, B.vel, B.fc, B.fctab, B.vorig, B.vpartial, B.csum, B.ccnt,
+        B.norig);
+    return cudaGetLastError();
+}
+
+}  // namespace
+
 cudaError_t launch_pair_force_integrate(const StepParams& P, const ParticleBuffers& B, cudaStream_t st)
 {
     const unsigned grid = (unsigned)((P.n + kPairThreads - 1) / kPairThreads);
     const bool fast = P.Q == 1 && P.Qs == 0 && !P.perp;
+    if (lanes_for(P.n) == 8) return fast ? pair_lanes_launch<true, 8>(P, B, st) : pair_lanes_launch<false, 8>(P, B, st);
     auto k = fast ? pair_force_integrate<true> : pair_force_integrate<false>;
     const unsigned pgrid = fast ? (unsigned)(((long long)P.n * kPairLanes + kPairThreads - 1) / kPairThreads) : grid;
     k<<<pgrid, kPairThreads, 0, st>>>(P, B.ctrl, B.pos, B.perm, B.nbr, B.nbr_cnt, B.vel, B.fc,
@@ -1584,6 +1815,8 @@ cudaError_t launch_cforce(const StepParams& P, const ParticleBuffers& B, int mod
     const unsigned grid = (unsigned)(((long long)P.n * kCforceLanes + kThreads - 1) / kThreads);
     const bool vac = mode && P.vacf_len > 0;
     if (vac && (P.n_os > kVacfMaxOrigins || (int)grid != B.vacf_gx)) return cudaErrorInvalidValue;
+    // (four lanes: a block of 256 particles for the VACF has 1024 threads)
+    if (mode && lanes_for(P.n) > 1) return cforce_lanes_launch<4>(P, B, vac, st);
     auto k = mode ? (vac ? cforce<true, true> : cforce<true, false>) : cforce<false, false>;
     k<<<grid, kThreads, 0, st>>>(P, B.ctrl, B.pos_next, B.pos, B.perm, B.nbr, B.nbr_cnt, B.vhalf, B.vel, B.fc,
                                  B.fctab, B.vorig, B.vpartial, B.csum, B.ccnt, B.norig);
@@ -1633,10 +1866,12 @@ cudaError_t launch_pair_noise(const StepParams& P, const ParticleBuffers& B, con
 {
     const int K = P.pn_deg;
     if (K <= 0) return cudaSuccess;
-    const unsigned grid = (unsigned)((P.n + kThreads - 1) / kThreads);
+    const int L = lanes_for(P.n);
+    auto kern = L == 8 ? pn_stage_lanes<8> : pn_stage;
+    const unsigned grid = (unsigned)(((long long)P.n * L + kThreads - 1) / kThreads);
     for (int k = K - 1; k >= 0; --k) {
-        pn_stage<<<grid, kThreads, 0, st>>>(P, B.ctrl, B.pos, B.nbr, B.nbr_cnt, B.ftab, B.fptab,
-                                            pn_stage_args(P, B.frblock, zblk, bvec, K, k));
+        kern<<<grid, kThreads, 0, st>>>(P, B.ctrl, B.pos, B.nbr, B.nbr_cnt, B.ftab, B.fptab,
+                                        pn_stage_args(P, B.frblock, zblk, bvec, K, k));
         const cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return e;
     }

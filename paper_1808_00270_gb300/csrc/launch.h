@@ -186,13 +186,18 @@ cudaError_t launch_batch_noise(const BatchPlan& bp, cudaStream_t st);     // k_n
 // size allow it; a system alone for nsteps steps of its noise block (rel0:
 // number of the first step in its block of the convolution, > 0: that block's
 // parts are formed; G and len as conv_block_shape).
+// Sizes (us per step, cluster against the graph of the step kernels): a whole
+// noise block 15.1 / 17.9 at 1000 particles, 17.9 / 16.6 at 2048, 21.4 / 17.1 at
+// 4096; launched for single steps 20.2 / 30.9, 23.7 / 31.0, 27.4 / 30.4.
 constexpr int kClusterMaxN = 4096;
+constexpr int kClusterBlockMaxN = 1536;
 bool cluster_ok(const StepParams& P, int kahan);
 cudaError_t launch_steps_cluster(const SysDesc& d, int nsteps, int rel0, int G, int len, cudaStream_t st);
 
 // The list build of launch_rebuild by one cluster (gated on ctrl->rebuild), for
-// systems where that is faster than the four kernels.
-constexpr int kClusterRebuildMaxN = 12288;
+// systems where that is faster than the four kernels (us per step 13.5 / 15.6 at
+// 4096 particles, 16.4 / 16.9 at 8192, 18.8 / 17.7 at 10007).
+constexpr int kClusterRebuildMaxN = 8192;
 bool rebuild_in_cluster(const StepParams& P);
 cudaError_t launch_rebuild_cluster(const StepParams& P, const ParticleBuffers& B, cudaStream_t st);
 
