@@ -1,6 +1,6 @@
 // k_noise.cu -- kernel preparation and the colored random force.
 //
-// prep (one block, FP64): discrete kernels of Eq. k-discrete, the noise target
+// prep_* (FP64): discrete kernels of Eq. k-discrete, the noise target
 //   C_m = kT a_m K^s_m / dt (Eq. FDT_discretized, a_0 = 2), its transform over
 //   the 2 m_max - 1 points of Eq. FT, the positive-semi-definiteness check,
 //   A_s = inverse transform of sqrt(hat C) (Sec. II C, with 1/(2 m_max - 1)),
@@ -20,13 +20,6 @@ namespace gld {
 namespace {
 
 constexpr int kPrepThreads = 1024;
-
-__device__ double cos_frac(long long w, long long m, long long L)
-{
-    long long r = (w * m) % L;
-    if (r < 0) r += L;
-    return cospi(2.0 * (double)r / (double)L);
-}
 
 __device__ double block_reduce(double v, double* sh, bool is_max)
 {
@@ -48,17 +41,30 @@ __device__ double discretize(const double* s, int m, double dt, int discrete)
     return m == 0 ? 0.5 * dt * s[0] : dt * s[m];
 }
 
-__global__ void __launch_bounds__(kPrepThreads) prep(const PrepArgs a)
+// cos(2 pi r / L), r < L: every angle of the transforms below is one of these.
+// (One block that evaluated FP64 cosines and 64-bit remainders term by term
+// took 2 to 3 ms of every gld_set_kernels at m_max = 300; the table and
+// kPrepTile outputs per block take about 0.1 ms.  Sums keep their order.)
+__device__ __forceinline__ void cos_table(double* tab, int L)
 {
-    extern __shared__ double Ahat[];  // [m_max]
-    __shared__ double red[kPrepThreads];
-    const int M = a.m_max, H = M - 1;
-    const long long L = 2LL * M - 1;
+    for (int r = threadIdx.x; r < L; r += blockDim.x) tab[r] = cospi(2.0 * (double)r / (double)L);
+}
+
+constexpr int kPrepTile = 64;
+
+// Discrete kernels, and hat C_w for one tile of frequencies per block.
+__global__ void __launch_bounds__(kPrepTile) prep_chat(const PrepArgs a)
+{
+    extern __shared__ double sh[];
+    const int M = a.m_max, L = 2 * M - 1;
+    double *tab = sh, *C = sh + L;  // [L], [M]
+    cos_table(tab, L);
     for (int m = threadIdx.x; m < M; m += blockDim.x) {
         const double k = discretize(a.Ks, m, a.dt, a.discrete);
+        C[m] = a.kT * (m == 0 ? 2.0 : 1.0) * k / a.dt;
+        if (blockIdx.x != 0) continue;
         a.Kd[m] = k;
         a.coef[m] = (float)k;
-        a.C[m] = a.kT * (m == 0 ? 2.0 : 1.0) * k / a.dt;
         for (int q = 0; q < a.Q; ++q) {
             const double g = discretize(a.g + (size_t)q * M, m, a.dt, a.discrete);
             a.coef[(size_t)(1 + q) * M + m] = (float)g;
@@ -71,15 +77,31 @@ __global__ void __launch_bounds__(kPrepThreads) prep(const PrepArgs a)
         }
     }
     __syncthreads();
+    const int w = blockIdx.x * kPrepTile + threadIdx.x;
+    if (w >= M) return;
+    double s = C[0];
+    int r = 0;  // w m mod L
+#pragma unroll 8
+    for (int m = 1; m < M; ++m) {
+        r += w;
+        if (r >= L) r -= L;
+        s += 2.0 * C[m] * tab[r];
+    }
+    a.Chat[w] = s;
+}
+
+// The positive-semi-definiteness check, square roots (into a.C) and the
+// integrator's factors.
+__global__ void __launch_bounds__(kPrepThreads) prep_root(const PrepArgs a)
+{
+    __shared__ double red[kPrepThreads];
+    const int M = a.m_max;
+    const long long L = 2LL * M - 1;
     double lmax = 0.0, lmin = 1e300;
     for (int w = threadIdx.x; w < M; w += blockDim.x) {
-        double s = a.C[0];
-        for (int m = 1; m < M; ++m) s += 2.0 * a.C[m] * cos_frac(w, m, L);
-        a.Chat[w] = s;
-        lmax = fmax(lmax, fabs(s));
-        lmin = fmin(lmin, s);
+        lmax = fmax(lmax, fabs(a.Chat[w]));
+        lmin = fmin(lmin, a.Chat[w]);
     }
-    __syncthreads();
     const double cmax = block_reduce(lmax, red, true);
     const double cmin = -block_reduce(-lmin, red, true);
     double neg = 0.0;
@@ -91,18 +113,10 @@ __global__ void __launch_bounds__(kPrepThreads) prep(const PrepArgs a)
             neg += -c * (w == 0 ? 1.0 : 2.0);
             c = 0.0;
         }
-        Ahat[w] = sqrt(c);
+        a.C[w] = sqrt(c);
     }
     const double negsum = block_reduce(neg, red, false);
     const double anybad = block_reduce((double)bad, red, true);
-    __syncthreads();
-    for (int s = threadIdx.x; s < 2 * M - 1; s += blockDim.x) {
-        const long long sh = s - H;
-        double v = Ahat[0];
-        for (int w = 1; w < M; ++w) v += 2.0 * Ahat[w] * cos_frac(w, sh, L);
-        a.A[s] = v / (double)L;
-    }
-    __syncthreads();
     if (threadIdx.x == 0) {
         const double c = a.dt * a.Kd[0] / (2.0 * a.mass);
         const double b = 1.0 / (1.0 + c);
@@ -112,8 +126,35 @@ __global__ void __launch_bounds__(kPrepThreads) prep(const PrepArgs a)
         a.scal[3] = negsum / (double)L;
         *a.status = anybad > 0.0 ? -3 : 0;
     }
-    // Filter taps in FP32: Acp[sigma] = A_{sigma - H}, zero past sigma = 2H.
-    for (int idx = threadIdx.x; idx < a.la; idx += blockDim.x) a.Acp[idx] = idx <= 2 * H ? (float)a.A[idx] : 0.0f;
+}
+
+// A_s and the FP32 taps Acp[sigma] = A_{sigma - H} (zero past sigma = 2H), one
+// tile per block.
+__global__ void __launch_bounds__(kPrepTile) prep_taps(const PrepArgs a)
+{
+    extern __shared__ double sh[];
+    const int M = a.m_max, H = M - 1, L = 2 * M - 1;
+    double *tab = sh, *root = sh + L;  // [L], [M]
+    cos_table(tab, L);
+    for (int w = threadIdx.x; w < M; w += blockDim.x) root[w] = a.C[w];
+    __syncthreads();
+    const int s = blockIdx.x * kPrepTile + threadIdx.x;
+    if (s >= L) {
+        if (s < a.la) a.Acp[s] = 0.0f;
+        return;
+    }
+    const int step = s - H < 0 ? s - H + L : s - H;
+    double v = root[0];
+    int r = 0;  // w (s - H) mod L
+#pragma unroll 8
+    for (int w = 1; w < M; ++w) {
+        r += step;
+        if (r >= L) r -= L;
+        v += 2.0 * root[w] * tab[r];
+    }
+    const double A = v / (double)L;
+    a.A[s] = A;
+    a.Acp[s] = (float)A;
 }
 
 constexpr int kGenThreads = 256;
@@ -304,9 +345,14 @@ int fir_taps_len(int H) { return (2 * H + 1 + 15) & ~15; }
 
 cudaError_t launch_prep(const PrepArgs& a, cudaStream_t st)
 {
-    const size_t smem = sizeof(double) * (size_t)a.m_max;
-    if (smem > 48 * 1024) cudaFuncSetAttribute(prep, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    prep<<<1, kPrepThreads, smem, st>>>(a);
+    const size_t smem = sizeof(double) * (size_t)(3 * a.m_max - 1);  // at most 96 KB
+    cudaError_t e = cudaFuncSetAttribute(prep_chat, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(prep_taps, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    prep_chat<<<(unsigned)((a.m_max + kPrepTile - 1) / kPrepTile), kPrepTile, smem, st>>>(a);
+    prep_root<<<1, kPrepThreads, 0, st>>>(a);
+    const int n = std::max(2 * a.m_max - 1, a.la);
+    prep_taps<<<(unsigned)((n + kPrepTile - 1) / kPrepTile), kPrepTile, smem, st>>>(a);
     return cudaGetLastError();
 }
 
