@@ -53,6 +53,9 @@ struct Ctrl {
     int pv_nact, pv_lag0, pv_buf;
     // the same bookkeeping for the distance-binned pair correlations
     int pc_pending, pc_buf, pc_pv_nact, pc_pv_lag0, pc_pv_buf, pad3_;
+    // grid barrier of the cooperative Clenshaw sweeps: blocks arrived and gone
+    // (both reset by the last block to go)
+    unsigned bar_arrived, bar_gone;
 };
 
 // Everything a step kernel needs, passed by value.

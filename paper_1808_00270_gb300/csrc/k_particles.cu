@@ -1436,46 +1436,6 @@ __device__ __forceinline__ void pn_stage_body(const StepParams& P, Ctrl* __restr
     if (S.last && !P.pn_iv && rowsum > P.pn_lambda) atomicOr(&ctrl->err, kErrPnBound);
 }
 
-template <int L>
-__global__ void __launch_bounds__(kThreads)
-    pn_stage_lanes(const StepParams P, Ctrl* __restrict__ ctrl, const float4* __restrict__ pos, const int* __restrict__ nbr,
-                   const int* __restrict__ nbr_cnt, const float* __restrict__ ftab, const float* __restrict__ fptab,
-                   const PnStage S)
-{
-    const Lanes<L> ln;
-    const int id = (int)((blockIdx.x * blockDim.x + threadIdx.x) / L);
-    if (id >= P.n) return;  // uniform over the lanes of a particle
-    const size_t np = P.n_pad;
-    const long long row = ctrl->step - ctrl->noise_n0;
-    if (row < 0 || row >= P.T) {
-        if (id == 0 && ln.lane == 0) atomicOr(&ctrl->err, kErrNoise);
-        return;
-    }
-    const size_t roff = (size_t)row * 3 * np;
-    const float* b1 = S.b1 + (S.b1_rows ? roff : 0);
-    const float* b2 = S.b2 ? S.b2 + (S.b2_rows ? roff : 0) : nullptr;
-    float* out = S.out + (S.out_rows ? roff : 0);
-    const float* z = S.z + roff;
-    const float bi[3] = {b1[id], b1[np + id], b1[2 * np + id]};
-    float zi[3] = {0.f, 0.f, 0.f}, b2i[3] = {0.f, 0.f, 0.f};
-    if (ln.lane == 0)
-#pragma unroll
-        for (int c = 0; c < 3; ++c) {
-            zi[c] = z[c * np + id];
-            if (b2) b2i[c] = b2[c * np + id];
-        }
-    float m[3] = {0.f, 0.f, 0.f}, rowsum = 0.f;
-    pn_sums<LdConst, L, 2>(P, ln, pos, nbr + id, nbr_cnt + id, id, pos[id], ftab, fptab, b1, bi, m, rowsum);
-    if (ln.lane != 0) return;
-    const float c = (S.last ? 1.0f : 2.0f) * P.pn_inv_lambda;
-#pragma unroll
-    for (int x = 0; x < 3; ++x) {
-        if (P.pn_cen != 0.f) m[x] = fmaf(-P.pn_cen, bi[x], m[x]);  // the interval [cen - rho, cen + rho]: (M - cen) b1
-        out[x * np + id] = fmaf(c, m[x], zi[x]) - b2i[x];
-    }
-    if (S.last && !P.pn_iv && rowsum > P.pn_lambda) atomicOr(&ctrl->err, kErrPnBound);
-}
-
 // Clenshaw stage k of a degree-K evaluation: b_K = Z_K (read in place), b_k
 // for K > k >= 1 in bvec[k % 3], the last stage writes F over the Z_0 row.
 __host__ __device__ __forceinline__ PnStage pn_stage_args(const StepParams& P, const float* frblock, const float* zblk,
@@ -1493,6 +1453,158 @@ __host__ __device__ __forceinline__ PnStage pn_stage_args(const StepParams& P, c
     if (k == 0) { S.out = const_cast<float*>(frblock); S.out_rows = 1; }
     else { S.out = bvec + (size_t)(k % 3) * vec; }
     return S;
+}
+
+// Waits until all blocks of a cooperative launch have arrived `round` times; a
+// wait of more than about a second latches kErrTimeout and goes on.
+__device__ __forceinline__ void grid_barrier(Ctrl* ctrl, unsigned round)
+{
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        __threadfence();
+        atomicAdd(&ctrl->bar_arrived, 1u);
+        const long long t0 = clock64();
+        for (;;) {
+            unsigned v;
+            asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(&ctrl->bar_arrived) : "memory");
+            if (v >= round * gridDim.x) break;
+            if (clock64() - t0 > 2000000000LL) {
+                atomicOr(&ctrl->err, kErrTimeout);
+                break;
+            }
+        }
+        __threadfence();
+    }
+    __syncthreads();
+}
+
+// All sweeps of a step in one cooperative launch (every block resident), one
+// thread per particle, for parallel factors only.  The sweeps share their
+// geometry: the first pass over the list keeps each pair inside the cutoff (id,
+// e, f) in shared memory, room for `room` pairs per thread in list order (pairs
+// past it are formed again from list entry `rest` on), so that a sweep is one
+// gather of the vector from L2 and a grid barrier.  A launch per sweep walked
+// list, positions and table again: 8.6 us each whatever the size.
+constexpr int kSweepThreads = 128;
+
+__global__ void __launch_bounds__(kSweepThreads)
+    pn_sweeps(const StepParams P, Ctrl* ctrl, const float4* __restrict__ pos, const int* __restrict__ nbr,
+              const int* __restrict__ nbr_cnt, const float* __restrict__ ftab, const float* frblock, const float* zblk,
+              float* bvec, int room)
+{
+    extern __shared__ float sm[];  // [5][room][kSweepThreads]: id, ex, ey, ez, f
+    const int id = (int)(blockIdx.x * kSweepThreads + threadIdx.x);
+    const size_t np = P.n_pad;
+    const long long row = ctrl->step - ctrl->noise_n0;
+    const bool ok = row >= 0 && row < P.T;  // uniform over the grid
+    if (!ok && id == 0) atomicOr(&ctrl->err, kErrNoise);
+    const bool own = ok && id < P.n;
+    const size_t roff = ok ? (size_t)row * 3 * np : 0;
+    const int K = P.pn_deg, pl = room * kSweepThreads;
+    float* my = sm + threadIdx.x;
+    float4 pi = make_float4(0.f, 0.f, 0.f, 0.f);
+    int cnt = 0, have = 0, rest = 0;
+    float rowsum = 0.f;
+    // calls f(entry, j, ex, ey, ez, f) for the pairs of the list entries from s0 on
+    auto walk = [&](int s0, auto&& f) {
+        for (int s = s0; s < cnt; s += 4) {
+            int j[4];
+            float4 pj[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) j[u] = s + u < cnt ? __ldg(nbr + (size_t)(s + u) * np + id) : id;
+#pragma unroll
+            for (int u = 0; u < 4; ++u) pj[u] = __ldg(pos + j[u]);
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                if (j[u] == id) continue;
+                const float dx = min_image_fma(pi.x, pj[u].x, P.box, P.inv_box);
+                const float dy = min_image_fma(pi.y, pj[u].y, P.box, P.inv_box);
+                const float dz = min_image_fma(pi.z, pj[u].z, P.box, P.inv_box);
+                const float r2 = dist2(dx, dy, dz);
+                if (!(r2 < P.rc2)) continue;
+                const float r = sqrtf(r2);
+                const float inv_r = 1.0f / r;
+                const float fr = table_at(ftab, P.nr, fmaxf(r, P.rc_min) * P.inv_dr);
+                f(s + u, j[u], dx * inv_r, dy * inv_r, dz * inv_r, fr);
+            }
+        }
+    };
+    if (own) {
+        pi = pos[id];
+        cnt = nbr_cnt[id];
+        rest = cnt;
+        walk(0, [&](int s, int j, float ex, float ey, float ez, float f) {
+            rowsum += fabsf(f);  // the block's spectral norm
+            if (have < room) {
+                float* q = my + have * kSweepThreads;
+                q[0] = __int_as_float(j);
+                q[pl] = ex;
+                q[2 * pl] = ey;
+                q[3 * pl] = ez;
+                q[4 * pl] = f;
+                ++have;
+            } else if (rest == cnt) {
+                rest = s;
+            }
+        });
+    }
+    for (int k = K - 1; k >= 0; --k) {
+        if (own) {
+            const PnStage S = pn_stage_args(P, frblock, zblk, bvec, K, k);
+            const float* b1 = S.b1 + (S.b1_rows ? roff : 0);
+            const float* b2 = S.b2 ? S.b2 + (S.b2_rows ? roff : 0) : nullptr;
+            float* out = S.out + (S.out_rows ? roff : 0);
+            const float* z = S.z + roff;
+            float zi[3], b2i[3] = {0.f, 0.f, 0.f}, bi[3], m[3] = {0.f, 0.f, 0.f};
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {
+                zi[c] = __ldcg(z + c * np + id);
+                if (b2) b2i[c] = __ldcg(b2 + c * np + id);
+                bi[c] = P.pn_cen != 0.f ? __ldcg(b1 + c * np + id) : 0.f;
+            }
+            auto add = [&](float bx, float by, float bz, float ex, float ey, float ez, float f) {
+                const float eb = f * dot3(ex, ey, ez, bx, by, bz);
+                m[0] = fmaf(eb, ex, m[0]);
+                m[1] = fmaf(eb, ey, m[1]);
+                m[2] = fmaf(eb, ez, m[2]);
+            };
+            for (int p = 0; p < have; p += 4) {
+                float bx[4], by[4], bz[4];
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    const int j = __float_as_int(my[min(p + u, have - 1) * kSweepThreads]);
+                    bx[u] = __ldcg(b1 + j);
+                    by[u] = __ldcg(b1 + np + j);
+                    bz[u] = __ldcg(b1 + 2 * np + j);
+                }
+#pragma unroll
+                for (int u = 0; u < 4; ++u)
+                    if (p + u < have) {
+                        const float* q = my + (p + u) * kSweepThreads;
+                        add(bx[u], by[u], bz[u], q[pl], q[2 * pl], q[3 * pl], q[4 * pl]);
+                    }
+            }
+            if (rest < cnt)
+                walk(rest, [&](int, int j, float ex, float ey, float ez, float f) {
+                    add(__ldcg(b1 + j), __ldcg(b1 + np + j), __ldcg(b1 + 2 * np + j), ex, ey, ez, f);
+                });
+            const float c = (S.last ? 1.0f : 2.0f) * P.pn_inv_lambda;
+#pragma unroll
+            for (int x = 0; x < 3; ++x) {
+                if (P.pn_cen != 0.f) m[x] = fmaf(-P.pn_cen, bi[x], m[x]);  // the interval [cen - rho, cen + rho]
+                out[x * np + id] = fmaf(c, m[x], zi[x]) - b2i[x];
+            }
+            if (S.last && !P.pn_iv && rowsum > P.pn_lambda) atomicOr(&ctrl->err, kErrPnBound);
+        }
+        if (k > 0) grid_barrier(ctrl, (unsigned)(K - k));
+    }
+    if (threadIdx.x == 0 && K > 1) {
+        __threadfence();
+        if (atomicAdd(&ctrl->bar_gone, 1u) == gridDim.x - 1) {
+            ctrl->bar_arrived = ctrl->bar_gone = 0u;
+            __threadfence();
+        }
+    }
 }
 
 __global__ void __launch_bounds__(kThreads)
@@ -1861,19 +1973,60 @@ cudaError_t launch_pcorr_flush(const StepParams& P, const ParticleBuffers& B, cu
     return cudaGetLastError();
 }
 
+namespace {
+
+// The sweeps as one cooperative launch when all of its blocks are resident at
+// once with room for a typical particle's pairs; *done = false: they are not.
+cudaError_t pn_sweeps_launch(const StepParams& P, const ParticleBuffers& B, const float* zblk, float* bvec,
+                             cudaStream_t st, bool* done)
+{
+    *done = false;
+    if (P.perp || P.Qs > 0 || P.pn_deg < 2) return cudaSuccess;
+    int dev = 0, sms = 0, coop = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev);
+    if (e != cudaSuccess) return e;
+    const int grid = (P.n + kSweepThreads - 1) / kSweepThreads, per_sm = (grid + sms - 1) / sms;
+    // pairs per thread: the list's capacity, or what the blocks of an SM share
+    // of 200 KB; lists hold about 1.7 times the pairs inside the cutoff
+    const int room = std::min(P.maxnb, (int)(200 * 1024 / ((size_t)per_sm * 20 * kSweepThreads)));
+    if (!coop || per_sm > 8 || room < 8) return cudaSuccess;
+    const size_t smem = (size_t)20 * kSweepThreads * room;
+    if ((e = cudaFuncSetAttribute(pn_sweeps, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess) return e;
+    int occ = 0;
+    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, pn_sweeps, kSweepThreads, smem)) != cudaSuccess) return e;
+    if (occ < per_sm) return cudaSuccess;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)grid);
+    cfg.blockDim = dim3(kSweepThreads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeCooperative;
+    at[0].val.cooperative = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    *done = true;
+    return cudaLaunchKernelEx(&cfg, pn_sweeps, P, B.ctrl, (const float4*)B.pos, (const int*)B.nbr, (const int*)B.nbr_cnt,
+                              B.ftab, (const float*)B.frblock, zblk, bvec, room);
+}
+
+}  // namespace
+
 cudaError_t launch_pair_noise(const StepParams& P, const ParticleBuffers& B, const float* zblk, float* bvec,
                               cudaStream_t st)
 {
     const int K = P.pn_deg;
     if (K <= 0) return cudaSuccess;
-    const int L = lanes_for(P.n);
-    auto kern = L == 8 ? pn_stage_lanes<8> : pn_stage;
-    const unsigned grid = (unsigned)(((long long)P.n * L + kThreads - 1) / kThreads);
+    bool done = false;
+    cudaError_t e = pn_sweeps_launch(P, B, zblk, bvec, st, &done);
+    if (e != cudaSuccess || done) return e;
+    const unsigned grid = (unsigned)((P.n + kThreads - 1) / kThreads);
     for (int k = K - 1; k >= 0; --k) {
-        kern<<<grid, kThreads, 0, st>>>(P, B.ctrl, B.pos, B.nbr, B.nbr_cnt, B.ftab, B.fptab,
-                                        pn_stage_args(P, B.frblock, zblk, bvec, K, k));
-        const cudaError_t e = cudaGetLastError();
-        if (e != cudaSuccess) return e;
+        pn_stage<<<grid, kThreads, 0, st>>>(P, B.ctrl, B.pos, B.nbr, B.nbr_cnt, B.ftab, B.fptab,
+                                            pn_stage_args(P, B.frblock, zblk, bvec, K, k));
+        if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
     return cudaSuccess;
 }

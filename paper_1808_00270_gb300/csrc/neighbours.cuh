@@ -259,73 +259,4 @@ __device__ __forceinline__ void cforce_sums(const StepParams& P, const Lanes<L>&
         });
 }
 
-// (M b)_i of the pair-correlated noise and its Gershgorin row sum (pn_apply).
-template <class LD, int L, int E>
-__device__ __forceinline__ void pn_sums(const StepParams& P, const Lanes<L>& ln, const float4* pos, const int* nb,
-                                        const int* pcnt, int i, const float4 pi, const float* __restrict__ ftab,
-                                        const float* __restrict__ fptab, const float* b, const float (&bi)[3],
-                                        float (&m)[3], float& rowsum)
-{
-    const size_t np = P.n_pad;
-    float4 pj[E];
-    float bx[E], by[E], bz[E], eb[E], ex[E], ey[E], ez[E], fp[E], rs[E], ei[E], fsp[E], rss[E];
-    walk_list<LD, L, E>(
-        ln, nb, pcnt, P.n_pad, P.maxnb, i,
-        [&](int u, int j) {
-            pj[u] = LD::f4(pos + j);
-            bx[u] = LD::f1(b + j);
-            by[u] = LD::f1(b + np + j);
-            bz[u] = LD::f1(b + 2 * np + j);
-        },
-        [&](int u, bool listed) {
-            const float dx = min_image_fma(pi.x, pj[u].x, P.box, P.inv_box);
-            const float dy = min_image_fma(pi.y, pj[u].y, P.box, P.inv_box);
-            const float dz = min_image_fma(pi.z, pj[u].z, P.box, P.inv_box);
-            const float r2 = dist2(dx, dy, dz);
-            eb[u] = ex[u] = ey[u] = ez[u] = fp[u] = rs[u] = ei[u] = fsp[u] = rss[u] = 0.f;
-            if (!listed || !(r2 < P.rc2)) return;
-            const float r = sqrtf(r2);
-            const float inv_r = 1.0f / r;
-            ex[u] = dx * inv_r;
-            ey[u] = dy * inv_r;
-            ez[u] = dz * inv_r;
-            const float xr = fmaxf(r, P.rc_min) * P.inv_dr;
-            const float f = table_at(ftab, P.nr, xr);
-            fp[u] = P.perp ? table_at(fptab, P.nr, xr) : 0.f;  // block f e e^T + fp (1 - e e^T)
-            eb[u] = (f - fp[u]) * nb_dot3(ex[u], ey[u], ez[u], bx[u], by[u], bz[u]);
-            rs[u] = fmaxf(fabsf(f), fabsf(fp[u]));  // the block's spectral norm
-            if (P.Qs > 0) {
-                const float fs = P.pn_cs * table_at(ftab + P.Q * P.nr, P.nr, xr);
-                fsp[u] = P.perp ? P.pn_cs * table_at(fptab + P.Q * P.nr, P.nr, xr) : 0.f;
-                ei[u] = (fs - fsp[u]) * nb_dot3(ex[u], ey[u], ez[u], bi[0], bi[1], bi[2]);
-                rss[u] = fmaxf(fabsf(fs), fabsf(fsp[u]));
-            }
-        },
-        [&](int l, int u) {
-            const float k = ln.get(eb[u], l), x = ln.get(ex[u], l), y = ln.get(ey[u], l), z = ln.get(ez[u], l);
-            if (P.perp) {
-                const float p = ln.get(fp[u], l);
-                m[0] = fmaf(p, ln.get(bx[u], l), m[0]);
-                m[1] = fmaf(p, ln.get(by[u], l), m[1]);
-                m[2] = fmaf(p, ln.get(bz[u], l), m[2]);
-            }
-            m[0] = fmaf(k, x, m[0]);
-            m[1] = fmaf(k, y, m[1]);
-            m[2] = fmaf(k, z, m[2]);
-            rowsum += ln.get(rs[u], l);
-            if (P.Qs > 0) {
-                const float q = ln.get(ei[u], l);
-                if (P.perp) {
-                    const float p = ln.get(fsp[u], l);
-#pragma unroll
-                    for (int c = 0; c < 3; ++c) m[c] = fmaf(p, bi[c], m[c]);
-                }
-                m[0] = fmaf(q, x, m[0]);
-                m[1] = fmaf(q, y, m[1]);
-                m[2] = fmaf(q, z, m[2]);
-                rowsum += ln.get(rss[u], l);
-            }
-        });
-}
-
 }  // namespace gld
