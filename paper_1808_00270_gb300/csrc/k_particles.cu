@@ -540,22 +540,29 @@ __global__ void __launch_bounds__(kThreads) nbr_build(const StepParams P, Ctrl* 
 // read four candidates at a time, collect ids in shared memory, and write each
 // to the place of its rank among the particle's ids.  Particles are taken in
 // cell order, so the groups of a warp read the same cells.
+// Alone up to 65536 particles (us per step 18.2 against 21.5 at 10007, 48.4
+// against 49.2 at 65536, but 99 against 93 at 131072: its shared memory takes L1
+// from the convolution that runs beside it).
+constexpr int kNbrLanesMaxN = 65536;
 constexpr int kNbrLanes = 4;
 constexpr int kNbrGroups = kThreads / kNbrLanes;  // particles per block
 
 __device__ __forceinline__ void nbr_lanes_body(const StepParams& P, Ctrl* ctrl, const float4* __restrict__ pos_sorted,
                                                const int* __restrict__ cell_start, int* __restrict__ nbr,
                                                int* __restrict__ nbr_cnt, int* __restrict__ perm,
-                                               const float4* __restrict__ disp, float4* __restrict__ disp_build, int blk)
+                                               const float4* __restrict__ disp, float4* __restrict__ disp_build, int blk,
+                                               int nblk)
 {
     if (ctrl->rebuild == 0) return;
     extern __shared__ int lists[];  // [kNbrGroups][maxnb]
     __shared__ int lcnt[kNbrGroups];
     constexpr int L = kNbrLanes, R = (9 + L - 1) / L;
-    const int lane = threadIdx.x & (L - 1), grp = threadIdx.x / L, k = blk * kNbrGroups + grp;
+    const int lane = threadIdx.x & (L - 1), grp = threadIdx.x / L;
     const unsigned gmask = ((1u << L) - 1u) << ((threadIdx.x & 31) & ~(L - 1));
     if (blk == 0 && threadIdx.x == 0) ctrl->rebuilds += 1;
-    if (k >= P.n) return;  // uniform over the lanes of a particle
+    // (a grid of at most six blocks per SM: a launch that finds nothing to do
+    // costs by its blocks)
+    for (int k = blk * kNbrGroups + grp; k < P.n; k += nblk * kNbrGroups) {  // uniform over the lanes of a particle
     const float4 pi = pos_sorted[k];
     const int id = __float_as_int(pi.w), nc = P.nc;
     int* list = lists + grp * P.maxnb;
@@ -627,13 +634,15 @@ __device__ __forceinline__ void nbr_lanes_body(const StepParams& P, Ctrl* ctrl, 
         perm[k] = id;
         disp_build[id] = disp[id];
     }
+    __syncwarp(gmask);  // the scratch is read before the next particle's
+    }
 }
 
 __global__ void __launch_bounds__(kThreads) nbr_lanes(const StepParams P, Ctrl* ctrl, const float4* __restrict__ pos_sorted,
               const int* __restrict__ cell_start, int* __restrict__ nbr, int* __restrict__ nbr_cnt,
               int* __restrict__ perm, const float4* __restrict__ disp, float4* __restrict__ disp_build)
 {
-    nbr_lanes_body(P, ctrl, pos_sorted, cell_start, nbr, nbr_cnt, perm, disp, disp_build, blockIdx.x);
+    nbr_lanes_body(P, ctrl, pos_sorted, cell_start, nbr, nbr_cnt, perm, disp, disp_build, blockIdx.x, gridDim.x);
 }
 
 // ---- velocity autocorrelation ------------------------------------------------
@@ -665,6 +674,31 @@ __device__ __forceinline__ void df_add(float& hi, float& lo, float bhi, float bl
     lo = e - (hi - s);
 }
 
+// The same for at most 32 blocks: one warp per origin (the other warps of the
+// form below would only add zeros), so a system of few blocks does not fold its
+// origins one after another (ten origins at 64 particles: 15 us per step).
+__device__ __forceinline__ void vacf_fold_warps(const StepParams& P, const float* __restrict__ base,
+                                                double* __restrict__ csum, long long* __restrict__ ccnt, int nact, int lag0,
+                                                int nblk, int first, int step)
+{
+    const int lane = threadIdx.x & 31, nw = blockDim.x >> 5;
+    for (int q = first * nw + (threadIdx.x >> 5); q < nact; q += step * nw) {
+        const int lg = lag0 + q * P.vacf_stride;  // < vacf_len for q < nact
+        const double s0 = csum[lg];
+        const long long c0 = ccnt[lg];
+        float hi = lane < nblk ? __ldcg(base + (size_t)q * nblk + lane) : 0.f, lo = 0.f;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            const float h2 = __shfl_xor_sync(0xffffffffu, hi, o), l2 = __shfl_xor_sync(0xffffffffu, lo, o);
+            df_add(hi, lo, h2, l2);
+        }
+        if (lane == 0) {
+            csum[lg] = s0 + ((double)hi + (double)lo);
+            ccnt[lg] = c0 + 1;
+        }
+    }
+}
+
 // Adds the block partials of origins q = first, first + step, ... (buffer
 // buf, nblk partials each) to C(lag0 + q*stride): double-float sums on the
 // FP32 pipes in a fixed order, one FP64 addition per origin.
@@ -675,6 +709,10 @@ __device__ __forceinline__ void vacf_fold(const StepParams& P, const float* __re
     __shared__ float sh[kThreads / 32][2];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const float* base = partial + (size_t)buf * P.n_os * nblk;
+    if (nblk <= 32) {  // blocks first, first + step, ... of the launch
+        vacf_fold_warps(P, base, csum, ccnt, nact, lag0, nblk, first, step);
+        return;
+    }
     // the first kThreads threads of the block (there may be more); its barriers
     // are joined by all
     const bool act = threadIdx.x < kThreads;
@@ -1048,6 +1086,7 @@ __global__ void __launch_bounds__(kThreads) vacf_flush(const StepParams P, Ctrl*
 {
     if (!ctrl->vacf_pending) return;
     vacf_fold(P, partial, csum, ccnt, ctrl->vacf_buf, ctrl->vacf_nact, ctrl->vacf_lag0, nblk, 0, 1);
+    __syncthreads();
     if (threadIdx.x == 0) ctrl->vacf_pending = 0;
 }
 
@@ -1323,7 +1362,7 @@ __global__ void __launch_bounds__(kThreads) b_nbr_lanes(const SysDesc* __restric
     const Tile t = tiles[blockIdx.x];
     const SysDesc& d = D[t.m];
     const ParticleBuffers& B = d.B;
-    nbr_lanes_body(d.P, B.ctrl, B.pos_sorted, B.cell_start, B.nbr, B.nbr_cnt, B.perm, B.disp, B.disp_build, t.b);
+    nbr_lanes_body(d.P, B.ctrl, B.pos_sorted, B.cell_start, B.nbr, B.nbr_cnt, B.perm, B.disp, B.disp_build, t.b, t.nb);
 }
 
 __global__ void __launch_bounds__(kThreads) b_cforce(const SysDesc* __restrict__ D, const Tile* __restrict__ tiles)
@@ -1914,8 +1953,8 @@ cudaError_t launch_rebuild(const StepParams& P, const ParticleBuffers& B, cudaSt
     if (rebuild_in_cluster(P)) return launch_rebuild_cluster(P, B, st);
     cudaError_t e = launch_cell_build(P, B, B.pos_next, &B.ctrl->rebuild, st);
     if (e != cudaSuccess) return e;
-    if (P.maxnb <= kNbrSortCap)
-        return launch_nbr_lanes(nbr_lanes, (P.n + kNbrGroups - 1) / kNbrGroups, P.maxnb, st, P, B.ctrl, B.pos_sorted,
+    if (P.maxnb <= kNbrSortCap && P.n <= kNbrLanesMaxN)
+        return launch_nbr_lanes(nbr_lanes, std::min((P.n + kNbrGroups - 1) / kNbrGroups, 6 * 152), P.maxnb, st, P, B.ctrl, B.pos_sorted,
                                 B.cell_start, B.nbr, B.nbr_cnt, B.perm, B.disp, B.disp_build);
     nbr_build<<<(P.n + kThreads - 1) / kThreads, kThreads, 0, st>>>(P, B.ctrl, B.pos_sorted, B.cell_start, B.nbr,
                                                                      B.nbr_cnt, B.perm, B.disp, B.disp_build);

@@ -187,10 +187,11 @@ cudaError_t launch_batch_noise(const BatchPlan& bp, cudaStream_t st);     // k_n
 // number of the first step in its block of the convolution, > 0: that block's
 // parts are formed; G and len as conv_block_shape).
 // Sizes (us per step, cluster against the graph of the step kernels): a whole
-// noise block 15.1 / 17.9 at 1000 particles, 17.9 / 16.6 at 2048, 21.4 / 17.1 at
-// 4096; launched for single steps 20.2 / 30.9, 23.7 / 31.0, 27.4 / 30.4.
+// noise block 7.2 / 10.7 at 64 particles, 10.5 / 10.4 at 200, 11.8 / 10.7 at 512;
+// launched for single steps 20.2 / 30.9 at 1000, 23.7 / 31.0 at 2048, 27.4 / 30.4
+// at 4096.
 constexpr int kClusterMaxN = 4096;
-constexpr int kClusterBlockMaxN = 1536;
+constexpr int kClusterBlockMaxN = 192;
 bool cluster_ok(const StepParams& P, int kahan);
 cudaError_t launch_steps_cluster(const SysDesc& d, int nsteps, int rel0, int G, int len, cudaStream_t st);
 
