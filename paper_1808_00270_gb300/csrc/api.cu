@@ -2630,6 +2630,28 @@ gld_status batch_autotune(gld_batch* b)
     return batch_plan(b, best);
 }
 
+// A block's launches as a graph.  Capturing some 500 launches costs more host
+// time than launching them twice, so a composition that lasts for fewer than
+// three blocks (as in serving, where members come and go) is launched eagerly.
+void batch_capture(gld_batch* b)
+{
+    if (b->gexec || b->graph_failed || b->same_blocks < 2) return;
+    cudaGraph_t g = nullptr;
+    bool ok = cudaStreamBeginCapture(b->cap, cudaStreamCaptureModeThreadLocal) == cudaSuccess;
+    if (ok) {
+        const cudaError_t e = batch_launch_block(b, b->cap);
+        const cudaError_t e2 = cudaStreamEndCapture(b->cap, &g);
+        ok = e == cudaSuccess && e2 == cudaSuccess && g;
+    }
+    if (ok) ok = cudaGraphInstantiate(&b->gexec, g, 0) == cudaSuccess;
+    if (g) cudaGraphDestroy(g);
+    if (!ok) {
+        cudaGetLastError();
+        b->gexec = nullptr;  // eager launches
+        b->graph_failed = true;
+    }
+}
+
 gld_status batch_prepare(gld_batch* b)
 {
     if (!b->dirty) return GLD_OK;
@@ -2642,19 +2664,8 @@ gld_status batch_prepare(gld_batch* b)
         GLD_TRY(batch_autotune(b));
         b->tuned_cols = cols;
     }
-    cudaGraph_t g = nullptr;
-    bool ok = cudaStreamBeginCapture(b->cap, cudaStreamCaptureModeThreadLocal) == cudaSuccess;
-    if (ok) {
-        const cudaError_t e = batch_launch_block(b, b->cap);
-        const cudaError_t e2 = cudaStreamEndCapture(b->cap, &g);
-        ok = e == cudaSuccess && e2 == cudaSuccess && g;
-    }
-    if (ok) ok = cudaGraphInstantiate(&b->gexec, g, 0) == cudaSuccess;
-    if (g) cudaGraphDestroy(g);
-    if (!ok) {
-        cudaGetLastError();
-        b->gexec = nullptr;  // eager launches below
-    }
+    b->same_blocks = 0;
+    b->graph_failed = false;
     b->dirty = false;
     return GLD_OK;
 }
@@ -2733,6 +2744,8 @@ gld_status gld_batch_step(gld_batch* b, int64_t nsteps)
             b->dirty = true;
     GLD_TRY(batch_prepare(b));
     for (int64_t k = 0; k < nsteps; k += kMaxNoiseBlock) {
+        batch_capture(b);
+        ++b->same_blocks;
         const cudaError_t e = b->gexec ? cudaGraphLaunch(b->gexec, b->st) : batch_launch_block(b, b->st);
         if (e != cudaSuccess) return bfail(b, GLD_E_CUDA, std::string("gld_batch_step: ") + cudaGetErrorString(e));
         for (gld_ctx* c : b->members) {

@@ -110,6 +110,8 @@ struct gld_batch {
     int schedule = -1;  // chosen convolution schedule (autotuned), -1: not yet
     double schedule_ms[4] = {0, 0, 0, 0};
     cudaGraphExec_t gexec = nullptr;
+    int same_blocks = 0;        // blocks stepped with this composition
+    bool graph_failed = false;
     std::vector<SysDesc> snap;  // member descriptors the plan was built from
     std::string msg;
 };
