@@ -12,6 +12,7 @@
 #include <cmath>
 #include <cstdio>
 #include <cstring>
+#include <mutex>
 #include <numeric>
 #include <string>
 #include <vector>
@@ -123,14 +124,103 @@ gld_status upload_vec(gld_ctx* c, float4* dst, const double* src, bool wrap)
     return GLD_OK;
 }
 
-gld_status download_vec(gld_ctx* c, const float4* src, double* dst)
+// Page-locked staging of results read back, kept for the next read of any
+// context (allocating it costs more than most reads): at most kPinnedKept bytes
+// are kept, the rest is freed when it is given back.
+struct Pinned {
+    char* p = nullptr;
+    size_t cap = 0;
+};
+constexpr size_t kPinnedKept = (size_t)64 << 20;
+std::mutex g_pinned_mu;
+std::vector<Pinned> g_pinned;
+
+Pinned take_pinned(size_t bytes)
 {
-    const int n = c->P.n;
-    std::vector<float4> h((size_t)n);
-    GLD_CUDA(c, cudaMemcpyAsync(h.data(), src, sizeof(float4) * n, cudaMemcpyDeviceToHost, c->st));
-    GLD_CUDA(c, cudaStreamSynchronize(c->st));
-    ctx_to_caller(c, h.data(), dst);
-    return GLD_OK;
+    Pinned b;
+    {
+        std::lock_guard<std::mutex> lock(g_pinned_mu);
+        size_t best = g_pinned.size();
+        for (size_t k = 0; k < g_pinned.size(); ++k)
+            if (g_pinned[k].cap >= bytes && (best == g_pinned.size() || g_pinned[k].cap < g_pinned[best].cap)) best = k;
+        if (best < g_pinned.size()) {
+            b = g_pinned[best];
+            g_pinned.erase(g_pinned.begin() + (long)best);
+            return b;
+        }
+    }
+    b.cap = std::max(bytes, (size_t)1 << 16);
+    if (cudaHostAlloc((void**)&b.p, b.cap, cudaHostAllocPortable) != cudaSuccess) {
+        cudaGetLastError();
+        b = Pinned{};
+    }
+    return b;
+}
+
+void give_pinned(Pinned b)
+{
+    if (!b.p) return;
+    {
+        std::lock_guard<std::mutex> lock(g_pinned_mu);
+        size_t kept = b.cap;
+        for (const Pinned& x : g_pinned) kept += x.cap;
+        if (kept <= kPinnedKept) {
+            g_pinned.push_back(b);
+            return;
+        }
+    }
+    cudaFreeHost(b.p);
+}
+
+// Copies queued behind the context's work, then one wait for all of them and
+// for the device's error word.
+class Readback {
+public:
+    Readback(gld_ctx* ctx, size_t bytes) : c(ctx), pin(take_pinned(bytes + 256))
+    {
+        if (!pin.p) plain.resize(bytes + 256);
+    }
+    ~Readback() { give_pinned(pin); }
+    Readback(const Readback&) = delete;
+    Readback& operator=(const Readback&) = delete;
+    // Queues a copy; *host holds the data after wait().  Room for each copy is
+    // its bytes rounded up to 16.
+    gld_status add(const void* dev, size_t bytes, const void** host)
+    {
+        char* h = base() + off;
+        off += (bytes + 15) & ~(size_t)15;
+        *host = h;
+        GLD_CUDA(c, cudaMemcpyAsync(h, dev, bytes, cudaMemcpyDeviceToHost, c->st));
+        return GLD_OK;
+    }
+    // xyz of a particle array in the caller's order (through the sorted
+    // positions' buffer, which only a list build uses).
+    gld_status add_vec(const float4* src, const void** host)
+    {
+        float* tmp = (float*)c->B.pos_sorted;
+        GLD_CUDA(c, launch_export_vec(c->P.n, src, c->d_int2ext, tmp, c->st));
+        return add(tmp, 12 * (size_t)c->P.n, host);
+    }
+    gld_status wait()
+    {
+        const void* err = nullptr;
+        GLD_TRY(add(&c->B.ctrl->err, sizeof(unsigned), &err));
+        GLD_CUDA(c, cudaStreamSynchronize(c->st));
+        return ctx_check_err(c, *(const unsigned*)err);
+    }
+
+private:
+    char* base() { return pin.p ? pin.p : plain.data(); }
+    gld_ctx* c;
+    Pinned pin;
+    std::vector<char> plain;
+    size_t off = 0;
+};
+
+void to_doubles(const void* src, size_t n, double* dst)
+{
+    const float* f = (const float*)src;
+    for (size_t k = 0; k < n; ++k) dst[k] = f[k];
 }
 
 // [rows][3][n_pad] float planes <-> [rows][n][3] doubles.
@@ -1258,15 +1348,20 @@ gld_status gld_vacf(gld_ctx* c, double* out, int64_t* n_origins)
 {
     if (!c) return GLD_E_INVAL;
     if (c->latched == GLD_OK) GLD_CUDA(c, launch_vacf_flush(c->P, c->B, c->st));
-    GLD_TRY(sync_and_check(c));
     const int L = c->P.vacf_len;
+    Readback rb(c, 16 * (size_t)std::max(L, 0) + 64);
+    const void *hs = nullptr, *hk = nullptr, *hn = nullptr;
+    if (L > 0) {
+        GLD_TRY(rb.add(c->B.csum, sizeof(double) * L, &hs));
+        GLD_TRY(rb.add(c->B.ccnt, sizeof(long long) * L, &hk));
+        GLD_TRY(rb.add(c->B.norig, sizeof(long long), &hn));
+    }
+    GLD_TRY(rb.wait());
     long long no = 0;
     if (L > 0) {
-        std::vector<double> s(L);
-        std::vector<long long> k(L);
-        GLD_CUDA(c, cudaMemcpy(s.data(), c->B.csum, sizeof(double) * L, cudaMemcpyDeviceToHost));
-        GLD_CUDA(c, cudaMemcpy(k.data(), c->B.ccnt, sizeof(long long) * L, cudaMemcpyDeviceToHost));
-        GLD_CUDA(c, cudaMemcpy(&no, c->B.norig, sizeof(long long), cudaMemcpyDeviceToHost));
+        const double* s = (const double*)hs;
+        const long long* k = (const long long*)hk;
+        no = *(const long long*)hn;
         if (out)
             for (int l = 0; l < L; ++l) out[l] = k[l] > 0 ? s[l] / (3.0 * c->P.n * (double)k[l]) : 0.0;
     }
@@ -1277,24 +1372,38 @@ gld_status gld_vacf(gld_ctx* c, double* out, int64_t* n_origins)
 gld_status gld_get_state(gld_ctx* c, double* pos, double* vel)
 {
     if (!c) return GLD_E_INVAL;
-    GLD_TRY(sync_and_check(c));
-    if (pos) GLD_TRY(download_vec(c, c->B.pos, pos));
-    if (vel) GLD_TRY(download_vec(c, c->B.vel, vel));
+    const size_t n3 = 3 * (size_t)c->P.n;
+    Readback rb(c, 2 * (4 * n3 + 16));
+    const void *hp = nullptr, *hv = nullptr;
+    if (pos) GLD_TRY(rb.add_vec(c->B.pos, &hp));
+    if (vel) GLD_TRY(rb.add_vec(c->B.vel, &hv));
+    GLD_TRY(rb.wait());
+    if (pos) to_doubles(hp, n3, pos);
+    if (vel) to_doubles(hv, n3, vel);
     return GLD_OK;
 }
 
 gld_status gld_get_array(gld_ctx* c, int32_t which, double* out)
 {
     if (!c || !out) return GLD_E_INVAL;
-    GLD_TRY(sync_and_check(c));
     const StepParams& P = c->P;
     const size_t np = P.n_pad;
+    const float4* vec = which == GLD_ARR_POS    ? c->B.pos
+                        : which == GLD_ARR_VEL  ? c->B.vel
+                        : which == GLD_ARR_FC   ? c->B.fc
+                        : which == GLD_ARR_FD   ? c->B.fd
+                        : which == GLD_ARR_DISP ? c->B.disp
+                                                : nullptr;
+    if (vec) {
+        Readback rb(c, 12 * (size_t)P.n + 16);
+        const void* h = nullptr;
+        GLD_TRY(rb.add_vec(vec, &h));
+        GLD_TRY(rb.wait());
+        to_doubles(h, 3 * (size_t)P.n, out);
+        return GLD_OK;
+    }
+    GLD_TRY(sync_and_check(c));
     switch (which) {
-    case GLD_ARR_POS: return download_vec(c, c->B.pos, out);
-    case GLD_ARR_VEL: return download_vec(c, c->B.vel, out);
-    case GLD_ARR_FC: return download_vec(c, c->B.fc, out);
-    case GLD_ARR_FD: return download_vec(c, c->B.fd, out);
-    case GLD_ARR_DISP: return download_vec(c, c->B.disp, out);
     case GLD_ARR_FR:
         if (c->last_fr_row < 0) return fail(c, GLD_E_STATE, "gld_get_array: no step has run");
         return download_planes(c, c->B.frblock + (size_t)c->last_fr_row * 3 * np, 1, out);

@@ -1293,6 +1293,19 @@ __global__ void pair_list(const StepParams P, const float4* __restrict__ pos_sor
     });
 }
 
+// xyz of a particle array in the caller's order, [n][3].
+__global__ void __launch_bounds__(kThreads) export_vec(int n, const float4* __restrict__ src, const int* __restrict__ int2ext,
+                                                       float* __restrict__ out)
+{
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n) return;
+    const float4 v = src[i];
+    float* o = out + 3 * (size_t)int2ext[i];
+    o[0] = v.x;
+    o[1] = v.y;
+    o[2] = v.z;
+}
+
 // Sets the graph condition that guards the rebuild kernels.
 __global__ void rebuild_decide(cudaGraphConditionalHandle h, const Ctrl* __restrict__ ctrl)
 {
@@ -1881,6 +1894,12 @@ cudaError_t launch_batch_particles(const BatchPlan& bp, cudaStream_t st)
 cudaError_t launch_rebuild_decide(cudaGraphConditionalHandle h, const Ctrl* ctrl, cudaStream_t st)
 {
     rebuild_decide<<<1, 1, 0, st>>>(h, ctrl);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_export_vec(int n, const float4* src, const int* int2ext, float* out, cudaStream_t st)
+{
+    export_vec<<<(unsigned)((n + kThreads - 1) / kThreads), kThreads, 0, st>>>(n, src, int2ext, out);
     return cudaGetLastError();
 }
 

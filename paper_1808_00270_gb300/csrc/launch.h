@@ -66,6 +66,8 @@ struct ParticleBuffers {
 };
 
 cudaError_t launch_pair_force_integrate(const StepParams& P, const ParticleBuffers& B, cudaStream_t st);
+// xyz of the array src, [n][3] in the caller's order.
+cudaError_t launch_export_vec(int n, const float4* src, const int* int2ext, float* out, cudaStream_t st);
 // One thread idles for ns nanoseconds (at most 10 ms) on the device.
 cudaError_t launch_delay(unsigned long long ns, cudaStream_t st);
 // Cell list of the positions `src`; skipped on the device when gate != nullptr
