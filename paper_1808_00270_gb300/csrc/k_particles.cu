@@ -1912,11 +1912,12 @@ cudaError_t launch_delay(unsigned long long ns, cudaStream_t st)
 namespace {
 
 // Lanes per particle of the neighbour kernels of a system alone: eight while
-// they are at most about 1000 threads per SM.  Pair kernel, us (events) with
-// eight / one: 8.4 / 12.2 at 4096 particles, 9.7 / 12.2 at 10007, general form
-// 20.5 / 32.8 at 20000; with four / one 12.6 / 10.8 at 32768, with two / one
-// 19.7 / 16.7 at 65536: the shuffled additions cost more than they hide.
-int lanes_for(int n) { return n <= kLanesMaxN ? 8 : 1; }
+// that is at most 1024 threads per SM, then four.  Pair kernel, us (events)
+// with eight / one: 8.4 / 12.2 at 4096 particles, 9.7 / 12.2 at 10007; general
+// form with eight / four / one 24.4 / 20.5 / 32.8 at 20000.  Above kLanesMaxN
+// one: with four / one 12.6 / 10.8 at 32768, with two / one 19.7 / 16.7 at
+// 65536, the shuffled additions cost more than they hide.
+int lanes_for(int n) { return n <= 1024 * 152 / 8 ? 8 : n <= kLanesMaxN ? 4 : 1; }
 
 template <bool FAST, int L>
 cudaError_t pair_lanes_launch(const StepParams& P, const ParticleBuffers& B, cudaStream_t st)
@@ -1945,6 +1946,7 @@ cudaError_t launch_pair_force_integrate(const StepParams& P, const ParticleBuffe
     const unsigned grid = (unsigned)((P.n + kPairThreads - 1) / kPairThreads);
     const bool fast = P.Q == 1 && P.Qs == 0 && !P.perp;
     if (lanes_for(P.n) == 8) return fast ? pair_lanes_launch<true, 8>(P, B, st) : pair_lanes_launch<false, 8>(P, B, st);
+    if (lanes_for(P.n) == 4) return fast ? pair_lanes_launch<true, 4>(P, B, st) : pair_lanes_launch<false, 4>(P, B, st);
     auto k = fast ? pair_force_integrate<true> : pair_force_integrate<false>;
     const unsigned pgrid = fast ? (unsigned)(((long long)P.n * kPairLanes + kPairThreads - 1) / kPairThreads) : grid;
     k<<<pgrid, kPairThreads, 0, st>>>(P, B.ctrl, B.pos, B.perm, B.nbr, B.nbr_cnt, B.vel, B.fc,
