@@ -356,13 +356,19 @@ cudaError_t part_launch(const Shape& sh, const void* ring, int n_pad, int M, con
 {
     const int H = M - 1;
     const size_t smem = sizeof(float) * (size_t)H * NACC;
-    if (sh.kind == 0) {  // one range, one wave of 16-byte columns
+    const long long bytes = 3LL * n_pad * (BF16 ? 2 : 4);
+    // One range, one wave of 16-byte columns.  Compensated sums have one range
+    // at every size and are chains of four dependent operations a term: below
+    // 384 threads per SM narrower columns hide them better (us per step, 16-byte
+    // / narrower: 20.3 / 12.3 at 4096 particles in BF16, 29.9 / 20.0 at 10007 and
+    // 48.2 / 42.5 at 50000 in FP32, 68.3 / 58.6 at 100003 in BF16; above it
+    // 68.8 / 75.4 at 100003 in FP32).
+    if (sh.kind == 0 && !(KAHAN && bytes / 16 < 384LL * 152)) {
         auto k = hist_conv_col<NACC, KAHAN, BF16, true>;
         if (smem > 48 * 1024) cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         k<<<sh.grid, sh.block, smem, st>>>((const typename Col<BF16>::V*)ring, 3LL * n_pad / Col<BF16>::W, H, coef, M,
                                            nstep, step, out, bp);
     } else {
-        const long long bytes = 3LL * n_pad * (BF16 ? 2 : 4);
         const int vb = bytes / 16 >= 512LL * 152 ? 16 : bytes / 8 >= 512LL * 152 ? 8 : 4;
         auto k = vb == 16 ? conv_tail<NACC, KAHAN, BF16, 16>
                           : vb == 8 ? conv_tail<NACC, KAHAN, BF16, 8> : conv_tail<NACC, KAHAN, BF16, 4>;

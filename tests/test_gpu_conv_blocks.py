@@ -40,10 +40,12 @@ def _whole_sums(g, w, hist, coef, step, bf16, kahan):
 
 # shortest ring with blocks (32 slots), a split into four ranges, odd sizes, one
 # range (columns that fill the chip), three accumulators, BF16, compensated sums
+# (columns of 4, 8 and 16 bytes)
 @pytest.mark.parametrize("n,m_max,terms,hist,kahan", [
     (64, 33, "pair", "f32", False), (77, 34, "pair", "f32", False), (1001, 100, "pair", "f32", False),
     (1001, 131, "general", "f32", False), (1001, 100, "pair", "bf16", False), (1001, 100, "pair", "f32", True),
-    (333, 70, "general", "bf16", True), (90001, 66, "pair", "f32", False), (90001, 66, "pair", "bf16", True)])
+    (333, 70, "general", "bf16", True), (90001, 66, "pair", "f32", False), (90001, 66, "pair", "bf16", True),
+    (120001, 40, "pair", "bf16", True), (160001, 40, "pair", "bf16", True)])
 def test_resumed_sums_are_the_whole_sums(n, m_max, terms, hist, kahan):
     from paper_1808_00270_gb300 import ARR_CONV, ARR_HIST, inputs
     short = m_max < 58
