@@ -1,13 +1,16 @@
 // api.cu -- the C ABI of include/gld.h: context life cycle, device memory,
 // step orchestration and CUDA-graph replay.
 //
-// One step n -> n+1 is five kernels on the context's stream:
-//   hist_conv -> pair_force_integrate -> cell build (3 small kernels)
-//   -> cforce (F^C_{n+1}, V_{n+1}, n += 1, and the VACF terms when enabled)
+// One step n -> n+1 on the context's stream:
+//   memory sums (every 8 or 16 steps also their parts) -> pair force and
+//   positions -> list build when requested -> cforce (F^C_{n+1}, V_{n+1},
+//   n += 1, and the VACF terms when enabled)
 // and every T steps one noise block (wgen + fir) produces F^R for the next T
 // steps.  The step counter lives on the device, so a graph holding one noise
 // block and T steps is captured once and replayed for as long as the kernels
-// stay the same.
+// stay the same; a program that steps in other numbers replays a segment of
+// steps captured once it has taken a block's worth of them.  Small systems run
+// the steps of a block inside one cluster kernel (k_cluster.cu).
 #include <algorithm>
 #include <cmath>
 #include <cstdio>
@@ -180,7 +183,12 @@ public:
     {
         if (!pin.p) plain.resize(bytes + 256);
     }
-    ~Readback() { give_pinned(pin); }
+    ~Readback()
+    {
+        // an early return: no copy may land in staging that the next read takes
+        if (queued) cudaStreamSynchronize(c->st);
+        give_pinned(pin);
+    }
     Readback(const Readback&) = delete;
     Readback& operator=(const Readback&) = delete;
     // Queues a copy; *host holds the data after wait().  Room for each copy is
@@ -190,6 +198,7 @@ public:
         char* h = base() + off;
         off += (bytes + 15) & ~(size_t)15;
         *host = h;
+        queued = true;
         GLD_CUDA(c, cudaMemcpyAsync(h, dev, bytes, cudaMemcpyDeviceToHost, c->st));
         return GLD_OK;
     }
@@ -206,6 +215,7 @@ public:
         const void* err = nullptr;
         GLD_TRY(add(&c->B.ctrl->err, sizeof(unsigned), &err));
         GLD_CUDA(c, cudaStreamSynchronize(c->st));
+        queued = false;
         return ctx_check_err(c, *(const unsigned*)err);
     }
 
@@ -215,6 +225,7 @@ private:
     Pinned pin;
     std::vector<char> plain;
     size_t off = 0;
+    bool queued = false;
 };
 
 void to_doubles(const void* src, size_t n, double* dst)
