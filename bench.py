@@ -173,6 +173,29 @@ class ClockSampler:
         return {"sm_mhz": statistics.median(sm), "sm_max_mhz": mx, "reasons": sorted(reasons), "samples": len(sm)}
 
 
+def conv_bytes(n: int, m_max: int, elem: int, nacc: int, kahan: bool, first: int, steps: int) -> float:
+    """Bytes per step that the memory sums of steps first .. first + steps - 1
+    need in blocks of steps: the parts of a block read each range of ring rows up
+    to its first rewritten row, once for the block's 8 or 16 steps; a step reads
+    the rest of the ranges, reads its parts and writes its sums.  (One range from
+    about 80000 particles on, two from 40000, else four.)"""
+    H, ranges = m_max - 1, 1 if kahan or n > 80000 else 2 if n > 40000 else 4
+    length = 8 if kahan or ranges > 1 else 16
+    rows = parts = 0.0
+    for k in range(first, first + steps):
+        h0 = (first + (k - first) // length * length) % H
+        for r in range(ranges):
+            lo, hi = r * H // ranges, (r + 1) * H // ranges
+            if lo < h0 + length - H or h0 <= lo < h0 + length:
+                e = lo  # the range begins with a rewritten row
+            else:
+                e = h0 if lo <= h0 < hi else hi
+            rows += (e - lo) / length + (hi - e)
+            parts += 2 if e > lo else 0  # written and read
+    sums = 4 * 3 * nacc * (1 + parts / steps * (2 if kahan else 1))
+    return n * (elem * 3 * rows / steps + sums)
+
+
 def kernel_source_hash() -> str:
     src = os.path.join(ROOT, "paper_1808_00270_gb300", "csrc", "k_history.cu")
     return hashlib.sha256(open(src, "rb").read()).hexdigest()[:16]
@@ -281,6 +304,7 @@ def batch_leg(args, rank: int, world: int, local: int, quiet: bool = False):
     seq = world * n_tot * K / (ms_seq / 1e3)
     elem = 2 if args.hist == "bf16" else 4
     alg = sum((elem * 3 * (w.m_max - 1) + 4 * 3 * 2) * w.n for w in ws)
+    # (timed before the first step, where a step still streams its whole ring)
     conv_ms = info["schedule_ms"][info["schedule"]]
     peak, peak_kind = peaks()
     hist_bytes = sum(elem * 3 * (w.m_max - 1) * ((w.n + 31) // 32 * 32) for w in ws)
@@ -304,7 +328,7 @@ def batch_leg(args, rank: int, world: int, local: int, quiet: bool = False):
                         "achieved": alg / (conv_ms / 1e3) / 1e9, "peak": peak, "unit": "GB/s",
                         "frac": alg / (conv_ms / 1e3) / 1e9 / peak, "peak_source": f"{peak_kind} hbm_gbs",
                         "traffic": None, "algorithmic_bytes_per_launch": alg, "avg_launch_ms": conv_ms},
-           "clocks": clk, "gpu_launches": (K // T) * (2 + T * 8)}
+           "clocks": clk, "gpu_launches": (K // T) * (2 + T * 7 + T // (8 if args.kahan else 16))}
     if rank == 0 and not quiet:
         print(json.dumps(out))
     for g in systems:
@@ -407,7 +431,7 @@ def serve_leg(args, rank: int, world: int, local: int, quiet: bool = False):
            "served": served, "sequential": seq,
            "throughput_vs_sequential": served["throughput"] / seq["throughput"] if seq else None,
            "max_sustainable_rate_per_s": served["throughput"] / mean_work,
-           "clocks": clk, "gpu_launches": st["blocks"] * (2 + 64 * 8)}
+           "clocks": clk, "gpu_launches": st["blocks"] * (2 + 64 * 8 + 4)}
     if rank == 0 and not quiet:
         print(json.dumps(out))
     return out
@@ -527,13 +551,13 @@ def main():
         sim.set_pair_noise_lanczos(0.0)
         cfg["pair_noise"]["krylov_dimension"] = kdim
         cfg["pair_noise"]["kernel_profile"] = "without the pair noise"
+    prof_first = sim.step_index
     prof = sim.profile_steps(args.profile_steps)
     h_ms, h_n = prof["hist_conv"]
     nacc = 2
-    alg_bytes = (4 * 3 * (w.m_max - 1) + 4 * 3 * nacc) * w.n * (0.5 if args.hist == "bf16" else 1.0)
-    if args.hist == "bf16":
-        alg_bytes = (2 * 3 * (w.m_max - 1) + 4 * 3 * nacc) * w.n
-    kname, traffic = "hist_conv", measured_traffic(args.workload)
+    alg_bytes = conv_bytes(w.n, w.m_max, 2 if args.hist == "bf16" else 4, nacc, bool(args.kahan), prof_first,
+                           args.profile_steps)
+    kname, traffic = "history convolution (a step's sums and its share of the block's parts)", measured_traffic(args.workload)
     if args.modes:  # per column: Y' of every mode read and written, two ring values, the projections
         nm = len(inputs.memory_modes(w)[0])
         elem = 2 if args.hist == "bf16" else 4
@@ -555,15 +579,21 @@ def main():
                  // vacf["vacf_stride"]})
     T_blocks = (K + T - 1) // T
     # per step: convolution, pair kernel, F^C with the VACF terms, and the
-    # rebuild decision (conditional form) or the four gated rebuild kernels
+    # rebuild decision (conditional form) or the gated rebuild kernels (one up to
+    # 8192 particles, else four); per 8 or 16 steps the parts of the convolution
+    parts = 0 if args.modes else K // (16 if w.n > 80000 and not args.kahan else 8)
+    plain = not args.modes and args.pcorr <= 0 and args.pair_noise <= 0
     if d0["graph_mode"] == 2:  # rebuild kernels only on the steps that rebuild
-        launches = K * 4 + 4 * (d1["rebuilds"] - d0["rebuilds"]) + 2 * T_blocks
+        launches = K * 4 + 4 * (d1["rebuilds"] - d0["rebuilds"]) + 2 * T_blocks + parts
+    elif w.n <= 192 and plain and not args.kahan:  # a block of steps in one kernel
+        launches = 3 * T_blocks
     else:
-        launches = K * 7 + 2 * T_blocks
+        launches = K * (3 + (1 if w.n <= 8192 else 4)) + 2 * T_blocks + parts
     if args.pcorr > 0:
         launches += K
     if args.pair_noise > 0:  # Clenshaw sweeps per step; filters and the Lanczos check per block
-        launches += args.pair_noise * (K + T_blocks) + (2 + 2 * 32) * T_blocks
+        sweeps = 1 if w.n <= 152 * 8 * 128 else args.pair_noise  # one launch per step while it fits the chip
+        launches += sweeps * K + args.pair_noise * T_blocks + (2 + 2 * 32) * T_blocks
     if args.pair_noise_lanczos >= 0:  # eager steps; per run: transform, norm, 4 launches per iteration, output
         iters = 4 * ((cfg["pair_noise"]["krylov_dimension"] + 3) // 4)
         runs = T_blocks if args.pair_noise_lanczos == 1 else K

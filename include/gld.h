@@ -88,11 +88,14 @@ typedef struct gld_params {
                           * selects 2 m_max                                    */
     int32_t noise_block; /* steps of F^R produced per noise launch (0 = 64)          */
     int32_t psd_clamp;   /* 1: clamp negative noise modes to 0 instead of failing    */
-    int32_t use_graphs;  /* 1 (default): replay steps from a captured CUDA graph
-                          * whose list rebuild is a conditional node; 2: the same
-                          * graph with device-gated rebuild kernels instead (every
-                          * node a plain kernel, e.g. for per-kernel profilers);
-                          * 0: launch every kernel from the host              */
+    int32_t use_graphs;  /* 1 (default): replay steps from captured CUDA graphs,
+                          * list rebuilds gated on the device, from 262144 particles
+                          * on in a conditional node; up to 4096 particles the
+                          * steps of a part of a noise block (up to 192: of any)
+                          * run inside one kernel; 2: graphs of the step
+                          * kernels with gated rebuilds at every size (e.g. for
+                          * per-kernel profilers); 0: launch every kernel from the
+                          * host.  The bits are the same                       */
     const int32_t* order; /* optional [n]: internal storage order (see gld_get_order) */
     void* stream;        /* cudaStream_t for all work of this context                */
     gld_alloc_fn alloc;  /* optional device allocator (NULL: cudaMalloc)             */
@@ -171,7 +174,7 @@ enum {
     GLD_ARR_HIST = 6, /* [m_max-1][n][3]: entry m-1 holds dR_{n-m} (rw)           */
     GLD_ARR_CONV = 7  /* [1+Q+Qs][n][3]: history projections as last computed (r):
                        * of the last step, or of the next one after a
-                       * replayed graph block, which computes them early */
+                       * replayed graph, which may compute them early */
 };
 gld_status gld_get_array(gld_ctx* ctx, int32_t which, double* out);
 gld_status gld_set_array(gld_ctx* ctx, int32_t which, const double* in);
@@ -426,7 +429,8 @@ gld_status gld_get_bytes(gld_ctx* ctx, int64_t* bytes);
  * table points: exactly what gld_get_bytes then reports.  Needs a current
  * device (the VACF partial sums scale with its SM count); no device memory
  * is touched.  The history ring is (m_max-1)*3*n_pad*{4,2} bytes of it, the
- * white-noise window (64 + 2(m_max-1))*3*n_pad*4 bytes. */
+ * white-noise window (64 + 2(m_max-1))*3*n_pad*4 bytes, the parts of a block of
+ * steps (m_max > 32) 16 or, for small systems, 32 times (1+Q+Qs)*3*n_pad*4. */
 gld_status gld_bytes_needed(const gld_params* params, int32_t Q, int32_t Qs, int32_t nr, int64_t* bytes);
 
 const char* gld_last_error(const gld_ctx* ctx);
@@ -436,7 +440,7 @@ gld_status gld_destroy(gld_ctx* ctx);
  * Many GLD systems of different sizes, densities and memory lengths stepped
  * together: every kernel family runs as ONE launch over a tile list of
  * (member, block) for all members, and a 64-step block of the whole batch is
- * one captured CUDA graph.  Members remain ordinary contexts (their arrays,
+ * one captured CUDA graph once a composition has lasted two blocks.  Members remain ordinary contexts (their arrays,
  * VACF and state are read through the gld_* calls above); a member must have
  * its kernels set, use the batch's stream, sit at a 64-step boundary, and
  * share the number of kernel terms, the history type and compensation with
@@ -459,7 +463,8 @@ gld_status gld_batch_step(gld_batch* batch, int64_t nsteps);
 /* Waits, then returns the first latched error of the members. */
 gld_status gld_batch_sync(gld_batch* batch);
 /* members, chosen convolution schedule (-1 before the first step), and the
- * timed milliseconds of the four schedules; pointers may be NULL. */
+ * timed milliseconds of the four schedules (one step's convolution at the
+ * members' position in their rings); pointers may be NULL. */
 gld_status gld_batch_info(gld_batch* batch, int32_t* members, int32_t* schedule, double* schedule_ms);
 /* policy 0 (default): re-time the schedules whenever the members change;
  * 1: re-time only when the total number of convolution columns has moved by

@@ -15,9 +15,9 @@
 // A thread keeps its particles, so own data needs no barrier; positions swap
 // between two buffers, so nothing that others read is overwritten before the
 // next barrier.  All sums run in the order of the kernels for single systems
-// (k_particles.cu, k_history*.cu): the same bits.  A batch runs every small
-// member in a cluster of its own: members no longer wait for each other's
-// launches and list rebuilds.
+// (k_particles.cu, k_history*.cu): the same bits.  Batches keep their tile kernels:
+// a cluster per small member left the chip's other SMs waiting for the longest
+// member (226 to 300 us per step of 64 systems against 192).
 //
 // Arrays that other CTAs write during the kernel are read by plain loads
 // behind the cluster barrier (release / acquire), never through the read-only

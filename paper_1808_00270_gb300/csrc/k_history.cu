@@ -6,8 +6,9 @@
 //   Ps_{i,q} = sum_{m=1}^{m_max-1} gs_q[m]     dR_{i,n-m}     (dK^s terms)
 // With separable kernels K^p_m(r) = sum_q f_q(r) g_q[m] the pair sums of
 // Eq. dissipative_force2 become sum_j f_q(r_ij) e e^T P_{j,q}, so the history
-// ring is streamed exactly once per step, here.  This is the step that sets
-// the cost: 12 (m_max-1) bytes per particle (FP32) against ~2 flops per
+// ring is streamed at most once per step, here (inside a block of steps only
+// the part of it from the first rewritten slot on: k_history_blk.cu).  This is
+// the step that sets the cost: 12 (m_max-1) bytes per particle (FP32) against ~2 flops per
 // byte per accumulator -- bound by HBM bandwidth, so no tensor cores.
 //
 // Layout: ring[slot][3][n_pad], slot = k mod (m_max-1) for dR_k.  Every slot

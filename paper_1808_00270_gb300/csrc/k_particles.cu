@@ -13,6 +13,10 @@
 //                         r_c + skin in the (fixed) stencil traversal order.
 //   cforce                F^C_{n+1} = sum_j 2A/r_c (1 - r/r_c) e_ij and the
 //                         rest of the velocity update; advances n.
+//   pair_lanes, cforce_lanes, nbr_lanes  the same with several lanes per
+//                         particle, where one thread each leaves the SMs idle.
+//   pn_sweeps, pn_stage   the pair-correlated noise: all sweeps of a step in
+//                         one cooperative launch, or a launch each.
 //   vacf                  FP64 accumulation of <V(t0+tau) V(t0)> (Sec. III A).
 //
 // Every neighbour sum runs over a Verlet list with the exact FP32 r < r_c test
