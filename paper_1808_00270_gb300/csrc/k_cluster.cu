@@ -683,8 +683,7 @@ __global__ void __launch_bounds__(kClThreads, 1)
 template <class K, class... A>
 cudaError_t launch_clusters(K kern, int ctas, int csize, size_t smem, cudaStream_t st, const A&... args)
 {
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e == cudaSuccess && csize > 8) e = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    const cudaError_t e = allow_smem(kern, smem, true);  // clusters of up to 16 CTAs
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3((unsigned)ctas);

@@ -63,13 +63,12 @@ cudaError_t choose_shape(long long cols, int H, size_t smem, Shape* out)
     // the order of its sum, does not depend on whether the step is in a block)
     auto kc = hist_conv_col<NACC, KAHAN, BF16, false>;
     auto kg = hist_conv<NACC, KAHAN, BF16>;
-    if (smem > 48 * 1024) {
-        cudaFuncSetAttribute(kc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        cudaFuncSetAttribute(kg, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    }
+    cudaError_t e = allow_smem(kc, smem);
+    if (e == cudaSuccess) e = allow_smem(kg, smem);
+    if (e != cudaSuccess) return e;
     int b1 = 0, bcap_b = kThreads;
     long long bcap = 0;
-    cudaError_t e = one_wave_block(kc, cols, smem, &b1, &bcap, &bcap_b);
+    e = one_wave_block(kc, cols, smem, &b1, &bcap, &bcap_b);
     if (e != cudaSuccess) return e;
     // Room for twice the threads in one wave: split each column's slots (not
     // with compensated sums, which stay one sequence over all m).

@@ -178,7 +178,8 @@ cudaError_t pre_launch(const void* ring, int n_pad, int M, const float* coef, in
 {
     const size_t smem = sizeof(float) * (size_t)NA * (M + LEN);
     auto k = conv_pre<NA, LEN, KAHAN, BF16>;
-    if (smem > 48 * 1024) cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    const cudaError_t e = allow_smem(k, smem);
+    if (e != cudaSuccess) return e;
     const int C = 3 * n_pad / pre_streams(LEN, KAHAN);
     const dim3 grid((unsigned)((C + kPreThreads - 1) / kPreThreads), (unsigned)G, (unsigned)passes);
     k<<<grid, kPreThreads, smem, st>>>(ring, n_pad, M - 1, M, coef, nacc, nstep, part, a0, G);
@@ -190,7 +191,8 @@ cudaError_t b_pre_launch(const BatchPlan& bp, int a0, int passes, cudaStream_t s
 {
     const size_t smem = sizeof(float) * (size_t)NA * (bp.max_H + 1 + LEN);
     auto k = b_conv_pre<NA, LEN, KAHAN, BF16>;
-    if (smem > 48 * 1024) cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    const cudaError_t e = allow_smem(k, smem);
+    if (e != cudaSuccess) return e;
     k<<<dim3((unsigned)bp.n_pre, 1u, (unsigned)passes), kPreThreads, smem, st>>>(bp.desc, bp.pre, a0);
     return cudaGetLastError();
 }
@@ -345,7 +347,8 @@ cudaError_t launch_b_conv_t(const BatchPlan& bp, int t, cudaStream_t st)
 {
     const size_t smem = sizeof(float) * (size_t)bp.max_H * NACC;
     auto k = bp.bf16 ? b_conv<NACC, KAHAN, true> : b_conv<NACC, KAHAN, false>;
-    if (smem > 48 * 1024) cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    const cudaError_t e = allow_smem(k, smem);
+    if (e != cudaSuccess) return e;
     k<<<bp.n_conv, bp.conv_block, smem, st>>>(bp.desc, bp.conv, t);
     return cudaGetLastError();
 }
@@ -365,14 +368,16 @@ cudaError_t part_launch(const Shape& sh, const void* ring, int n_pad, int M, con
     // 68.8 / 75.4 at 100003 in FP32).
     if (sh.kind == 0 && !(KAHAN && bytes / 16 < 384LL * 152)) {
         auto k = hist_conv_col<NACC, KAHAN, BF16, true>;
-        if (smem > 48 * 1024) cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        const cudaError_t e = allow_smem(k, smem);
+        if (e != cudaSuccess) return e;
         k<<<sh.grid, sh.block, smem, st>>>((const typename Col<BF16>::V*)ring, 3LL * n_pad / Col<BF16>::W, H, coef, M,
                                            nstep, step, out, bp);
     } else {
         const int vb = bytes / 16 >= 512LL * 152 ? 16 : bytes / 8 >= 512LL * 152 ? 8 : 4;
         auto k = vb == 16 ? conv_tail<NACC, KAHAN, BF16, 16>
                           : vb == 8 ? conv_tail<NACC, KAHAN, BF16, 8> : conv_tail<NACC, KAHAN, BF16, 4>;
-        if (smem > 48 * 1024) cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        const cudaError_t e = allow_smem(k, smem);
+        if (e != cudaSuccess) return e;
         const int C = (int)(bytes / vb), block = vb == 4 ? 128 : kThreads;
         k<<<(unsigned)((C + block - 1) / block), block, smem, st>>>(ring, n_pad, H, M, coef, nstep, step, bp, sh.G, out);
     }

@@ -346,8 +346,8 @@ int fir_taps_len(int H) { return (2 * H + 1 + 15) & ~15; }
 cudaError_t launch_prep(const PrepArgs& a, cudaStream_t st)
 {
     const size_t smem = sizeof(double) * (size_t)(3 * a.m_max - 1);  // at most 96 KB
-    cudaError_t e = cudaFuncSetAttribute(prep_chat, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(prep_taps, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_smem(prep_chat, smem);
+    if (e == cudaSuccess) e = allow_smem(prep_taps, smem);
     if (e != cudaSuccess) return e;
     prep_chat<<<(unsigned)((a.m_max + kPrepTile - 1) / kPrepTile), kPrepTile, smem, st>>>(a);
     prep_root<<<1, kPrepThreads, 0, st>>>(a);
@@ -371,7 +371,7 @@ cudaError_t launch_noise_block(const StepParams& P, Ctrl* ctrl, float* W, const 
     const int ntaps = fir_taps_len(P.H);
     const int chunk = std::min(ntaps, kFirChunk);
     const size_t smem = fir_smem(chunk);
-    cudaError_t e = cudaFuncSetAttribute(fir, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_smem(fir, smem);
     if (e != cudaSuccess) return e;
     const unsigned grid = (unsigned)((streams + kFirStreams - 1) / kFirStreams);
     fir<<<grid, kFirThreads, smem, st>>>(P, ctrl, W, Acp, ntaps, chunk, frblock);
@@ -386,7 +386,7 @@ cudaError_t launch_noise_filter(const StepParams& P, Ctrl* ctrl, const float* W,
     const int ntaps = fir_taps_len(P.H);
     const int chunk = std::min(ntaps, kFirChunk);
     const size_t smem = fir_smem(chunk);
-    cudaError_t e = cudaFuncSetAttribute(fir, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_smem(fir, smem);
     if (e != cudaSuccess) return e;
     const unsigned grid = (unsigned)((3LL * P.n_pad + kFirStreams - 1) / kFirStreams);
     fir<<<grid, kFirThreads, smem, st>>>(P, ctrl, W, taps, ntaps, chunk, out);
@@ -414,13 +414,12 @@ cudaError_t launch_batch_noise(const BatchPlan& bp, cudaStream_t st)
     b_wgen<<<g, kGenThreads, 0, st>>>(bp.desc, bp.part);
     const int chunk = std::min(bp.max_ntaps, kFirChunk);
     const size_t smem = fir_smem(chunk);
-    cudaError_t e = cudaFuncSetAttribute(b_fir, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_smem(b_fir, smem);
     if (e != cudaSuccess) return e;
     b_fir<<<bp.n_fir, kFirThreads, smem, st>>>(bp.desc, bp.fir, chunk);
     if (bp.pn_kmax > 0) {
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
-        if ((e = cudaFuncSetAttribute(b_fir_pn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess)
-            return e;
+        if ((e = allow_smem(b_fir_pn, smem)) != cudaSuccess) return e;
         for (int k = 1; k <= bp.pn_kmax; ++k) b_fir_pn<<<bp.n_fir, kFirThreads, smem, st>>>(bp.desc, bp.fir, chunk, k);
     }
     return cudaGetLastError();

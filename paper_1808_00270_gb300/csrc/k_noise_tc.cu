@@ -502,7 +502,7 @@ cudaError_t launch_noise_filter_tc(const StepParams& P, Ctrl* ctrl, const CUtens
 {
     if (!noise_filter_tc_ok(P) || !P.wsplit) return cudaErrorInvalidValue;  // it reads the split ring
     const size_t smem = tc_smem_bytes(P.H, P.T);
-    cudaError_t e = cudaFuncSetAttribute(fir_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_smem(fir_tc, smem);
     if (e != cudaSuccess) return e;
     const long long ntiles = (3LL * P.n_pad + 127) / 128;
     const int grid = (int)std::min<long long>(ntiles, std::max(num_sms, 1));

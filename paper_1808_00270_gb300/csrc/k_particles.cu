@@ -2020,11 +2020,8 @@ cudaError_t launch_pcorr(const StepParams& P, const ParticleBuffers& B, cudaStre
     if (P.pc_nbins <= 0 || P.vacf_len <= 0) return cudaSuccess;
     const unsigned grid = (unsigned)std::max(1, (P.n + kThreads - 1) / kThreads);
     const size_t smem = sizeof(long long) * (3 * (size_t)P.n_os * P.pc_nbins + P.pc_nbins);
-    // beside the static pair queues (16 KB)
-    if (smem + sizeof(PcPair) * (kThreads / 32) * kPcQueue > 48 * 1024) {
-        const cudaError_t e = cudaFuncSetAttribute(pcorr, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-    }
+    const cudaError_t e = allow_smem(pcorr, smem);
+    if (e != cudaSuccess) return e;
     pcorr<<<grid, kThreads, smem, st>>>(P, B.ctrl, B.pos, B.vel, B.vorig, B.nbr, B.nbr_cnt, B.pc_step, B.pc_sa,
                                         B.pc_sc, B.pc_n);
     return cudaGetLastError();
@@ -2057,7 +2054,7 @@ cudaError_t pn_sweeps_launch(const StepParams& P, const ParticleBuffers& B, cons
     const int room = std::min(P.maxnb, (int)(200 * 1024 / ((size_t)per_sm * 20 * kSweepThreads)));
     if (!coop || per_sm > 8 || room < 8) return cudaSuccess;
     const size_t smem = (size_t)20 * kSweepThreads * room;
-    if ((e = cudaFuncSetAttribute(pn_sweeps, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess) return e;
+    if ((e = allow_smem(pn_sweeps, smem)) != cudaSuccess) return e;
     int occ = 0;
     if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, pn_sweeps, kSweepThreads, smem)) != cudaSuccess) return e;
     if (occ < per_sm) return cudaSuccess;

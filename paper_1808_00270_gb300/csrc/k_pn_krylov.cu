@@ -456,12 +456,6 @@ size_t sweep_smem(const StepParams& P, int Mp)
     return sizeof(double) * kKryWarps * Mp + sizeof(float) * (size_t)(1 + P.Q + P.Qs + 1) * Mp;
 }
 
-cudaError_t set_smem(const void* f, size_t bytes)
-{
-    if (bytes <= 48 * 1024) return cudaSuccess;
-    return cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-}
-
 }  // namespace
 
 bool kry_fits(const StepParams& P, int Mp)
@@ -480,7 +474,7 @@ cudaError_t kry_ft(const StepParams& P, const Ctrl* ctrl, const float* W, const 
     const long long np3 = 3LL * P.n_pad;
     const dim3 g((unsigned)(Mp / 32), (unsigned)((np3 + kFtThreads - 1) / kFtThreads));
     const size_t smem = (size_t)(P.H + 1) * 8 * sizeof(float4);
-    cudaError_t e = set_smem((const void*)pnk_ft, smem);
+    cudaError_t e = allow_smem(pnk_ft, smem);
     if (e != cudaSuccess) return e;
     pnk_ft<<<g, kFtThreads, smem, st>>>(P, ctrl, W, cosT, M, Mp, Mc, V0);
     return cudaGetLastError();
@@ -522,7 +516,7 @@ cudaError_t kry_matvec(const StepParams& P, const ParticleBuffers& B, const doub
 {
     const unsigned nb = sweep_blocks(P.n);
     const size_t smem = sweep_smem(P, Mp);
-    cudaError_t e = set_smem((const void*)pnk_matvec, smem);
+    cudaError_t e = allow_smem(pnk_matvec, smem);
     if (e != cudaSuccess) return e;
     pnk_matvec<<<nb, 32 * kKryWarps, smem, st>>>(P, B.pos, B.nbr, B.nbr_cnt, B.ftab, B.fptab, wc, beta_k, alive, Mp,
                                                  R, Z, part);

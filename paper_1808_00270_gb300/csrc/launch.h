@@ -7,6 +7,7 @@
 #include <cuda_runtime.h>
 
 #include "gld_internal.cuh"
+#include "kernel_attrs.h"
 
 namespace gld {
 
