@@ -188,12 +188,12 @@ gld_status gld_set_array(gld_ctx* ctx, int32_t which, const double* in);
  * the particle stored at position k; pass it as gld_params.order. */
 gld_status gld_get_order(gld_ctx* ctx, int32_t* int2ext);
 
-/* Diagnostics, out[count] (count <= 5 filled): {graph form of gld_step (0: not
+/* Diagnostics, out[count] (count <= 6 filled): {graph form of gld_step (0: not
  * captured yet, 1: rebuild kernels gated on the device, 2: rebuild in a
  * conditional graph node), neighbour-list builds so far, list capacity per
  * particle, cells per box edge, the largest Krylov dimension any frequency
  * used in the last step's pair-correlated noise (gld_set_pair_noise_krylov;
- * 0 when off)}.
+ * 0 when off), steps taken inside one kernel (use_graphs = 1) so far}.
  * Synchronizes. */
 gld_status gld_get_diag(gld_ctx* ctx, int64_t* out, int32_t count);
 

@@ -715,8 +715,9 @@ SysDesc make_desc(const gld_ctx* c)
 }
 
 // Small systems: steps of a noise block in one kernel (k_cluster.cu), unless
-// the launches of the gated graph were asked for (use_graphs = 2).
-bool steps_in_cluster(const gld_ctx* c) { return c->prm.use_graphs != 2 && cluster_ok(c->P, c->prm.kahan); }
+// the step kernels were asked for, launched one by one (use_graphs = 0) or as
+// the gated graph (2).
+bool steps_in_cluster(const gld_ctx* c) { return c->prm.use_graphs == 1 && cluster_ok(c->P, c->prm.kahan); }
 
 // A noise block and its 64 steps as a graph of three kernels.
 bool capture_cluster_graph(gld_ctx* c)
@@ -757,7 +758,7 @@ gld_status step_cluster(gld_ctx* c, int64_t k, bool boundary)
         c->block_start = first;
         c->noise_end = first + T;
     }
-    if (boundary && c->prm.use_graphs && k == T && rel0 == 0 && c->P.n <= kClusterBlockMaxN && capture_cluster_graph(c)) {
+    if (boundary && k == T && rel0 == 0 && c->P.n <= kClusterBlockMaxN && capture_cluster_graph(c)) {
         GLD_CUDA(c, cudaGraphLaunch(c->gexec, c->st));
     } else {
         if (boundary) GLD_CUDA(c, launch_noise(c, c->st));
@@ -765,6 +766,7 @@ gld_status step_cluster(gld_ctx* c, int64_t k, bool boundary)
     }
     c->noise_valid = true;
     c->host_step += k;
+    c->cluster_steps += k;
     c->last_fr_row = c->host_step - 1 - c->block_start;
     c->conv_valid_step = -1;
     const long long origin = first - rel0;
@@ -1504,8 +1506,8 @@ gld_status gld_get_diag(gld_ctx* c, int64_t* out, int32_t count)
     GLD_TRY(sync_and_check(c));
     long long rebuilds = 0;
     GLD_CUDA(c, cudaMemcpy(&rebuilds, &c->B.ctrl->rebuilds, sizeof(rebuilds), cudaMemcpyDeviceToHost));
-    const int64_t v[5] = {c->graph_mode, rebuilds, c->P.maxnb, c->P.nc, c->kry.last_iters};
-    for (int k = 0; k < count; ++k) out[k] = k < 5 ? v[k] : 0;
+    const int64_t v[6] = {c->graph_mode, rebuilds, c->P.maxnb, c->P.nc, c->kry.last_iters, c->cluster_steps};
+    for (int k = 0; k < count; ++k) out[k] = k < 6 ? v[k] : 0;
     return GLD_OK;
 }
 

@@ -145,7 +145,7 @@ gld_status admit(gld_server* s, Req* r)
     p.free = pool_free;
     p.alloc_user = s;
     p.order = nullptr;
-    p.use_graphs = 0;
+    p.use_graphs = 1;  // (the last steps, less than a block: too few for a graph to be captured)
     gld_ctx* c = nullptr;
     gld_status st = gld_create(&p, r->pos.data(), r->vel.data(), &c);
     if (st != GLD_OK) return st;
