@@ -26,14 +26,13 @@
 
 #include <cuda_bf16.h>
 
+#include "cluster_fit.h"
 #include "history.cuh"
 #include "neighbours.cuh"
 
 namespace gld {
 
 namespace {
-
-constexpr int kClThreads = 512;
 
 __device__ __forceinline__ void cluster_barrier()
 {
@@ -680,68 +679,109 @@ __global__ void __launch_bounds__(kClThreads, 1)
     cl_rebuild<kRebLanes>(P, B, B.pos_next, rlists, cluster_rank(), (int)gridDim.x);
 }
 
-template <class K, class... A>
-cudaError_t launch_clusters(K kern, int ctas, int csize, size_t smem, cudaStream_t st, const A&... args)
-{
-    const cudaError_t e = allow_smem(kern, smem, true);  // clusters of up to 16 CTAs
-    if (e != cudaSuccess) return e;
+// A launch of one cluster of `ctas` CTAs.
+struct ClusterLaunch {
     cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3((unsigned)ctas);
-    cfg.blockDim = dim3(kClThreads);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = st;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = (unsigned)csize;
-    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
-    cfg.attrs = at;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kern, args...);
+    cudaLaunchAttribute at{};
+    ClusterLaunch(int ctas, size_t smem, cudaStream_t st)
+    {
+        cfg.gridDim = dim3((unsigned)ctas);
+        cfg.blockDim = dim3(kClThreads);
+        cfg.dynamicSmemBytes = smem;
+        cfg.stream = st;
+        at.id = cudaLaunchAttributeClusterDimension;
+        at.val.clusterDim.x = (unsigned)ctas;
+        at.val.clusterDim.y = at.val.clusterDim.z = 1;
+        cfg.attrs = &at;
+        cfg.numAttrs = 1;
+    }
+    ClusterLaunch(const ClusterLaunch&) = delete;
+};
+
+template <class... P, class... A>
+cudaError_t launch_cluster(void (*kern)(P...), int ctas, size_t smem, cudaStream_t st, const A&... args)
+{
+    const cudaError_t e = allow_smem(kern, smem, true);
+    if (e != cudaSuccess) return e;
+    ClusterLaunch l(ctas, smem, st);
+    return cudaLaunchKernelEx(&l.cfg, kern, args...);
 }
 
-template <int NACC, bool BF16, int L>
-cudaError_t launch_l(const SysDesc& d, int ncta, int nsteps, int rel0, int G, int len, cudaStream_t st)
+template <class... P>
+bool cluster_fits(void (*kern)(P...), int ctas, size_t smem)
 {
-    auto kern = steps_cluster<NACC, BF16, L>;
-    const size_t smem = sizeof(float) * NACC * (size_t)(d.P.m_max + std::max(len, 8)) +
-                        sizeof(int) * (kClThreads / L) * (size_t)d.P.maxnb;
-    return launch_clusters(kern, ncta, ncta, smem, st, d, nsteps, rel0, G, len);
+    static ClusterFit fit;
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) return false;
+    return fit(dev, (const void*)kern, ctas, smem, [&](size_t bytes) {
+        int active = 0;
+        cudaError_t e = allow_smem(kern, bytes, true);
+        if (e == cudaSuccess) {
+            ClusterLaunch l(ctas, bytes, nullptr);
+            e = cudaOccupancyMaxActiveClusters(&active, kern, &l.cfg);
+        }
+        if (e != cudaSuccess) {
+            cudaGetLastError();
+            return 0;
+        }
+        return active;
+    });
 }
+
+using StepsKernel = void (*)(const SysDesc, int, int, int, int);
+
+// The instantiation, CTAs and shared memory for the steps of a system: eight
+// lanes per particle, in up to 16 CTAs.
+StepsKernel steps_kernel(const StepParams& P, int* ctas, size_t* smem)
+{
+    *ctas = cluster_ctas(P.n, 8);
+    const int lanes = cluster_lanes(P.n, *ctas);
+    *smem = sizeof(float) * P.nacc * (size_t)(P.m_max + pre_len(0, 1)) +  // (no block is longer)
+            sizeof(int) * (size_t)(kClThreads / lanes) * (size_t)P.maxnb;
+    auto of = [&](auto na, auto bf) -> StepsKernel {
+        constexpr int N = decltype(na)::value;
+        constexpr bool B = decltype(bf)::value;
+        return lanes == 8 ? steps_cluster<N, B, 8> : lanes == 4 ? steps_cluster<N, B, 4> : steps_cluster<N, B, 2>;
+    };
+    using I1 = std::integral_constant<int, 1>;
+    using I2 = std::integral_constant<int, 2>;
+    if (P.nacc == 1) return P.hist_bf16 ? of(I1{}, std::true_type{}) : of(I1{}, std::false_type{});
+    return P.hist_bf16 ? of(I2{}, std::true_type{}) : of(I2{}, std::false_type{});
+}
+
+size_t rebuild_smem(const StepParams& P) { return sizeof(int) * (kClThreads / kRebLanes) * (size_t)P.maxnb; }
 
 }  // namespace
 
 bool cluster_ok(const StepParams& P, int kahan)
 {
-    return P.n <= kClusterMaxN && P.maxnb <= 128 && !kahan && !P.perp && P.Qs == 0 && P.Q <= 1 && P.nmodes == 0 &&
-           P.pn_deg == 0 && !P.pn_kry && P.pc_nbins == 0 && P.T == kMaxNoiseBlock;
+    if (P.n > kClusterMaxN || P.maxnb > 128 || kahan || P.perp || P.Qs > 0 || P.Q > 1 || P.nmodes > 0 || P.pn_deg > 0 ||
+        P.pn_kry || P.pc_nbins > 0 || P.T != kMaxNoiseBlock)
+        return false;
+    int ctas = 0;
+    size_t smem = 0;
+    const StepsKernel kern = steps_kernel(P, &ctas, &smem);
+    return cluster_fits(kern, ctas, smem);
 }
 
 cudaError_t launch_steps_cluster(const SysDesc& d, int nsteps, int rel0, int G, int len, cudaStream_t st)
 {
     if (!d.P.cblk) G = len = 1;  // no blocks: one range over the whole ring
-    int c = 1;  // CTAs: eight lanes per particle, up to 16
-    while (c < 16 && c * kClThreads / 8 < d.P.n) c *= 2;
-    const int lanes = c * kClThreads / 8 >= d.P.n ? 8 : c * kClThreads / 4 >= d.P.n ? 4 : 2;
-    auto go = [&](auto na, auto bf) {
-        constexpr int N = decltype(na)::value;
-        constexpr bool B = decltype(bf)::value;
-        return lanes == 8   ? launch_l<N, B, 8>(d, c, nsteps, rel0, G, len, st)
-               : lanes == 4 ? launch_l<N, B, 4>(d, c, nsteps, rel0, G, len, st)
-                            : launch_l<N, B, 2>(d, c, nsteps, rel0, G, len, st);
-    };
-    using I1 = std::integral_constant<int, 1>;
-    using I2 = std::integral_constant<int, 2>;
-    if (d.P.nacc == 1) return d.P.hist_bf16 ? go(I1{}, std::true_type{}) : go(I1{}, std::false_type{});
-    return d.P.hist_bf16 ? go(I2{}, std::true_type{}) : go(I2{}, std::false_type{});
+    int ctas = 0;
+    size_t smem = 0;
+    const StepsKernel kern = steps_kernel(d.P, &ctas, &smem);
+    return launch_cluster(kern, ctas, smem, st, d, nsteps, rel0, G, len);
 }
 
-bool rebuild_in_cluster(const StepParams& P) { return P.n <= kClusterRebuildMaxN && P.maxnb <= 128; }
+bool rebuild_in_cluster(const StepParams& P)
+{
+    return P.n <= kClusterRebuildMaxN && P.maxnb <= 128 &&
+           cluster_fits(rebuild_cluster, cluster_ctas(P.n, kRebLanes), rebuild_smem(P));
+}
 
 cudaError_t launch_rebuild_cluster(const StepParams& P, const ParticleBuffers& B, cudaStream_t st)
 {
-    int c = 1;
-    while (c < 16 && c * (kClThreads / kRebLanes) < P.n) c *= 2;
-    return launch_clusters(rebuild_cluster, c, c, sizeof(int) * (kClThreads / kRebLanes) * (size_t)P.maxnb, st, P, B);
+    return launch_cluster(rebuild_cluster, cluster_ctas(P.n, kRebLanes), rebuild_smem(P), st, P, B);
 }
 
 }  // namespace gld

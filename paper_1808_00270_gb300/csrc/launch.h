@@ -186,7 +186,7 @@ cudaError_t launch_batch_conv(const BatchPlan& bp, int step, cudaStream_t st);  
 cudaError_t launch_batch_particles(const BatchPlan& bp, cudaStream_t st); // k_particles.cu
 cudaError_t launch_batch_noise(const BatchPlan& bp, cudaStream_t st);     // k_noise.cu
 // Whole steps of small systems (k_cluster.cu): whether a system's features and
-// size allow it; a system alone for nsteps steps of its noise block (rel0:
+// size allow it and the device can hold its cluster; a system alone for nsteps steps of its noise block (rel0:
 // number of the first step in its block of the convolution, > 0: that block's
 // parts are formed; G and len as conv_block_shape).
 // Sizes (us per step, cluster against the graph of the step kernels): a whole
