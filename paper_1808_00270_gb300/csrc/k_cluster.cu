@@ -766,7 +766,10 @@ bool cluster_ok(const StepParams& P, int kahan)
 
 cudaError_t launch_steps_cluster(const SysDesc& d, int nsteps, int rel0, int G, int len, cudaStream_t st)
 {
-    if (!d.P.cblk) G = len = 1;  // no blocks: one range over the whole ring
+    if (!d.P.cblk) {  // no parts: whole sums, in the ranges of the step kernels (one for memories too short for blocks)
+        len = 1;
+        G = std::max(G, 1);
+    }
     int ctas = 0;
     size_t smem = 0;
     const StepsKernel kern = steps_kernel(d.P, &ctas, &smem);
