@@ -34,9 +34,13 @@ namespace gld {
 
 namespace {
 
+// (Without .aligned: the barriers stand behind loops that lanes leave one by one,
+// and nothing obliges the compiler to bring a warp together before inline
+// assembly.  us per step without / with it: 7.42 / 7.40 at 64 particles, 15.94 /
+// 15.91 at 2048, 18.75 / 18.78 at 4096.)
 __device__ __forceinline__ void cluster_barrier()
 {
-    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+    asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
 }
 
 // Data written by other CTAs: plain loads.

@@ -50,3 +50,10 @@ def test_the_cluster_kernels_ask_first():
     for rule in ("bool cluster_ok(", "bool rebuild_in_cluster("):
         body = s[s.index(rule):]
         assert "cluster_fits(" in body[: body.index("\n}\n")]
+
+
+def test_cluster_barriers_take_lanes_one_by_one():
+    """The barriers stand behind loops that lanes leave by break and continue: the
+    form that presumes a converged warp is not used."""
+    asm = [x for x in open(os.path.join(B.CSRC, "k_cluster.cu")) if "barrier.cluster" in x]
+    assert asm and not any(".aligned" in x for x in asm)
