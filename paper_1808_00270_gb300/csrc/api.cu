@@ -302,7 +302,7 @@ gld_status ring_form(gld_ctx* c, bool alone, cudaStream_t s)
 gld_status rebuild_cells_and_fc(gld_ctx* c)
 {
     const int one = 1;
-    GLD_CUDA(c, cudaMemcpyAsync(&c->B.ctrl->rebuild, &one, sizeof(int), cudaMemcpyHostToDevice, c->st));
+    GLD_CUDA(c, cudaMemcpyAsync(c->B.ctrl->rebuild, &one, sizeof(int), cudaMemcpyHostToDevice, c->st));
     GLD_CUDA(c, launch_rebuild(c->P, c->B, c->st));
     GLD_CUDA(c, launch_cforce(c->P, c->B, 0, c->st));
     return GLD_OK;
@@ -388,7 +388,7 @@ cudaError_t launch_one_step(gld_ctx* c, cudaStream_t s)
 }
 
 // One step captured with the rebuild kernels in the body of a conditional
-// (IF) node whose condition a one-thread kernel sets from ctrl->rebuild, so
+// (IF) node whose condition a one-thread kernel sets from ctrl->rebuild[0], so
 // steps without a rebuild launch none of them.
 // With `overlap`, the step's own convolution is not captured (the previous
 // step computed it) and the next step's convolution is forked onto a second
@@ -1468,9 +1468,9 @@ gld_status gld_set_array(gld_ctx* c, int32_t which, const double* in)
         // replaced displacement gets fresh lists (positions are unchanged).
         GLD_TRY(upload_vec(c, c->B.disp, in, false));
         const int one = 1, zero = 0;
-        GLD_CUDA(c, cudaMemcpyAsync(&c->B.ctrl->rebuild, &one, sizeof(int), cudaMemcpyHostToDevice, c->st));
+        GLD_CUDA(c, cudaMemcpyAsync(c->B.ctrl->rebuild, &one, sizeof(int), cudaMemcpyHostToDevice, c->st));
         GLD_CUDA(c, launch_rebuild(c->P, c->B, c->st));
-        GLD_CUDA(c, cudaMemcpyAsync(&c->B.ctrl->rebuild, &zero, sizeof(int), cudaMemcpyHostToDevice, c->st));
+        GLD_CUDA(c, cudaMemcpyAsync(c->B.ctrl->rebuild, &zero, sizeof(int), cudaMemcpyHostToDevice, c->st));
         return sync_and_check(c);
     }
     case GLD_ARR_HIST: {

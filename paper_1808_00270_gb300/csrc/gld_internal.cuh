@@ -37,8 +37,9 @@ struct Ctrl {
     unsigned done_cforce;  // last-block counters (reset by the last block)
     unsigned done_scan;
     unsigned done_fir;
-    int rebuild;           // != 0: rebuild cells and neighbour lists after this step's move
-    int pad_;
+    // [0] != 0: rebuild cells and neighbour lists after this step's move (the
+    // steps inside a cluster take [0] and [1] in turn, for even and odd steps)
+    int rebuild[2];
     long long rebuilds;    // neighbour-list builds so far
     long long hslot;       // step mod H: the history slot this step writes
     long long conv_step;   // n + 1, written by the pair kernel of step n

@@ -527,7 +527,8 @@ __device__ __forceinline__ void cl_steps(const SysDesc& d, int nsteps, int rel0,
         vs.pending = ctrl->vacf_pending;
     }
     float4 *cur = B.pos, *nxt = B.pos_next;
-    int* flags = &ctrl->rebuild;  // [2]: requests of even and odd steps (ctrl->rebuild, ctrl->pad_)
+    static_assert(sizeof(Ctrl::rebuild) == 2 * sizeof(int), "requests of even and odd steps");
+    int* flags = ctrl->rebuild;
     const float g00 = NACC > 1 ? __ldg(B.g0) : 0.f;
     int rel = rel0;
     auto barrier = [&]() {
@@ -679,7 +680,7 @@ __global__ void __launch_bounds__(kClThreads, 1)
     rebuild_cluster(const __grid_constant__ StepParams P, const __grid_constant__ ParticleBuffers B)
 {
     extern __shared__ int rlists[];
-    if (B.ctrl->rebuild == 0) return;  // the same for the whole cluster
+    if (B.ctrl->rebuild[0] == 0) return;  // the same for the whole cluster
     cl_rebuild<kRebLanes>(P, B, B.pos_next, rlists, cluster_rank(), (int)gridDim.x);
 }
 

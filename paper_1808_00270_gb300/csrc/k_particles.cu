@@ -143,10 +143,10 @@ __device__ __forceinline__ void pair_finish(const StepParams& P, Ctrl* __restric
     // Verlet criterion: a particle moved more than half the skin since the build.
     const float4 db = disp_build[id];
     const float mx = dn.x - db.x, my = dn.y - db.y, mz = dn.z - db.z;
-    if (mx * mx + my * my + mz * mz > P.trig2) atomicOr(&ctrl->rebuild, 1);
+    if (mx * mx + my * my + mz * mz > P.trig2) atomicOr(ctrl->rebuild, 1);
     if (!(isfinite(dRx) && isfinite(dRy) && isfinite(dRz))) {
         atomicOr(err, kErrNonFinite);
-        atomicOr(&ctrl->rebuild, 1);
+        atomicOr(ctrl->rebuild, 1);
     }
 }
 
@@ -492,7 +492,7 @@ __device__ __forceinline__ void nbr_build_body(const StepParams& P, Ctrl* __rest
               const int* __restrict__ cell_start, int* __restrict__ nbr, int* __restrict__ nbr_cnt,
               int* __restrict__ perm, const float4* __restrict__ disp, float4* __restrict__ disp_build, int blk, int nblk)
 {
-    if (ctrl->rebuild == 0) return;
+    if (ctrl->rebuild[0] == 0) return;
     const int k = blk * blockDim.x + threadIdx.x;
     if (k == 0) ctrl->rebuilds += 1;
     if (k >= P.n) return;
@@ -557,7 +557,7 @@ __device__ __forceinline__ void nbr_lanes_body(const StepParams& P, Ctrl* ctrl, 
                                                const float4* __restrict__ disp, float4* __restrict__ disp_build, int blk,
                                                int nblk)
 {
-    if (ctrl->rebuild == 0) return;
+    if (ctrl->rebuild[0] == 0) return;
     extern __shared__ int lists[];  // [kNbrGroups][maxnb]
     __shared__ int lcnt[kNbrGroups];
     constexpr int L = kNbrLanes, R = (9 + L - 1) / L;
@@ -870,7 +870,7 @@ __device__ __forceinline__ void cforce_body(const StepParams& P, Ctrl* __restric
     // kCforceLanes consecutive lanes share a particle and split its list
     const int k = (blk * blockDim.x + threadIdx.x) / kCforceLanes;
     const int lr = threadIdx.x & (kCforceLanes - 1);
-    if (blk == 0 && threadIdx.x == 0) ctrl->rebuild = 0;  // the lists are current for R_{n+1}
+    if (blk == 0 && threadIdx.x == 0) ctrl->rebuild[0] = 0;  // the lists are current for R_{n+1}
     if (k < P.n) {  // uniform over the lanes of a particle
         const int id = k;
         const float4 pi = pos_next[id];
@@ -963,7 +963,7 @@ __global__ void __launch_bounds__(kThreads * L) cforce_lanes(const StepParams P,
     __shared__ float4 vsh[VACF ? kThreads : 1];
     const Lanes<L> ln;
     const int grp = threadIdx.x / L, id = (int)(blockIdx.x * blockDim.x / L) + grp;
-    if (blockIdx.x == 0 && threadIdx.x == 0) ctrl->rebuild = 0;  // the lists are current for R_{n+1}
+    if (blockIdx.x == 0 && threadIdx.x == 0) ctrl->rebuild[0] = 0;  // the lists are current for R_{n+1}
     if (id < P.n) {  // uniform over the lanes of a particle
         const float4 pi = pos_next[id];
         float4 vh;
@@ -1313,7 +1313,7 @@ __global__ void __launch_bounds__(kThreads) export_vec(int n, const float4* __re
 // Sets the graph condition that guards the rebuild kernels.
 __global__ void rebuild_decide(cudaGraphConditionalHandle h, const Ctrl* __restrict__ ctrl)
 {
-    cudaGraphSetConditional(h, ctrl->rebuild != 0 ? 1u : 0u);
+    cudaGraphSetConditional(h, ctrl->rebuild[0] != 0 ? 1u : 0u);
 }
 
 // A bounded idle wait of one thread (lets the host run ahead of the device
@@ -1344,7 +1344,7 @@ __global__ void b_cell_assign(const SysDesc* __restrict__ D, const Tile* __restr
     const Tile t = tiles[blockIdx.x];
     const SysDesc& d = D[t.m];
     const ParticleBuffers& B = d.B;
-    cell_assign_body(d.P, &B.ctrl->rebuild, B.pos_next, B.cell_head, B.cell_next, B.cell_count, t.b, d.nb_part);
+    cell_assign_body(d.P, B.ctrl->rebuild, B.pos_next, B.cell_head, B.cell_next, B.cell_count, t.b, d.nb_part);
 }
 
 __global__ void __launch_bounds__(kCellThreads) b_cell_scan(const SysDesc* __restrict__ D, const Tile* __restrict__ tiles)
@@ -1352,7 +1352,7 @@ __global__ void __launch_bounds__(kCellThreads) b_cell_scan(const SysDesc* __res
     const Tile t = tiles[blockIdx.x];
     const SysDesc& d = D[t.m];
     const ParticleBuffers& B = d.B;
-    cell_scan_body(&B.ctrl->rebuild, B.cell_count, B.ncells, B.chunk_sum, B.chunk_off, &B.ctrl->done_scan, t.b,
+    cell_scan_body(B.ctrl->rebuild, B.cell_count, B.ncells, B.chunk_sum, B.chunk_off, &B.ctrl->done_scan, t.b,
                    d.nb_cell);
 }
 
@@ -1361,7 +1361,7 @@ __global__ void __launch_bounds__(kCellThreads) b_cell_fill(const SysDesc* __res
     const Tile t = tiles[blockIdx.x];
     const SysDesc& d = D[t.m];
     const ParticleBuffers& B = d.B;
-    cell_fill_body(d.P, &B.ctrl->rebuild, B.ncells, B.pos_next, B.cell_count, B.cell_head, B.cell_next, B.chunk_off,
+    cell_fill_body(d.P, B.ctrl->rebuild, B.ncells, B.pos_next, B.cell_count, B.cell_head, B.cell_next, B.chunk_off,
                    B.cell_start, B.pos_sorted, t.b, d.nb_cell);
 }
 
@@ -1976,7 +1976,7 @@ cudaError_t launch_cell_build(const StepParams& P, const ParticleBuffers& B, con
 cudaError_t launch_rebuild(const StepParams& P, const ParticleBuffers& B, cudaStream_t st)
 {
     if (rebuild_in_cluster(P)) return launch_rebuild_cluster(P, B, st);
-    cudaError_t e = launch_cell_build(P, B, B.pos_next, &B.ctrl->rebuild, st);
+    cudaError_t e = launch_cell_build(P, B, B.pos_next, B.ctrl->rebuild, st);
     if (e != cudaSuccess) return e;
     if (P.maxnb <= kNbrSortCap && P.n <= kNbrLanesMaxN)
         return launch_nbr_lanes(nbr_lanes, std::min((P.n + kNbrGroups - 1) / kNbrGroups, 6 * 152), P.maxnb, st, P, B.ctrl, B.pos_sorted,

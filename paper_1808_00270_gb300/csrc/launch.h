@@ -75,12 +75,12 @@ cudaError_t launch_delay(unsigned long long ns, cudaStream_t st);
 // and *gate == 0.
 cudaError_t launch_cell_build(const StepParams& P, const ParticleBuffers& B, const float4* src, const int* gate,
                               cudaStream_t st);
-// Cell list and neighbour lists at R_{n+1} (pos_next), when ctrl->rebuild != 0.
+// Cell list and neighbour lists at R_{n+1} (pos_next), when ctrl->rebuild[0] != 0.
 cudaError_t launch_rebuild(const StepParams& P, const ParticleBuffers& B, cudaStream_t st);
-// Inside a captured graph: sets conditional handle h to (ctrl->rebuild != 0).
+// Inside a captured graph: sets conditional handle h to (ctrl->rebuild[0] != 0).
 cudaError_t launch_rebuild_decide(cudaGraphConditionalHandle h, const Ctrl* ctrl, cudaStream_t st);
 // mode 0: F^C only (initialisation); mode 1: F^C_{n+1}, V_{n+1}, step += 1.
-// Both copy pos_next into pos and clear ctrl->rebuild.
+// Both copy pos_next into pos and clear ctrl->rebuild[0].
 cudaError_t launch_cforce(const StepParams& P, const ParticleBuffers& B, int mode, cudaStream_t st);
 cudaError_t launch_vacf(const StepParams& P, const ParticleBuffers& B, cudaStream_t st);
 // Adds the last VACF launch's partials to the FP64 sums (before reading them).
@@ -198,7 +198,7 @@ constexpr int kClusterBlockMaxN = 192;
 bool cluster_ok(const StepParams& P, int kahan);
 cudaError_t launch_steps_cluster(const SysDesc& d, int nsteps, int rel0, int G, int len, cudaStream_t st);
 
-// The list build of launch_rebuild by one cluster (gated on ctrl->rebuild), for
+// The list build of launch_rebuild by one cluster (gated on ctrl->rebuild[0]), for
 // systems where that is faster than the four kernels (us per step 13.5 / 15.6 at
 // 4096 particles, 16.4 / 16.9 at 8192, 18.8 / 17.7 at 10007).
 constexpr int kClusterRebuildMaxN = 8192;
