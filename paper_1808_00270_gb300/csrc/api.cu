@@ -22,6 +22,7 @@
 
 #include <cuda_bf16.h>
 
+#include "cluster_fit.h"
 #include "ctx.h"
 
 using namespace gld;
@@ -976,7 +977,7 @@ size_t ctx_bytes_needed(const gld_params* p, int Q, int Qs, int nr, int num_sms)
         sizeof(Ctrl), 16 * np, 16 * np, 16 * np, 16 * np, 4 * (size_t)P.maxnb * np, 4 * np, 4 * np,
         16 * np, 16 * np, 16 * np, 16 * np, 16 * np, elem * n3 * P.H, 4 * (size_t)kMaxAcc * n3,
         4 * (size_t)P.T * n3, 4 * (size_t)P.lw * n3, 4 * ((size_t)ncells + 1), 4 * (size_t)ncells,
-        4 * (size_t)ncells, 4 * np, 4 * (size_t)chunks, 4 * (size_t)chunks,
+        4 * (size_t)ncells, 4 * np, 4 * (size_t)scan_totals(ncells), 4 * (size_t)chunks,
         16 * (size_t)std::max(P.n_os, 1) * P.n, 8 * (size_t)std::max(P.n_os, 1) * vacf_gx,
         8 * (size_t)std::max(P.vacf_len, 1), 8 * (size_t)std::max(P.vacf_len, 1), 8,
         4 * (size_t)fir_taps_len(P.H), 4 * (size_t)kMaxAcc * P.m_max, 4 * 2 * (size_t)kMaxQ,
@@ -1119,7 +1120,7 @@ gld_status gld_create(const gld_params* p, const double* pos, const double* vel,
     B.cell_count = alloc_n<int>(c, ncells, ok);
     B.cell_head = alloc_n<int>(c, ncells, ok);
     B.cell_next = alloc_n<int>(c, np, ok);
-    B.chunk_sum = alloc_n<int>(c, chunks, ok);
+    B.chunk_sum = alloc_n<int>(c, scan_totals(ncells), ok);
     B.chunk_off = alloc_n<int>(c, chunks, ok);
     B.vacf_gx = vacf_blocks(P.n, c->num_sms);
     B.vorig = alloc_n<float4>(c, (size_t)std::max(P.n_os, 1) * P.n, ok);

@@ -31,6 +31,14 @@ inline int cluster_lanes(int n, int ctas)
     return ctas * kClThreads / 8 >= n ? 8 : ctas * kClThreads / 4 >= n ? 4 : 2;
 }
 
+// Totals of the cell scan: one per chunk of 512 cells, or one per CTA of the list
+// build in a cluster, whichever is more.
+inline int scan_totals(int ncells)
+{
+    const int chunks = (ncells + 511) / 512;
+    return chunks > kClMaxCtas ? chunks : kClMaxCtas;
+}
+
 class ClusterFit {
 public:
     // ask(smem): clusters that can be resident at once (0: none, or it failed).

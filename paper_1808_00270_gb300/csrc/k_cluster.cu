@@ -204,7 +204,7 @@ template <int L>
 __device__ __forceinline__ void cl_rebuild(const StepParams& P, const ParticleBuffers& B, const float4* nxt, int* lists,
                                            int rank, int ncta)
 {
-    __shared__ int lcnt[kClThreads / L], cbase[16];
+    __shared__ int lcnt[kClThreads / L], cbase[kClMaxCtas];
     Ctrl* ctrl = B.ctrl;
     const int n = P.n, tid = threadIdx.x, np = P.n_pad;
     const int lane = tid & (L - 1), grp = tid / L;

@@ -17,6 +17,7 @@ int main() {
     CHECK(cluster_ctas(1, 8) == 1 && cluster_ctas(64, 8) == 1 && cluster_ctas(65, 8) == 2);
     CHECK(cluster_ctas(1024, 8) == 16 && cluster_ctas(4096, 8) == 16 && cluster_ctas(8192, 4) == 16);
     CHECK(cluster_lanes(1024, 16) == 8 && cluster_lanes(1025, 16) == 4 && cluster_lanes(2049, 16) == 2);
+    CHECK(scan_totals(1) == 16 && scan_totals(8192) == 16 && scan_totals(8193) == 17);  // a word per CTA at least
     int a = 0, b = 0, asked = 0;
     size_t seen = 0;
     ClusterFit fit;
