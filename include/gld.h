@@ -188,12 +188,15 @@ gld_status gld_set_array(gld_ctx* ctx, int32_t which, const double* in);
  * the particle stored at position k; pass it as gld_params.order. */
 gld_status gld_get_order(gld_ctx* ctx, int32_t* int2ext);
 
-/* Diagnostics, out[count] (count <= 6 filled): {graph form of gld_step (0: not
+/* Diagnostics, out[count] (count <= 8 filled): {graph form of gld_step (0: not
  * captured yet, 1: rebuild kernels gated on the device, 2: rebuild in a
  * conditional graph node), neighbour-list builds so far, list capacity per
  * particle, cells per box edge, the largest Krylov dimension any frequency
  * used in the last step's pair-correlated noise (gld_set_pair_noise_krylov;
- * 0 when off), steps taken inside one kernel (use_graphs = 1) so far}.
+ * 0 when off), steps taken inside one kernel (use_graphs = 1) so far,
+ * ranges of slots that a memory sum is split into (0: m_max <= 32 or no
+ * kernels), steps of a block whose parts the convolution forms at once (0: it
+ * streams whole rings)}.
  * Synchronizes. */
 gld_status gld_get_diag(gld_ctx* ctx, int64_t* out, int32_t count);
 
@@ -226,9 +229,10 @@ gld_status gld_get_pairs(gld_ctx* ctx, int32_t* pairs, int64_t cap, int64_t* cou
  * Synchronizes. */
 enum {
     GLD_PROF_NOISE = 0,  /* white-noise generation + moving average (per block) */
-    GLD_PROF_HIST = 1,   /* history convolution                               */
+    GLD_PROF_HIST = 1,   /* history convolution: a kernel per step, and the    */
+                         /* parts' one or two per block of 8 or 16 steps       */
     GLD_PROF_PAIR = 2,   /* F^D, position update, history write               */
-    GLD_PROF_CELL = 3,   /* cell + neighbour-list rebuild (4 kernels, gated)  */
+    GLD_PROF_CELL = 3,   /* cell + neighbour-list rebuild (1 or 4 kernels)    */
     GLD_PROF_CFORCE = 4, /* F^C_{n+1}, velocity update and the VACF terms     */
     GLD_PROF_VACF = 5,   /* velocity autocorrelation in batches only (single  */
                          /* contexts accumulate it inside the F^C kernel: 0)  */

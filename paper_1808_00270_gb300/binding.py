@@ -321,10 +321,11 @@ class GLD:
         self._check(lib().gld_set_step(self._h, int(step)))
 
     def diag(self) -> dict:
-        out = np.zeros(6, dtype=np.int64)
-        self._check(lib().gld_get_diag(self._h, _ptr(out), 6))
+        out = np.zeros(8, dtype=np.int64)
+        self._check(lib().gld_get_diag(self._h, _ptr(out), 8))
         return dict(graph_mode=int(out[0]), rebuilds=int(out[1]), maxnb=int(out[2]), cells_per_edge=int(out[3]),
-                    krylov_iterations=int(out[4]), cluster_steps=int(out[5]))
+                    krylov_iterations=int(out[4]), cluster_steps=int(out[5]), conv_ranges=int(out[6]),
+                    conv_block=int(out[7]))
 
     def set_memory_modes(self, rates, omegas):
         """Carries the memory sums in auxiliary-variable form for kernels that

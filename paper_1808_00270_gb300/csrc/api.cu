@@ -1507,8 +1507,9 @@ gld_status gld_get_diag(gld_ctx* c, int64_t* out, int32_t count)
     GLD_TRY(sync_and_check(c));
     long long rebuilds = 0;
     GLD_CUDA(c, cudaMemcpy(&rebuilds, &c->B.ctrl->rebuilds, sizeof(rebuilds), cudaMemcpyDeviceToHost));
-    const int64_t v[6] = {c->graph_mode, rebuilds, c->P.maxnb, c->P.nc, c->kry.last_iters, c->cluster_steps};
-    for (int k = 0; k < count; ++k) out[k] = k < 6 ? v[k] : 0;
+    const int64_t v[8] = {c->graph_mode,      rebuilds,         c->P.maxnb, c->P.nc,
+                          c->kry.last_iters, c->cluster_steps, c->conv_G,  c->P.cblk ? c->conv_len : 0};
+    for (int k = 0; k < count; ++k) out[k] = k < 8 ? v[k] : 0;
     return GLD_OK;
 }
 
@@ -1611,7 +1612,11 @@ gld_status gld_profile_steps(gld_ctx* c, int64_t nsteps, double* ms, int64_t* la
     const bool pnoise = c->P.pn_deg > 0;
     const size_t nk = 1 + (size_t)T * (4 + (pcor ? 1 : 0) + (pnoise ? 1 : 0));
     std::vector<cudaEvent_t> ev(2 * nk, nullptr);
-    std::vector<int> fam(nk);
+    std::vector<int> fam(nk), kernels(nk);
+    // kernels of a noise block (filters and the check of an estimated interval),
+    // of a list rebuild and of a step's sweeps
+    const int noise_kernels = 2 + c->P.pn_deg + (c->P.pn_iv ? pn_spectrum_launches() : 0);
+    const int list_kernels = rebuild_in_cluster(c->P) ? 1 : 4, sweep_kernels = pnoise ? pair_noise_launches(c->P) : 0;
     gld_status s = GLD_OK;
     for (auto& e : ev)
         if (cudaEventCreate(&e) != cudaSuccess) s = fail(c, GLD_E_CUDA, "cudaEventCreate");
@@ -1623,27 +1628,27 @@ gld_status gld_profile_steps(gld_ctx* c, int64_t nsteps, double* ms, int64_t* la
             break;
         }
         size_t k = 0;
-        auto timed = [&](int f, auto&& launch) {
+        auto timed = [&](int f, int count, auto&& launch) {
             if (s != GLD_OK) return;
             fam[k] = f;
+            kernels[k] = count;
             if (cudaEventRecord(ev[2 * k], c->st) != cudaSuccess || launch() != cudaSuccess ||
                 cudaEventRecord(ev[2 * k + 1], c->st) != cudaSuccess)
                 s = fail(c, GLD_E_CUDA, "gld_profile_steps: launch failed");
             ++k;
         };
-        timed(GLD_PROF_NOISE, [&] { return launch_noise(c, c->st); });
+        timed(GLD_PROF_NOISE, noise_kernels, [&] { return launch_noise(c, c->st); });
         c->block_start = c->host_step;
         c->noise_end = c->host_step + T;
         c->noise_valid = true;
         for (int t = 0; t < T; ++t) {
-            timed(GLD_PROF_HIST, [&] {
-                return launch_memory(c, c->st);
-            });
-            if (pnoise) timed(GLD_PROF_PNOISE, [&] { return launch_pair_noise(c->P, c->B, c->d_zblk, c->d_bvec, c->st); });
-            timed(GLD_PROF_PAIR, [&] { return launch_pair_force_integrate(c->P, c->B, c->st); });
-            timed(GLD_PROF_CELL, [&] { return launch_rebuild(c->P, c->B, c->st); });
-            timed(GLD_PROF_CFORCE, [&] { return launch_cforce(c->P, c->B, 1, c->st); });  // with the VACF terms
-            if (pcor) timed(GLD_PROF_PCORR, [&] { return launch_pcorr(c->P, c->B, c->st); });
+            const bool parts = c->P.cblk && c->P.nmodes == 0 && t % c->conv_len == 0;
+            timed(GLD_PROF_HIST, 1 + (parts ? conv_pre_launches(c->P.nacc) : 0), [&] { return launch_memory(c, c->st); });
+            if (pnoise) timed(GLD_PROF_PNOISE, sweep_kernels, [&] { return launch_pair_noise(c->P, c->B, c->d_zblk, c->d_bvec, c->st); });
+            timed(GLD_PROF_PAIR, 1, [&] { return launch_pair_force_integrate(c->P, c->B, c->st); });
+            timed(GLD_PROF_CELL, list_kernels, [&] { return launch_rebuild(c->P, c->B, c->st); });
+            timed(GLD_PROF_CFORCE, 1, [&] { return launch_cforce(c->P, c->B, 1, c->st); });  // with the VACF terms
+            if (pcor) timed(GLD_PROF_PCORR, 1, [&] { return launch_pcorr(c->P, c->B, c->st); });
             c->last_fr_row = t;
             ++c->host_step;
         }
@@ -1655,11 +1660,7 @@ gld_status gld_profile_steps(gld_ctx* c, int64_t nsteps, double* ms, int64_t* la
                 break;
             }
             acc[fam[q]] += t;
-            const int pd = c->P.pn_deg;
-            cnt[fam[q]] += fam[q] == GLD_PROF_CELL     ? (rebuild_in_cluster(c->P) ? 1 : 4)
-                           : fam[q] == GLD_PROF_NOISE  ? 2 + pd
-                           : fam[q] == GLD_PROF_PNOISE ? pd
-                                                       : 1;
+            cnt[fam[q]] += kernels[q];
         }
     }
     for (auto& e : ev)

@@ -418,6 +418,9 @@ cudaError_t launch_batch_conv(const BatchPlan& bp, int step, cudaStream_t st)
 int batch_pre_tiles(int n_pad) { return (3 * n_pad / 2 + kPreThreads - 1) / kPreThreads; }
 static_assert(pre_streams(16, false) == 2 && pre_streams(8, true) == 2, "tiles of a batch");
 
+// (pairs of accumulators in one launch, an odd last one in another)
+int conv_pre_launches(int nacc) { return (nacc > 1) + (nacc & 1); }
+
 cudaError_t launch_conv_pre(const void* ring, int bf16, int n_pad, int m_max, const long long* nstep, const float* coef,
                             int nacc, float* part, int G, int len, int kahan, cudaStream_t st)
 {

@@ -2036,12 +2036,11 @@ cudaError_t launch_pcorr_flush(const StepParams& P, const ParticleBuffers& B, cu
 
 namespace {
 
-// The sweeps as one cooperative launch when all of its blocks are resident at
-// once with room for a typical particle's pairs; *done = false: they are not.
-cudaError_t pn_sweeps_launch(const StepParams& P, const ParticleBuffers& B, const float* zblk, float* bvec,
-                             cudaStream_t st, bool* done)
+// Room for pairs per thread with which all blocks of the sweeps' one
+// cooperative launch are resident at once; 0: a launch per sweep.
+cudaError_t pn_sweeps_room(const StepParams& P, int* found)
 {
-    *done = false;
+    *found = 0;
     if (P.perp || P.Qs > 0 || P.pn_deg < 2) return cudaSuccess;
     int dev = 0, sms = 0, coop = 0;
     cudaError_t e = cudaGetDevice(&dev);
@@ -2057,18 +2056,23 @@ cudaError_t pn_sweeps_launch(const StepParams& P, const ParticleBuffers& B, cons
     if ((e = allow_smem(pn_sweeps, smem)) != cudaSuccess) return e;
     int occ = 0;
     if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, pn_sweeps, kSweepThreads, smem)) != cudaSuccess) return e;
-    if (occ < per_sm) return cudaSuccess;
+    if (occ >= per_sm) *found = room;
+    return cudaSuccess;
+}
+
+cudaError_t pn_sweeps_launch(const StepParams& P, const ParticleBuffers& B, const float* zblk, float* bvec, int room,
+                             cudaStream_t st)
+{
     cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3((unsigned)grid);
+    cfg.gridDim = dim3((unsigned)((P.n + kSweepThreads - 1) / kSweepThreads));
     cfg.blockDim = dim3(kSweepThreads);
-    cfg.dynamicSmemBytes = smem;
+    cfg.dynamicSmemBytes = (size_t)20 * kSweepThreads * room;
     cfg.stream = st;
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeCooperative;
     at[0].val.cooperative = 1;
     cfg.attrs = at;
     cfg.numAttrs = 1;
-    *done = true;
     return cudaLaunchKernelEx(&cfg, pn_sweeps, P, B.ctrl, (const float4*)B.pos, (const int*)B.nbr, (const int*)B.nbr_cnt,
                               B.ftab, (const float*)B.frblock, zblk, bvec, room);
 }
@@ -2080,9 +2084,10 @@ cudaError_t launch_pair_noise(const StepParams& P, const ParticleBuffers& B, con
 {
     const int K = P.pn_deg;
     if (K <= 0) return cudaSuccess;
-    bool done = false;
-    cudaError_t e = pn_sweeps_launch(P, B, zblk, bvec, st, &done);
-    if (e != cudaSuccess || done) return e;
+    int room = 0;
+    cudaError_t e = pn_sweeps_room(P, &room);
+    if (e != cudaSuccess) return e;
+    if (room > 0) return pn_sweeps_launch(P, B, zblk, bvec, room, st);
     const unsigned grid = (unsigned)((P.n + kThreads - 1) / kThreads);
     for (int k = K - 1; k >= 0; --k) {
         pn_stage<<<grid, kThreads, 0, st>>>(P, B.ctrl, B.pos, B.nbr, B.nbr_cnt, B.ftab, B.fptab,
@@ -2091,6 +2096,14 @@ cudaError_t launch_pair_noise(const StepParams& P, const ParticleBuffers& B, con
     }
     return cudaSuccess;
 }
+
+int pair_noise_launches(const StepParams& P)
+{
+    int room = 0;
+    return pn_sweeps_room(P, &room) == cudaSuccess && room > 0 ? 1 : P.pn_deg;
+}
+
+int pn_spectrum_launches() { return 2 + 2 * kPnLanczosSteps; }
 
 int batch_nbr_tiles(int n) { return (n + kNbrGroups - 1) / kNbrGroups; }
 

@@ -32,6 +32,7 @@ constexpr int kMinBlockedSlots = 32;
 cudaError_t conv_block_shape(int bf16, int n_pad, int m_max, int nacc, int kahan, int* G, int* len, size_t* bytes);
 cudaError_t launch_conv_pre(const void* ring, int bf16, int n_pad, int m_max, const long long* nstep, const float* coef,
                             int nacc, float* part, int G, int len, int kahan, cudaStream_t st);
+int conv_pre_launches(int nacc);
 int batch_pre_tiles(int n_pad);
 int batch_nbr_tiles(int n);  // tiles of the list build (k_particles.cu)
 
@@ -93,6 +94,7 @@ cudaError_t launch_pcorr_flush(const StepParams& P, const ParticleBuffers& B, cu
 // recurrence (pn_deg neighbour sweeps); Z_0 rows are frblock's, Z_k (k >= 1)
 // rows of zblk[k - 1]; bvec holds three vectors [3][n_pad]; F replaces the
 // Z_0 row of step n in frblock.
+int pair_noise_launches(const StepParams& P);  // kernels of the call below
 cudaError_t launch_pair_noise(const StepParams& P, const ParticleBuffers& B, const float* zblk, float* bvec,
                               cudaStream_t st);
 // Extreme eigenvalues of the pair matrix M (as the Clenshaw sweeps apply it)
@@ -103,6 +105,7 @@ cudaError_t launch_pair_noise(const StepParams& P, const ParticleBuffers& B, con
 cudaError_t launch_pn_spectrum(const StepParams& P, const ParticleBuffers& B, float* vec, double* part, double* ab,
                                double lo, double hi, int check, double* out, cudaStream_t st);
 int pn_spectrum_blocks(const StepParams& P);
+int pn_spectrum_launches();
 // Pair-correlated noise by Algorithm 1 (k_pn_krylov.cu): vectors [3 n_pad][Mp]
 // (frequency fastest), Lanczos vectors unnormalised (R_k, v_k = R_k / beta_k).
 // kry_ft: the transformed white-noise window of step ctrl->step into V0
@@ -182,7 +185,7 @@ struct BatchPlan {
     int pn_kmax;     // the largest Chebyshev degree of the members' pair noise (0: none)
 };
 // step: number of the step in its 64-step block
-cudaError_t launch_batch_conv(const BatchPlan& bp, int step, cudaStream_t st);  // k_history.cu
+cudaError_t launch_batch_conv(const BatchPlan& bp, int step, cudaStream_t st);  // k_history_blk.cu
 cudaError_t launch_batch_particles(const BatchPlan& bp, cudaStream_t st); // k_particles.cu
 cudaError_t launch_batch_noise(const BatchPlan& bp, cudaStream_t st);     // k_noise.cu
 // Whole steps of small systems (k_cluster.cu): whether a system's features and
