@@ -173,14 +173,17 @@ class ClockSampler:
         return {"sm_mhz": statistics.median(sm), "sm_max_mhz": mx, "reasons": sorted(reasons), "samples": len(sm)}
 
 
-def conv_bytes(n: int, m_max: int, elem: int, nacc: int, kahan: bool, first: int, steps: int) -> float:
+def conv_bytes(n: int, m_max: int, elem: int, nacc: int, kahan: bool, first: int, steps: int, ranges: int,
+               length: int) -> float:
     """Bytes per step that the memory sums of steps first .. first + steps - 1
-    need in blocks of steps: the parts of a block read each range of ring rows up
-    to its first rewritten row, once for the block's 8 or 16 steps; a step reads
-    the rest of the ranges, reads its parts and writes its sums.  (One range from
-    about 80000 particles on, two from 40000, else four.)"""
-    H, ranges = m_max - 1, 1 if kahan or n > 80000 else 2 if n > 40000 else 4
-    length = 8 if kahan or ranges > 1 else 16
+    need in blocks of `length` steps that begin at the first one: the parts of a
+    block read each of the `ranges` of ring rows up to its first rewritten row,
+    once for all of its steps; a step reads the rest of the ranges, reads its
+    parts and writes its sums.  (GLD.diag tells both; length 0: no blocks, every
+    step reads the ring.)"""
+    H = m_max - 1
+    if length == 0:
+        return n * (elem * 3 * H + 4 * 3 * nacc)
     rows = parts = 0.0
     for k in range(first, first + steps):
         h0 = (first + (k - first) // length * length) % H
@@ -196,14 +199,19 @@ def conv_bytes(n: int, m_max: int, elem: int, nacc: int, kahan: bool, first: int
     return n * (elem * 3 * rows / steps + sums)
 
 
+CONV_SOURCES = ("history.cuh", "k_history.cu", "k_history_blk.cu")  # the kernels of the history convolution
+
+
 def kernel_source_hash() -> str:
-    src = os.path.join(ROOT, "paper_1808_00270_gb300", "csrc", "k_history.cu")
-    return hashlib.sha256(open(src, "rb").read()).hexdigest()[:16]
+    h = hashlib.sha256()
+    for name in CONV_SOURCES:
+        h.update(open(os.path.join(ROOT, "paper_1808_00270_gb300", "csrc", name), "rb").read())
+    return h.hexdigest()[:16]
 
 
 def measured_traffic(workload: str):
-    """DRAM bytes per launch of the history convolution from the committed ncu
-    summary, if it was taken on the current kernel source."""
+    """DRAM bytes per step of the history convolution from the committed ncu
+    summary, if it was taken on the current kernel sources."""
     path = os.path.join(PROFILES, "hist_conv_traffic.json")
     try:
         d = json.load(open(path))
@@ -211,7 +219,7 @@ def measured_traffic(workload: str):
         return None
     if d.get("kernel_source_sha256_16") != kernel_source_hash() or d.get("workload") != workload:
         return None
-    return d.get("dram_bytes_per_launch")
+    return d.get("dram_bytes_per_step")
 
 
 def peaks():
@@ -317,7 +325,8 @@ def batch_leg(args, rank: int, world: int, local: int, quiet: bool = False):
                       "n_range": [min(w.n for w in ws), max(w.n for w in ws)],
                       "m_max_set": sorted({w.m_max for w in ws}), "history_bytes": hist_bytes,
                       "parallelism": f"replicas{world}",
-                      "l2": f"inputs larger than L2: {hist_bytes / 1e9:.2f} GB of history rings streamed every step"},
+                      "l2": f"inputs larger than L2: {hist_bytes / 1e9:.2f} GB of history rings, streamed every step from the "
+                            "first row on that the step's block rewrites"},
            "sequential": {"value": seq, "unit": UNIT, "ms_per_step": ms_seq / K,
                           "what": "the same systems one after another, each gld_step(K) replaying its own graph"},
            "speedup_vs_sequential": value / seq,
@@ -328,7 +337,7 @@ def batch_leg(args, rank: int, world: int, local: int, quiet: bool = False):
                         "achieved": alg / (conv_ms / 1e3) / 1e9, "peak": peak, "unit": "GB/s",
                         "frac": alg / (conv_ms / 1e3) / 1e9 / peak, "peak_source": f"{peak_kind} hbm_gbs",
                         "traffic": None, "algorithmic_bytes_per_launch": alg, "avg_launch_ms": conv_ms},
-           "clocks": clk, "gpu_launches": (K // T) * (2 + T * 7 + T // (8 if args.kahan else 16))}
+           "clocks": clk, "gpu_launches": (K // T) * (2 + T * 8 + T // (8 if args.kahan else 16))}
     if rank == 0 and not quiet:
         print(json.dumps(out))
     for g in systems:
@@ -460,8 +469,10 @@ def main():
     if args.pair_noise_lanczos >= 0:
         cfg["pair_noise"] = {"lanczos_window": args.pair_noise_lanczos, "tol": 1e-6, "kmax": 24,
                              "pair_kernel_scale": 1.0}
+    ring_mb = (2 if args.hist == "bf16" else 4) * 3e-6 * (w.m_max - 1) * w.n
     cfg.update({"global_batch": w.n * world, "parallelism": f"replicas{world}",
-                "l2": "inputs larger than L2: 1.26 GB FP32 history ring streamed every step"})
+                "l2": f"inputs {'larger than' if ring_mb > 129 else 'within'} L2: history ring of {ring_mb:.1f} MB, "
+                      "streamed every step from the first row on that the step's block rewrites"})
     if args.skin > 0:
         cfg["skin"] = args.skin
 
@@ -551,26 +562,25 @@ def main():
         sim.set_pair_noise_lanczos(0.0)
         cfg["pair_noise"]["krylov_dimension"] = kdim
         cfg["pair_noise"]["kernel_profile"] = "without the pair noise"
-    prof_first = sim.step_index
     prof = sim.profile_steps(args.profile_steps)
-    h_ms, h_n = prof["hist_conv"]
-    nacc = 2
-    alg_bytes = conv_bytes(w.n, w.m_max, 2 if args.hist == "bf16" else 4, nacc, bool(args.kahan), prof_first,
-                           args.profile_steps)
+    h_ms, prof_steps = prof["hist_conv"][0], prof["cforce"][1]
+    nacc, blocked = 2, sim.diag()
+    alg_bytes = conv_bytes(w.n, w.m_max, 2 if args.hist == "bf16" else 4, nacc, bool(args.kahan),
+                           sim.step_index - prof_steps, prof_steps, blocked["conv_ranges"], blocked["conv_block"])
     kname, traffic = "history convolution (a step's sums and its share of the block's parts)", measured_traffic(args.workload)
     if args.modes:  # per column: Y' of every mode read and written, two ring values, the projections
         nm = len(inputs.memory_modes(w)[0])
         elem = 2 if args.hist == "bf16" else 4
         alg_bytes = 3 * ((w.n + 31) // 32 * 32) * (16 * nm + 2 * elem + 4 * nacc)
         kname, traffic = "modes_step", None
-    avg_s = h_ms / 1e3 / max(h_n, 1)
+    avg_s = h_ms / 1e3 / max(prof_steps, 1)
     achieved = alg_bytes / avg_s / 1e9
     peak, peak_kind = peaks()
     total_ms = sum(v[0] for v in prof.values())
     roofline = {"bound": "hbm", "kernel": kname, "achieved": achieved, "peak": peak, "unit": "GB/s",
                 "frac": achieved / peak, "peak_source": f"{peak_kind} hbm_gbs",
                 "traffic": traffic, "algorithmic_bytes_per_launch": alg_bytes,
-                "avg_launch_ms": avg_s * 1e3,
+                "avg_launch_ms": avg_s * 1e3,  # both per step: its own launch and its share of the block's parts
                 "kernel_share": {k: v[0] / total_ms for k, v in prof.items() if total_ms > 0}}
 
     diag = sim.diag()
@@ -579,21 +589,19 @@ def main():
                  // vacf["vacf_stride"]})
     T_blocks = (K + T - 1) // T
     # per step: convolution, pair kernel, F^C with the VACF terms, and the
-    # rebuild decision (conditional form) or the gated rebuild kernels (one up to
-    # 8192 particles, else four); per 8 or 16 steps the parts of the convolution
-    parts = 0 if args.modes else K // (16 if w.n > 80000 and not args.kahan else 8)
-    plain = not args.modes and args.pcorr <= 0 and args.pair_noise <= 0
+    # rebuild decision (conditional form) or the gated rebuild kernels; per block
+    # of steps the parts of the convolution
+    parts = 0 if args.modes or not blocked["conv_block"] else K // blocked["conv_block"]
     if d0["graph_mode"] == 2:  # rebuild kernels only on the steps that rebuild
         launches = K * 4 + 4 * (d1["rebuilds"] - d0["rebuilds"]) + 2 * T_blocks + parts
-    elif w.n <= 192 and plain and not args.kahan:  # a block of steps in one kernel
+    elif d1["cluster_steps"] - d0["cluster_steps"] == K:  # (a part of) a noise block of steps in one kernel
         launches = 3 * T_blocks
     else:
-        launches = K * (3 + (1 if w.n <= 8192 else 4)) + 2 * T_blocks + parts
+        launches = K * (3 + prof["cell_build"][1] // prof_steps) + 2 * T_blocks + parts
     if args.pcorr > 0:
         launches += K
     if args.pair_noise > 0:  # Clenshaw sweeps per step; filters and the Lanczos check per block
-        sweeps = 1 if w.n <= 152 * 8 * 128 else args.pair_noise  # one launch per step while it fits the chip
-        launches += sweeps * K + args.pair_noise * T_blocks + (2 + 2 * 32) * T_blocks
+        launches += prof["pair_noise"][1] // prof_steps * K + (prof["noise"][1] // (prof_steps // T) - 2) * T_blocks
     if args.pair_noise_lanczos >= 0:  # eager steps; per run: transform, norm, 4 launches per iteration, output
         iters = 4 * ((cfg["pair_noise"]["krylov_dimension"] + 3) // 4)
         runs = T_blocks if args.pair_noise_lanczos == 1 else K
