@@ -43,7 +43,6 @@ constexpr int kPairBatch = 4;                 // list entries per round of the o
 constexpr int kCforceLanes = kBatchCforceLanes;  // lanes per particle in the F^C kernel
 constexpr int kCellThreads = kBatchCellChunk;
 constexpr int kThreads = kBatchPartBlock;
-constexpr int kLanesMaxN = 22528;  // particles up to which the neighbour kernels take several lanes each
 constexpr int kNbrSortCap = 128;  // list entries sorted by id at each build
 static_assert(kBatchVacfBlock == kThreads, "vacf blocks share the particle block size");
 
@@ -1915,13 +1914,33 @@ cudaError_t launch_delay(unsigned long long ns, cudaStream_t st)
 
 namespace {
 
-// Lanes per particle of the neighbour kernels of a system alone: eight while
-// that is at most 1024 threads per SM, then four.  Pair kernel, us (events)
-// with eight / one: 8.4 / 12.2 at 4096 particles, 9.7 / 12.2 at 10007; general
-// form with eight / four / one 24.4 / 20.5 / 32.8 at 20000.  Above kLanesMaxN
-// one: with four / one 12.6 / 10.8 at 32768, with two / one 19.7 / 16.7 at
-// 65536, the shuffled additions cost more than they hide.
-int lanes_for(int n) { return n <= 1024 * 152 / 8 ? 8 : n <= kLanesMaxN ? 4 : 1; }
+// Lanes per particle of the neighbour kernels of a system alone: as many as stay
+// in one wave, all blocks resident at once.  Lanes shorten a particle's chain of
+// loads; a second wave costs more than they save.  (On 152 SMs the registers
+// leave 768 threads per SM to the one-term form with eight lanes and to the
+// general form, 512 to the one-term form with four and two, 1024 to F^C.)  us by
+// events at 11 neighbours in the list, eight / four / two / one lane:
+//   one term   8192: 9.7/10.4/11.2/14.6    12288: 10.0/10.0/11.8/15.1   16384: 12.7/10.2/11.8/15.3
+//             20000: 14.1/14.0/12.1/15.7   32768: 17.8/16.0/12.6/16.1   49152: 22.2/20.3/18.9/16.2
+//   general   12288: 16.3/18.3/24.3/30.7   16384: 23.7/18.4/24.4/31.3   24576: 25.1/20.4/26.2/31.9
+//             32768: 32.9/31.2/26.5/32.2   49152: 42.8/34.5/30.1/33.3   65536: 51.3/44.5/45.6/34.9
+// F^C, four / two / one: 8.7/9.8/10.4 at 8192, 10.6/10.1/11.4 at 32768, 13.7/11.7/11.9
+// at 49152; with the VACF, in blocks of 1024 threads, 14.8/15.5/16.1 at 32768 and
+// 20.2/16.2/16.4 at 49152.
+template <bool FAST>
+int pair_lanes_for(int n)
+{
+    auto fits = [&](auto kern, int lanes) { return (long long)n * lanes <= resident_threads(kern, kThreads); };
+    return fits(pair_lanes<FAST, 8>, 8) ? 8 : fits(pair_lanes<FAST, 4>, 4) ? 4 : fits(pair_lanes<FAST, 2>, 2) ? 2 : 1;
+}
+
+template <bool VACF>
+int cforce_lanes_for(int n)
+{
+    // (with the VACF, a block per 256 particles)
+    const long long threads = VACF ? (long long)((n + kThreads - 1) / kThreads) * kThreads * 4 : 4LL * n;
+    return threads <= resident_threads(cforce_lanes<4, VACF>, VACF ? 4 * kThreads : kThreads) ? 4 : 1;
+}
 
 template <bool FAST, int L>
 cudaError_t pair_lanes_launch(const StepParams& P, const ParticleBuffers& B, cudaStream_t st)
@@ -1949,8 +1968,12 @@ cudaError_t launch_pair_force_integrate(const StepParams& P, const ParticleBuffe
 {
     const unsigned grid = (unsigned)((P.n + kPairThreads - 1) / kPairThreads);
     const bool fast = P.Q == 1 && P.Qs == 0 && !P.perp;
-    if (lanes_for(P.n) == 8) return fast ? pair_lanes_launch<true, 8>(P, B, st) : pair_lanes_launch<false, 8>(P, B, st);
-    if (lanes_for(P.n) == 4) return fast ? pair_lanes_launch<true, 4>(P, B, st) : pair_lanes_launch<false, 4>(P, B, st);
+    switch (fast ? pair_lanes_for<true>(P.n) : pair_lanes_for<false>(P.n)) {
+    case 8: return fast ? pair_lanes_launch<true, 8>(P, B, st) : pair_lanes_launch<false, 8>(P, B, st);
+    case 4: return fast ? pair_lanes_launch<true, 4>(P, B, st) : pair_lanes_launch<false, 4>(P, B, st);
+    case 2: return fast ? pair_lanes_launch<true, 2>(P, B, st) : pair_lanes_launch<false, 2>(P, B, st);
+    default: break;
+    }
     auto k = fast ? pair_force_integrate<true> : pair_force_integrate<false>;
     const unsigned pgrid = fast ? (unsigned)(((long long)P.n * kPairLanes + kPairThreads - 1) / kPairThreads) : grid;
     k<<<pgrid, kPairThreads, 0, st>>>(P, B.ctrl, B.pos, B.perm, B.nbr, B.nbr_cnt, B.vel, B.fc,
@@ -1992,7 +2015,8 @@ cudaError_t launch_cforce(const StepParams& P, const ParticleBuffers& B, int mod
     const bool vac = mode && P.vacf_len > 0;
     if (vac && (P.n_os > kVacfMaxOrigins || (int)grid != B.vacf_gx)) return cudaErrorInvalidValue;
     // (four lanes: a block of 256 particles for the VACF has 1024 threads)
-    if (mode && lanes_for(P.n) > 1) return cforce_lanes_launch<4>(P, B, vac, st);
+    if (mode && (vac ? cforce_lanes_for<true>(P.n) : cforce_lanes_for<false>(P.n)) > 1)
+        return cforce_lanes_launch<4>(P, B, vac, st);
     auto k = mode ? (vac ? cforce<true, true> : cforce<true, false>) : cforce<false, false>;
     k<<<grid, kThreads, 0, st>>>(P, B.ctrl, B.pos_next, B.pos, B.perm, B.nbr, B.nbr_cnt, B.vhalf, B.vel, B.fc,
                                  B.fctab, B.vorig, B.vpartial, B.csum, B.ccnt, B.norig);

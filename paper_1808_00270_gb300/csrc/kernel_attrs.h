@@ -7,6 +7,7 @@
 // function, to the most that the device gives, and never lowered.
 #pragma once
 
+#include <map>
 #include <mutex>
 #include <set>
 #include <utility>
@@ -42,6 +43,26 @@ template <class... A>
 cudaError_t allow_smem(void (*kern)(A...), size_t smem, bool nonportable = false)
 {
     return allow_smem((const void*)kern, smem, nonportable);
+}
+
+// Threads of a kernel, in blocks of `block` without dynamic shared memory, that
+// the device holds at once (0: the question failed); asked once per device and
+// function.
+template <class... A>
+int resident_threads(void (*kern)(A...), int block)
+{
+    static std::mutex mu;
+    static std::map<std::pair<int, const void*>, int> known;
+    int dev = 0, sms = 0, blocks = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) return 0;
+    std::lock_guard<std::mutex> lock(mu);
+    const auto key = std::make_pair(dev, (const void*)kern);
+    const auto it = known.find(key);
+    if (it != known.end()) return it->second;
+    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks, kern, block, 0) != cudaSuccess)
+        return 0;
+    return known[key] = sms * blocks * block;
 }
 
 }  // namespace gld
