@@ -15,7 +15,6 @@
 #include <cmath>
 #include <cstdio>
 #include <cstring>
-#include <mutex>
 #include <numeric>
 #include <string>
 #include <vector>
@@ -24,6 +23,7 @@
 
 #include "cluster_fit.h"
 #include "ctx.h"
+#include "pinned_pool.h"
 
 using namespace gld;
 
@@ -128,59 +128,21 @@ gld_status upload_vec(gld_ctx* c, float4* dst, const double* src, bool wrap)
     return GLD_OK;
 }
 
-// Page-locked staging of results read back, kept for the next read of any
-// context (allocating it costs more than most reads): at most kPinnedKept bytes
-// are kept, the rest is freed when it is given back.
-struct Pinned {
-    char* p = nullptr;
-    size_t cap = 0;
-};
-constexpr size_t kPinnedKept = (size_t)64 << 20;
-std::mutex g_pinned_mu;
-std::vector<Pinned> g_pinned;
-
-Pinned take_pinned(size_t bytes)
-{
-    Pinned b;
-    {
-        std::lock_guard<std::mutex> lock(g_pinned_mu);
-        size_t best = g_pinned.size();
-        for (size_t k = 0; k < g_pinned.size(); ++k)
-            if (g_pinned[k].cap >= bytes && (best == g_pinned.size() || g_pinned[k].cap < g_pinned[best].cap)) best = k;
-        if (best < g_pinned.size()) {
-            b = g_pinned[best];
-            g_pinned.erase(g_pinned.begin() + (long)best);
-            return b;
-        }
-    }
-    b.cap = std::max(bytes, (size_t)1 << 16);
-    if (cudaHostAlloc((void**)&b.p, b.cap, cudaHostAllocPortable) != cudaSuccess) {
+// Staging of results read back, at most 64 MB kept while there are contexts.
+PinnedPool g_pinned(
+    [](size_t bytes) {
+        void* p = nullptr;
+        if (cudaHostAlloc(&p, bytes, cudaHostAllocPortable) == cudaSuccess) return p;
         cudaGetLastError();
-        b = Pinned{};
-    }
-    return b;
-}
-
-void give_pinned(Pinned b)
-{
-    if (!b.p) return;
-    {
-        std::lock_guard<std::mutex> lock(g_pinned_mu);
-        size_t kept = b.cap;
-        for (const Pinned& x : g_pinned) kept += x.cap;
-        if (kept <= kPinnedKept) {
-            g_pinned.push_back(b);
-            return;
-        }
-    }
-    cudaFreeHost(b.p);
-}
+        return (void*)nullptr;
+    },
+    [](void* p) { cudaFreeHost(p); }, (size_t)64 << 20);
 
 // Copies queued behind the context's work, then one wait for all of them and
 // for the device's error word.
 class Readback {
 public:
-    Readback(gld_ctx* ctx, size_t bytes) : c(ctx), pin(take_pinned(bytes + 256))
+    Readback(gld_ctx* ctx, size_t bytes) : c(ctx), pin(g_pinned.take(bytes + 256))
     {
         if (!pin.p) plain.resize(bytes + 256);
     }
@@ -188,7 +150,7 @@ public:
     {
         // an early return: no copy may land in staging that the next read takes
         if (queued) cudaStreamSynchronize(c->st);
-        give_pinned(pin);
+        g_pinned.give(pin);
     }
     Readback(const Readback&) = delete;
     Readback& operator=(const Readback&) = delete;
@@ -1039,11 +1001,12 @@ gld_status gld_create(const gld_params* p, const double* pos, const double* vel,
     gld_ctx* c = new gld_ctx();
     c->prm = *p;
     c->st = (cudaStream_t)p->stream;
+    g_pinned.enter();  // gld_destroy leaves
     if (cudaGetDevice(&c->device) != cudaSuccess ||
         cudaDeviceGetAttribute(&c->num_sms, cudaDevAttrMultiProcessorCount, c->device) != cudaSuccess ||
         cudaStreamCreateWithFlags(&c->cap, cudaStreamNonBlocking) != cudaSuccess ||
         cudaStreamCreateWithFlags(&c->cap2, cudaStreamNonBlocking) != cudaSuccess) {
-        delete c;
+        gld_destroy(c);
         return GLD_E_CUDA;
     }
     StepParams& P = c->P;
@@ -1061,9 +1024,7 @@ gld_status gld_create(const gld_params* p, const double* pos, const double* vel,
         for (int k = 0; k < p->n; ++k) {
             const int e = p->order[k];
             if (e < 0 || e >= p->n || seen[e]) {
-                cudaStreamDestroy(c->cap);
-                cudaStreamDestroy(c->cap2);
-                delete c;
+                gld_destroy(c);
                 return GLD_E_INVAL;
             }
             seen[e] = 1;
@@ -2496,6 +2457,7 @@ gld_status gld_destroy(gld_ctx* c)
     if (c->ev_fork) cudaEventDestroy(c->ev_fork);
     if (c->ev_join) cudaEventDestroy(c->ev_join);
     delete c;
+    g_pinned.leave();
     return GLD_OK;
 }
 
