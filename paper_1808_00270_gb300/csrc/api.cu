@@ -740,30 +740,34 @@ gld_status step_cluster(gld_ctx* c, int64_t k, bool boundary)
 // Replays a captured graph of `steps` steps from a block of the convolution's
 // first step (a noise block has begun, or begins in it).  An overlapped graph
 // starts from its first step's memory sums and the parts of their block.
-gld_status replay(gld_ctx* c, cudaGraphExec_t g, int steps)
+gld_status replay(gld_ctx* c, cudaGraphExec_t g, int steps, bool overlap)
 {
     if (c->P.cblk && c->part_step != c->host_step) c->conv_valid_step = -1;
-    if (c->overlap_graph) GLD_CUDA(c, launch_memory(c, c->st));
+    if (overlap) GLD_CUDA(c, launch_memory(c, c->st));
     GLD_CUDA(c, cudaGraphLaunch(g, c->st));
     c->host_step += steps;
-    c->conv_valid_step = c->overlap_graph ? c->host_step : -1;
-    c->part_step = c->overlap_graph && c->P.cblk ? c->host_step : -1;
+    c->conv_valid_step = overlap ? c->host_step : -1;
+    c->part_step = overlap && c->P.cblk ? c->host_step : -1;
     return GLD_OK;
 }
 
-// Captures `steps` steps (with a noise block before them) into *exec.
-bool capture_graph_mode(gld_ctx* c, bool conditional, int steps, bool noise, cudaGraphExec_t* exec)
+// The stream and events of the overlapped form; false: one could not be had.
+bool overlap_streams(gld_ctx* c)
+{
+    const bool ok = (c->cap3 || cudaStreamCreateWithFlags(&c->cap3, cudaStreamNonBlocking) == cudaSuccess) &&
+                    (c->ev_fork || cudaEventCreateWithFlags(&c->ev_fork, cudaEventDisableTiming) == cudaSuccess) &&
+                    (c->ev_join || cudaEventCreateWithFlags(&c->ev_join, cudaEventDisableTiming) == cudaSuccess);
+    if (!ok) cudaGetLastError();
+    return ok;
+}
+
+// Captures `steps` steps (with a noise block before them) into *exec; *overlapped
+// tells the form, which the two graphs of a context need not share.
+bool capture_graph_mode(gld_ctx* c, bool conditional, int steps, bool noise, cudaGraphExec_t* exec, bool* overlapped)
 {
     // the overlapped form needs an idempotent convolution (not the recursive
     // memory form, whose kernel advances its auxiliary sums)
-    bool overlap = c->P.nmodes == 0;
-    if (overlap && !c->cap3 &&
-        (cudaStreamCreateWithFlags(&c->cap3, cudaStreamNonBlocking) != cudaSuccess ||
-         cudaEventCreateWithFlags(&c->ev_fork, cudaEventDisableTiming) != cudaSuccess ||
-         cudaEventCreateWithFlags(&c->ev_join, cudaEventDisableTiming) != cudaSuccess)) {
-        cudaGetLastError();
-        overlap = false;
-    }
+    const bool overlap = c->P.nmodes == 0 && overlap_streams(c);
     cudaGraph_t g = nullptr;
     bool ok = cudaStreamBeginCapture(c->cap, cudaStreamCaptureModeThreadLocal) == cudaSuccess;
     if (ok) {
@@ -780,7 +784,7 @@ bool capture_graph_mode(gld_ctx* c, bool conditional, int steps, bool noise, cud
         cudaGetLastError();
         return false;
     }
-    c->overlap_graph = overlap;
+    *overlapped = overlap;
     return true;
 }
 
@@ -801,7 +805,7 @@ bool capture_segment(gld_ctx* c)
     if (c->gseg) return true;
     if (c->graph_failed || c->P.pn_kry || c->eager_steps < c->P.T) return false;
     const bool conditional = c->prm.use_graphs != 2 && c->P.n >= kConditionalMinN;
-    if (!capture_graph_mode(c, conditional, segment_steps(c), false, &c->gseg)) {
+    if (!capture_graph_mode(c, conditional, segment_steps(c), false, &c->gseg, &c->overlap_seg)) {
         c->graph_failed = true;
         return false;
     }
@@ -817,11 +821,11 @@ bool capture_graph(gld_ctx* c)
     // conditional rebuild for large systems; the gated kernels otherwise, and
     // as the fallback
     if (c->prm.use_graphs != 2 && c->P.n >= kConditionalMinN &&
-        capture_graph_mode(c, true, c->P.T, true, &c->gexec)) {
+        capture_graph_mode(c, true, c->P.T, true, &c->gexec, &c->overlap_exec)) {
         c->graph_mode = 2;
         return true;
     }
-    if (capture_graph_mode(c, false, c->P.T, true, &c->gexec)) {
+    if (capture_graph_mode(c, false, c->P.T, true, &c->gexec, &c->overlap_exec)) {
         c->graph_mode = 1;
         return true;
     }
@@ -1275,7 +1279,7 @@ gld_status gld_step(gld_ctx* c, int64_t nsteps)
         // smallest systems
         if (boundary && c->prm.use_graphs && nsteps >= T && !(cluster && c->P.n <= kClusterBlockMaxN) && capture_graph(c)) {
             c->block_start = c->host_step;
-            GLD_TRY(replay(c, c->gexec, T));
+            GLD_TRY(replay(c, c->gexec, T, c->overlap_exec));
             c->noise_end = c->host_step;
             c->noise_valid = true;
             c->last_fr_row = T - 1;
@@ -1297,7 +1301,7 @@ gld_status gld_step(gld_ctx* c, int64_t nsteps)
         }
         const int seg = segment_steps(c);
         if (c->prm.use_graphs && nsteps >= seg && (c->host_step - c->block_start) % seg == 0 && capture_segment(c)) {
-            GLD_TRY(replay(c, c->gseg, seg));
+            GLD_TRY(replay(c, c->gseg, seg, c->overlap_seg));
             c->last_fr_row = c->host_step - 1 - c->block_start;
             nsteps -= seg;
             continue;

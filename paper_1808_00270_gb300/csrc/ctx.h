@@ -22,7 +22,7 @@ struct gld_ctx {
     cudaStream_t cap2 = nullptr; // fills the bodies of conditional graph nodes
     cudaStream_t cap3 = nullptr; // the overlapped next-step convolution of the graph
     cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
-    bool overlap_graph = false;  // the graph computes each step's successor convolution
+    bool overlap_exec = false, overlap_seg = false;  // gexec, gseg compute each step's successor convolution
     long long conv_valid_step = -1;  // the step whose projections `conv` already holds
     cudaGraphExec_t gseg = nullptr;  // a piece of a noise block (without the noise)
     long long eager_steps = 0;       // steps launched kernel by kernel since the graphs were dropped
