@@ -2685,9 +2685,10 @@ cudaError_t batch_launch_block(gld_batch* b, cudaStream_t s)
     return e;
 }
 
-// Times each convolution schedule on the current composition (the
-// convolution only reads the rings and rewrites the projections, so repeating
-// it leaves the state unchanged) and keeps the fastest.
+// Times each convolution schedule on the current composition and keeps the
+// fastest.  The convolution only reads the rings; the parts and projections it
+// rewrites are not those of a step to come (gld_batch_step forgets the members'),
+// and the block that follows forms its own.
 gld_status batch_autotune(gld_batch* b)
 {
     cudaEvent_t e0, e1;
@@ -2823,6 +2824,8 @@ gld_status gld_batch_step(gld_batch* b, int64_t nsteps)
             return bfail(b, GLD_E_STATE, "gld_batch_step: a member left its noise-block boundary");
     }
     for (gld_ctx* c : b->members) {
+        // timing the schedules and the block below rewrite the sums and the parts
+        c->conv_valid_step = c->part_step = -1;
         const gld_status st = ring_form(c, false, b->st);
         if (st != GLD_OK) return bfail(b, st, "gld_batch_step: the white-noise ring of a member");
     }
@@ -2839,7 +2842,6 @@ gld_status gld_batch_step(gld_batch* b, int64_t nsteps)
         const cudaError_t e = b->gexec ? cudaGraphLaunch(b->gexec, b->st) : batch_launch_block(b, b->st);
         if (e != cudaSuccess) return bfail(b, GLD_E_CUDA, std::string("gld_batch_step: ") + cudaGetErrorString(e));
         for (gld_ctx* c : b->members) {
-            c->conv_valid_step = c->part_step = -1;
             c->block_start = c->host_step;
             c->host_step += kMaxNoiseBlock;
             c->noise_end = c->host_step;
