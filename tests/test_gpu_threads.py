@@ -1,5 +1,6 @@
-"""Dynamic shared memory of the kernels is allowed per function, not per launch:
-what one system asks for must not take it from another (needs a GPU)."""
+"""Systems of several host threads and streams do not get in each other's way: the
+dynamic shared memory allowed per function, and grids that wait for all of their
+blocks (needs a GPU)."""
 import threading
 
 import numpy as np
@@ -71,3 +72,41 @@ def test_two_threads_step_systems_of_their_own(sizes):
         for rep in range(3):
             for x, y in zip(out[("alone", k), 0], out[("both", k), rep]):
                 assert np.array_equal(x, y)
+
+
+def test_two_threads_with_pair_noise():
+    """The sweeps are one launch whose blocks wait for each other (a bounded wait),
+    and each system's fill the chip: two of them, on streams of their own, one
+    step and one wait at a time, give the results of one after the other."""
+    from paper_1808_00270_gb300 import GLD, inputs
+    w = inputs.Workload("pn", n=32768, box=inputs.box_for_density(32768, 0.05), m_max=128, dt=0.005, r_c=2.0, tau_s=0.5,
+                        tau_p=0.3, steps=1, seed=5)
+    errors, out = [], {}
+
+    def work(key):
+        try:
+            torch.cuda.set_device(0)
+            with torch.cuda.stream(torch.cuda.Stream()):
+                g = make_gpu(w, torch_allocator=False, pair=False)
+                gk, f, dr = inputs.pair_kernel_tables(w)
+                g.set_kernels(inputs.self_kernel_samples(w), g=gk, f=0.2 * f, dr=dr)
+                g.set_pair_noise(2, lam=2.0)
+                for _ in range(400):
+                    g.step(1)
+                    g.sync()
+                out[key] = g.get_state()
+                g.close()
+        except Exception as e:  # noqa: BLE001
+            errors.append(repr(e))
+
+    work("alone")
+    assert not errors, errors
+    threads = [threading.Thread(target=work, args=(k,)) for k in range(2)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not errors, errors
+    for k in range(2):
+        for x, y in zip(out["alone"], out[k]):
+            assert np.array_equal(x, y)
