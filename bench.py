@@ -312,7 +312,7 @@ def batch_leg(args, rank: int, world: int, local: int, quiet: bool = False):
     seq = world * n_tot * K / (ms_seq / 1e3)
     elem = 2 if args.hist == "bf16" else 4
     alg = sum((elem * 3 * (w.m_max - 1) + 4 * 3 * 2) * w.n for w in ws)
-    # (timed before the first step, where a step still streams its whole ring)
+    # (the schedules are timed on whole sums)
     conv_ms = info["schedule_ms"][info["schedule"]]
     peak, peak_kind = peaks()
     hist_bytes = sum(elem * 3 * (w.m_max - 1) * ((w.n + 31) // 32 * 32) for w in ws)
@@ -333,7 +333,7 @@ def batch_leg(args, rank: int, world: int, local: int, quiet: bool = False):
            "autotune": {"schedule": info["schedule"], "schedule_ms": info["schedule_ms"],
                         "schedules": ["256-column tiles, longest memory first", "128-column tiles, longest first",
                                       "256-column tiles, member order", "one block per system"]},
-           "roofline": {"bound": "hbm", "kernel": "b_conv (batched history convolution)",
+           "roofline": {"bound": "hbm", "kernel": "b_conv (batched history convolution, whole sums)",
                         "achieved": alg / (conv_ms / 1e3) / 1e9, "peak": peak, "unit": "GB/s",
                         "frac": alg / (conv_ms / 1e3) / 1e9 / peak, "peak_source": f"{peak_kind} hbm_gbs",
                         "traffic": None, "algorithmic_bytes_per_launch": alg, "avg_launch_ms": conv_ms},

@@ -467,8 +467,8 @@ gld_status gld_batch_step(gld_batch* batch, int64_t nsteps);
 /* Waits, then returns the first latched error of the members. */
 gld_status gld_batch_sync(gld_batch* batch);
 /* members, chosen convolution schedule (-1 before the first step), and the
- * timed milliseconds of the four schedules (one step's convolution at the
- * members' position in their rings); pointers may be NULL. */
+ * timed milliseconds of the four schedules (one step's convolution over whole
+ * rings); pointers may be NULL. */
 gld_status gld_batch_info(gld_batch* batch, int32_t* members, int32_t* schedule, double* schedule_ms);
 /* policy 0 (default): re-time the schedules whenever the members change;
  * 1: re-time only when the total number of convolution columns has moved by

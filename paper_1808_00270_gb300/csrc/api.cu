@@ -2686,9 +2686,10 @@ cudaError_t batch_launch_block(gld_batch* b, cudaStream_t s)
 }
 
 // Times each convolution schedule on the current composition and keeps the
-// fastest.  The convolution only reads the rings; the parts and projections it
-// rewrites are not those of a step to come (gld_batch_step forgets the members'),
-// and the block that follows forms its own.
+// fastest: whole sums, whose time does not depend on where in their rings the
+// members are (a resumed step streams any part of a ring, from all to nothing).
+// The convolution only reads the rings and rewrites the projections, which the
+// block that follows forms again.
 gld_status batch_autotune(gld_batch* b)
 {
     cudaEvent_t e0, e1;
@@ -2699,9 +2700,8 @@ gld_status batch_autotune(gld_batch* b)
     for (int sc = 0; sc < 4; ++sc) {
         GLD_TRY(batch_plan(b, sc));
         float ms = 0.f;
-        // (step 0 of a block forms its parts; step 1 is what most steps launch)
-        bool ok = launch_batch_conv(b->plan, 0, b->st) == cudaSuccess && cudaEventRecord(e0, b->st) == cudaSuccess;
-        for (int r = 0; r < 5 && ok; ++r) ok = launch_batch_conv(b->plan, 1, b->st) == cudaSuccess;
+        bool ok = launch_batch_conv(b->plan, -1, b->st) == cudaSuccess && cudaEventRecord(e0, b->st) == cudaSuccess;
+        for (int r = 0; r < 5 && ok; ++r) ok = launch_batch_conv(b->plan, -1, b->st) == cudaSuccess;
         ok = ok && cudaEventRecord(e1, b->st) == cudaSuccess && cudaEventSynchronize(e1) == cudaSuccess &&
              cudaEventElapsedTime(&ms, e0, e1) == cudaSuccess;
         if (!ok) {
@@ -2824,7 +2824,7 @@ gld_status gld_batch_step(gld_batch* b, int64_t nsteps)
             return bfail(b, GLD_E_STATE, "gld_batch_step: a member left its noise-block boundary");
     }
     for (gld_ctx* c : b->members) {
-        // timing the schedules and the block below rewrite the sums and the parts
+        // timing the schedules and the block below rewrite the projections and the parts
         c->conv_valid_step = c->part_step = -1;
         const gld_status st = ring_form(c, false, b->st);
         if (st != GLD_OK) return bfail(b, st, "gld_batch_step: the white-noise ring of a member");

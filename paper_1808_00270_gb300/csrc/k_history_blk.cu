@@ -401,7 +401,7 @@ cudaError_t launch_hist_conv_part(const Shape& sh, int nacc, int kahan, const vo
 cudaError_t launch_batch_conv(const BatchPlan& bp, int step, cudaStream_t st)
 {
     if (!bp.n_conv) return cudaSuccess;
-    const int len = pre_len(bp.kahan, 1), t = step % len;
+    const int len = pre_len(bp.kahan, 1), t = step < 0 ? -1 : step % len;
     if (bp.n_pre && t == 0) {
         const cudaError_t e = by_pre(bp.nacc, bp.kahan, bp.bf16, len, [&](auto na, auto ln, auto ka, auto bf, int a0, int p) {
             return b_pre_launch<decltype(na)::value, decltype(ln)::value, decltype(ka)::value, decltype(bf)::value>(

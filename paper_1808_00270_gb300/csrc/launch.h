@@ -184,7 +184,7 @@ struct BatchPlan {
     int pair_fast;   // every member has one pair term and no self-difference term
     int pn_kmax;     // the largest Chebyshev degree of the members' pair noise (0: none)
 };
-// step: number of the step in its 64-step block
+// step: number of the step in its 64-step block (-1: whole sums, without parts)
 cudaError_t launch_batch_conv(const BatchPlan& bp, int step, cudaStream_t st);  // k_history_blk.cu
 cudaError_t launch_batch_particles(const BatchPlan& bp, cudaStream_t st); // k_particles.cu
 cudaError_t launch_batch_noise(const BatchPlan& bp, cudaStream_t st);     // k_noise.cu
