@@ -189,13 +189,16 @@ cudaError_t launch_batch_conv(const BatchPlan& bp, int step, cudaStream_t st);  
 cudaError_t launch_batch_particles(const BatchPlan& bp, cudaStream_t st); // k_particles.cu
 cudaError_t launch_batch_noise(const BatchPlan& bp, cudaStream_t st);     // k_noise.cu
 // Whole steps of small systems (k_cluster.cu): whether a system's features and
-// size allow it and the device can hold its cluster; a system alone for nsteps steps of its noise block (rel0:
-// number of the first step in its block of the convolution, > 0: that block's
-// parts are formed; G and len as conv_block_shape).
-// Sizes (us per step, cluster against the graph of the step kernels): a whole
-// noise block 7.2 / 10.7 at 64 particles, 10.5 / 10.4 at 200, 11.8 / 10.7 at 512;
-// launched for single steps 20.2 / 30.9 at 1000, 23.7 / 31.0 at 2048, 27.4 / 30.4
-// at 4096.
+// size allow it and the device can hold its cluster; a system alone for nsteps
+// steps of its noise block (rel0: number of the first step in its block of the
+// convolution, > 0: that block's parts are formed; G and len as conv_block_shape).
+// Sizes, in us per step, cluster / step kernels.  A whole noise block, against the
+// graph: 7.2 / 9.3 at 64 particles, 10.5 / 10.4 at 200, 11.8 / 10.7 at 512.  Parts of
+// a block (m_max = 200) in calls of one and of four steps, against single
+// launches: 16.9, 13.3 / 23.3 at 256, 20.8, 16.9 / 24.3 at 2048, 24.0, 19.9 / 25.3 at
+// 4096, and 27.5, 23.3 / 27.3 there with m_max = 400.  Calls of eight steps and more
+// take the cluster too; replayed pieces of a block are faster for those above
+// kClusterBlockMaxN: 12.7 / 11.7 at 256, 16.3 / 12.4 at 2048, 19.2 / 13.5 at 4096.
 constexpr int kClusterMaxN = 4096;
 constexpr int kClusterBlockMaxN = 192;
 bool cluster_ok(const StepParams& P, int kahan);
