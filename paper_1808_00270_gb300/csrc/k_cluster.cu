@@ -218,122 +218,122 @@ __device__ __forceinline__ void cl_rebuild(const StepParams& P, const ParticleBu
         if (ncta == 1) __syncthreads();
         else cluster_barrier();
     };
-                // particles counted into cells; their rank in the cell
-                for (int i = g0; i < n; i += cthreads)
-                    B.cell_next[i] = atomicAdd(B.cell_count + cell_of(ld4(nxt + i), P), 1);
-                if (g0 == 0) ctrl->rebuilds += 1;
-                barrier();
-                // starts within the CTA's 2^shift cells, and the CTA's total
-                const int c0 = rank << shift, c1 = min(B.ncells, c0 + (1 << shift));
-                int run = 0;
-                for (int cb = c0; cb < c0 + (1 << shift); cb += kClThreads) {  // uniform over the CTA
-                    const int c = cb + tid, k = c < c1 ? ldi(B.cell_count + c) : 0;
-                    int excl;
-                    const int tot = cl_scan(k, &excl);
-                    if (c < c1) {
-                        B.cell_start[c] = run + excl;
-                        B.cell_count[c] = 0;
+    // particles counted into cells; their rank in the cell
+    for (int i = g0; i < n; i += cthreads)
+        B.cell_next[i] = atomicAdd(B.cell_count + cell_of(ld4(nxt + i), P), 1);
+    if (g0 == 0) ctrl->rebuilds += 1;
+    barrier();
+    // starts within the CTA's 2^shift cells, and the CTA's total
+    const int c0 = rank << shift, c1 = min(B.ncells, c0 + (1 << shift));
+    int run = 0;
+    for (int cb = c0; cb < c0 + (1 << shift); cb += kClThreads) {  // uniform over the CTA
+        const int c = cb + tid, k = c < c1 ? ldi(B.cell_count + c) : 0;
+        int excl;
+        const int tot = cl_scan(k, &excl);
+        if (c < c1) {
+            B.cell_start[c] = run + excl;
+            B.cell_count[c] = 0;
+        }
+        run += tot;
+    }
+    if (tid == 0) B.chunk_sum[rank] = run;
+    barrier();
+    if (tid < 32) {  // particles in earlier CTAs' cells
+        int v = tid < ncta ? ldi(B.chunk_sum + tid) : 0, x = v;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int y = __shfl_up_sync(0xffffffffu, x, o);
+            if (tid >= o) x += y;
+        }
+        if (tid < ncta) cbase[tid] = x - v;
+    }
+    __syncthreads();
+    auto start = [&](int c) { return c < B.ncells ? ldi(B.cell_start + c) + cbase[c >> shift] : n; };
+    for (int i = g0; i < n; i += cthreads) {
+        const float4 x = ld4(nxt + i);
+        B.pos_sorted[start(cell_of(x, P)) + B.cell_next[i]] = make_float4(x.x, x.y, x.z, __int_as_float(i));
+    }
+    barrier();
+    // a row of three cells along x is one range of particles, or two at
+    // the box's faces; lane l takes the rows l, l + L, ... of the nine
+    // (one cell: its particles l, l + L, ...); candidates meet in shared
+    // memory and go to the place of their id's rank
+    int* list = lists + grp * P.maxnb;
+    for (int it = 0; it < iters; ++it) {
+        const int i = p0 + it * pstride;
+        if (i >= n) break;  // uniform over the lanes of a particle
+        if (lane == 0) lcnt[grp] = 0;
+        __syncwarp(gmask);
+        const float4 pi = ld4(nxt + i);
+        const int nc = P.nc;
+        auto test = [&](const float4 pj) {
+            const int jd = __float_as_int(pj.w);
+            const float dx = min_image(pi.x, pj.x, P.box, P.half_box);
+            const float dy = min_image(pi.y, pj.y, P.box, P.half_box);
+            const float dz = min_image(pi.z, pj.z, P.box, P.half_box);
+            if (jd != i && dist2(dx, dy, dz) < P.rl2) {
+                const int k = atomicAdd(lcnt + grp, 1);
+                if (k < P.maxnb) list[k] = jd;
+            }
+        };
+        if (nc == 1) {
+            for (int q = lane; q < n; q += L) test(ld4(B.pos_sorted + q));
+        } else {
+            constexpr int R = (9 + L - 1) / L;  // rows of a lane
+            const int cx = cell_coord(pi.x, P.inv_cell, nc), cy = cell_coord(pi.y, P.inv_cell, nc),
+                      cz = cell_coord(pi.z, P.inv_cell, nc);
+            int b0[R], n0[R], b1[R], n1[R];
+#pragma unroll
+            for (int r = 0; r < R; ++r) {
+                const int o = lane + r * L;
+                int z = cz + o / 3 - 1, y = cy + o % 3 - 1;
+                z = z < 0 ? z + nc : (z >= nc ? z - nc : z);
+                y = y < 0 ? y + nc : (y >= nc ? y - nc : y);
+                const int base = (z * nc + y) * nc;
+                const int xa = max(cx - 1, 0), xb = min(cx + 1, nc - 1);       // the row inside the box
+                const int xw = cx == 0 ? nc - 1 : cx == nc - 1 ? 0 : -1;       // the cell across a face
+                b0[r] = n0[r] = b1[r] = n1[r] = 0;
+                if (o < 9) {
+                    b0[r] = start(base + xa);
+                    n0[r] = start(base + xb + 1) - b0[r];
+                    if (xw >= 0) {
+                        b1[r] = start(base + xw);
+                        n1[r] = start(base + xw + 1) - b1[r];
                     }
-                    run += tot;
                 }
-                if (tid == 0) B.chunk_sum[rank] = run;
-                barrier();
-                if (tid < 32) {  // particles in earlier CTAs' cells
-                    int v = tid < ncta ? ldi(B.chunk_sum + tid) : 0, x = v;
-    #pragma unroll
-                    for (int o = 1; o < 32; o <<= 1) {
-                        const int y = __shfl_up_sync(0xffffffffu, x, o);
-                        if (tid >= o) x += y;
+            }
+#pragma unroll
+            for (int r = 0; r < R; ++r)
+                for (int q = 0; q < n0[r] + n1[r]; q += 4) {
+                    float4 pj[4];
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) {
+                        const int k = q + u < n0[r] + n1[r] ? q + u : q;
+                        pj[u] = ld4(B.pos_sorted + (k < n0[r] ? b0[r] + k : b1[r] + k - n0[r]));
                     }
-                    if (tid < ncta) cbase[tid] = x - v;
+#pragma unroll
+                    for (int u = 0; u < 4; ++u)
+                        if (q + u < n0[r] + n1[r]) test(pj[u]);
                 }
-                __syncthreads();
-                auto start = [&](int c) { return c < B.ncells ? ldi(B.cell_start + c) + cbase[c >> shift] : n; };
-                for (int i = g0; i < n; i += cthreads) {
-                    const float4 x = ld4(nxt + i);
-                    B.pos_sorted[start(cell_of(x, P)) + B.cell_next[i]] = make_float4(x.x, x.y, x.z, __int_as_float(i));
-                }
-                barrier();
-                // a row of three cells along x is one range of particles, or two at
-                // the box's faces; lane l takes the rows l, l + L, ... of the nine
-                // (one cell: its particles l, l + L, ...); candidates meet in shared
-                // memory and go to the place of their id's rank
-                int* list = lists + grp * P.maxnb;
-                for (int it = 0; it < iters; ++it) {
-                    const int i = p0 + it * pstride;
-                    if (i >= n) break;  // uniform over the lanes of a particle
-                    if (lane == 0) lcnt[grp] = 0;
-                    __syncwarp(gmask);
-                    const float4 pi = ld4(nxt + i);
-                    const int nc = P.nc;
-                    auto test = [&](const float4 pj) {
-                        const int jd = __float_as_int(pj.w);
-                        const float dx = min_image(pi.x, pj.x, P.box, P.half_box);
-                        const float dy = min_image(pi.y, pj.y, P.box, P.half_box);
-                        const float dz = min_image(pi.z, pj.z, P.box, P.half_box);
-                        if (jd != i && dist2(dx, dy, dz) < P.rl2) {
-                            const int k = atomicAdd(lcnt + grp, 1);
-                            if (k < P.maxnb) list[k] = jd;
-                        }
-                    };
-                    if (nc == 1) {
-                        for (int q = lane; q < n; q += L) test(ld4(B.pos_sorted + q));
-                    } else {
-                        constexpr int R = (9 + L - 1) / L;  // rows of a lane
-                        const int cx = cell_coord(pi.x, P.inv_cell, nc), cy = cell_coord(pi.y, P.inv_cell, nc),
-                                  cz = cell_coord(pi.z, P.inv_cell, nc);
-                        int b0[R], n0[R], b1[R], n1[R];
-    #pragma unroll
-                        for (int r = 0; r < R; ++r) {
-                            const int o = lane + r * L;
-                            int z = cz + o / 3 - 1, y = cy + o % 3 - 1;
-                            z = z < 0 ? z + nc : (z >= nc ? z - nc : z);
-                            y = y < 0 ? y + nc : (y >= nc ? y - nc : y);
-                            const int base = (z * nc + y) * nc;
-                            const int xa = max(cx - 1, 0), xb = min(cx + 1, nc - 1);       // the row inside the box
-                            const int xw = cx == 0 ? nc - 1 : cx == nc - 1 ? 0 : -1;       // the cell across a face
-                            b0[r] = n0[r] = b1[r] = n1[r] = 0;
-                            if (o < 9) {
-                                b0[r] = start(base + xa);
-                                n0[r] = start(base + xb + 1) - b0[r];
-                                if (xw >= 0) {
-                                    b1[r] = start(base + xw);
-                                    n1[r] = start(base + xw + 1) - b1[r];
-                                }
-                            }
-                        }
-    #pragma unroll
-                        for (int r = 0; r < R; ++r)
-                            for (int q = 0; q < n0[r] + n1[r]; q += 4) {
-                                float4 pj[4];
-    #pragma unroll
-                                for (int u = 0; u < 4; ++u) {
-                                    const int k = q + u < n0[r] + n1[r] ? q + u : q;
-                                    pj[u] = ld4(B.pos_sorted + (k < n0[r] ? b0[r] + k : b1[r] + k - n0[r]));
-                                }
-    #pragma unroll
-                                for (int u = 0; u < 4; ++u)
-                                    if (q + u < n0[r] + n1[r]) test(pj[u]);
-                            }
-                    }
-                    __syncwarp(gmask);
-                    int c = lcnt[grp];
-                    if (c > P.maxnb) {
-                        if (lane == 0) atomicOr(&ctrl->err, kErrNbrOverflow);
-                        c = P.maxnb;
-                    }
-                    for (int s = lane; s < c; s += L) {
-                        const int v = list[s];
-                        int r = 0;
-                        for (int k = 0; k < c; ++k) r += list[k] < v;
-                        B.nbr[(size_t)r * np + i] = v;
-                    }
-                    if (lane == 0) {
-                        B.nbr_cnt[i] = c;
-                        B.disp_build[i] = ld4(B.disp + i);
-                    }
-                    __syncwarp(gmask);  // the scratch is read before the next particle's; the lists before the forces
-                }
+        }
+        __syncwarp(gmask);
+        int c = lcnt[grp];
+        if (c > P.maxnb) {
+            if (lane == 0) atomicOr(&ctrl->err, kErrNbrOverflow);
+            c = P.maxnb;
+        }
+        for (int s = lane; s < c; s += L) {
+            const int v = list[s];
+            int r = 0;
+            for (int k = 0; k < c; ++k) r += list[k] < v;
+            B.nbr[(size_t)r * np + i] = v;
+        }
+        if (lane == 0) {
+            B.nbr_cnt[i] = c;
+            B.disp_build[i] = ld4(B.disp + i);
+        }
+        __syncwarp(gmask);  // the scratch is read before the next particle's; the lists before the forces
+    }
 }
 
 // Two adjacent streams of a ring row.

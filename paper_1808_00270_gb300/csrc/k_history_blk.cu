@@ -366,14 +366,14 @@ cudaError_t part_launch(const Shape& sh, const void* ring, int n_pad, int M, con
     // / narrower: 20.3 / 12.3 at 4096 particles in BF16, 29.9 / 20.0 at 10007 and
     // 48.2 / 42.5 at 50000 in FP32, 68.3 / 58.6 at 100003 in BF16; above it
     // 68.8 / 75.4 at 100003 in FP32).
-    if (sh.kind == 0 && !(KAHAN && bytes / 16 < 384LL * 152)) {
+    if (sh.kind == 0 && !(KAHAN && bytes / 16 < 384LL * kChipSms)) {
         auto k = hist_conv_col<NACC, KAHAN, BF16, true>;
         const cudaError_t e = allow_smem(k, smem);
         if (e != cudaSuccess) return e;
         k<<<sh.grid, sh.block, smem, st>>>((const typename Col<BF16>::V*)ring, 3LL * n_pad / Col<BF16>::W, H, coef, M,
                                            nstep, step, out, bp);
     } else {
-        const int vb = bytes / 16 >= 512LL * 152 ? 16 : bytes / 8 >= 512LL * 152 ? 8 : 4;
+        const int vb = bytes / 16 >= 512LL * kChipSms ? 16 : bytes / 8 >= 512LL * kChipSms ? 8 : 4;
         auto k = vb == 16 ? conv_tail<NACC, KAHAN, BF16, 16>
                           : vb == 8 ? conv_tail<NACC, KAHAN, BF16, 8> : conv_tail<NACC, KAHAN, BF16, 4>;
         const cudaError_t e = allow_smem(k, smem);

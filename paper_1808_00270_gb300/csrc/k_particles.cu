@@ -566,78 +566,78 @@ __device__ __forceinline__ void nbr_lanes_body(const StepParams& P, Ctrl* ctrl, 
     // (a grid of at most six blocks per SM: a launch that finds nothing to do
     // costs by its blocks)
     for (int k = blk * kNbrGroups + grp; k < P.n; k += nblk * kNbrGroups) {  // uniform over the lanes of a particle
-    const float4 pi = pos_sorted[k];
-    const int id = __float_as_int(pi.w), nc = P.nc;
-    int* list = lists + grp * P.maxnb;
-    if (lane == 0) lcnt[grp] = 0;
-    __syncwarp(gmask);
-    auto test = [&](const float4 pj) {
-        const int jd = __float_as_int(pj.w);
-        const float dx = min_image(pi.x, pj.x, P.box, P.half_box);
-        const float dy = min_image(pi.y, pj.y, P.box, P.half_box);
-        const float dz = min_image(pi.z, pj.z, P.box, P.half_box);
-        if (jd != id && dist2(dx, dy, dz) < P.rl2) {
-            const int c = atomicAdd(lcnt + grp, 1);
-            if (c < P.maxnb) list[c] = jd;
-        }
-    };
-    if (nc == 1) {
-        for (int q = lane; q < P.n; q += L) test(__ldg(pos_sorted + q));
-    } else {
-        const int cx = cell_coord(pi.x, P.inv_cell, nc), cy = cell_coord(pi.y, P.inv_cell, nc),
-                  cz = cell_coord(pi.z, P.inv_cell, nc);
-        const int xa = max(cx - 1, 0), xb = min(cx + 1, nc - 1);  // the row inside the box
-        const int xw = cx == 0 ? nc - 1 : cx == nc - 1 ? 0 : -1;  // the cell across a face
-        int b0[R], n0[R], b1[R], n1[R];
+        const float4 pi = pos_sorted[k];
+        const int id = __float_as_int(pi.w), nc = P.nc;
+        int* list = lists + grp * P.maxnb;
+        if (lane == 0) lcnt[grp] = 0;
+        __syncwarp(gmask);
+        auto test = [&](const float4 pj) {
+            const int jd = __float_as_int(pj.w);
+            const float dx = min_image(pi.x, pj.x, P.box, P.half_box);
+            const float dy = min_image(pi.y, pj.y, P.box, P.half_box);
+            const float dz = min_image(pi.z, pj.z, P.box, P.half_box);
+            if (jd != id && dist2(dx, dy, dz) < P.rl2) {
+                const int c = atomicAdd(lcnt + grp, 1);
+                if (c < P.maxnb) list[c] = jd;
+            }
+        };
+        if (nc == 1) {
+            for (int q = lane; q < P.n; q += L) test(__ldg(pos_sorted + q));
+        } else {
+            const int cx = cell_coord(pi.x, P.inv_cell, nc), cy = cell_coord(pi.y, P.inv_cell, nc),
+                      cz = cell_coord(pi.z, P.inv_cell, nc);
+            const int xa = max(cx - 1, 0), xb = min(cx + 1, nc - 1);  // the row inside the box
+            const int xw = cx == 0 ? nc - 1 : cx == nc - 1 ? 0 : -1;  // the cell across a face
+            int b0[R], n0[R], b1[R], n1[R];
 #pragma unroll
-        for (int r = 0; r < R; ++r) {
-            const int o = lane + r * L;
-            int z = cz + o / 3 - 1, y = cy + o % 3 - 1;
-            z = z < 0 ? z + nc : (z >= nc ? z - nc : z);
-            y = y < 0 ? y + nc : (y >= nc ? y - nc : y);
-            const int base = (z * nc + y) * nc;
-            b0[r] = n0[r] = b1[r] = n1[r] = 0;
-            if (o < 9) {
-                b0[r] = __ldg(cell_start + base + xa);
-                n0[r] = __ldg(cell_start + base + xb + 1) - b0[r];
-                if (xw >= 0) {
-                    b1[r] = __ldg(cell_start + base + xw);
-                    n1[r] = __ldg(cell_start + base + xw + 1) - b1[r];
+            for (int r = 0; r < R; ++r) {
+                const int o = lane + r * L;
+                int z = cz + o / 3 - 1, y = cy + o % 3 - 1;
+                z = z < 0 ? z + nc : (z >= nc ? z - nc : z);
+                y = y < 0 ? y + nc : (y >= nc ? y - nc : y);
+                const int base = (z * nc + y) * nc;
+                b0[r] = n0[r] = b1[r] = n1[r] = 0;
+                if (o < 9) {
+                    b0[r] = __ldg(cell_start + base + xa);
+                    n0[r] = __ldg(cell_start + base + xb + 1) - b0[r];
+                    if (xw >= 0) {
+                        b1[r] = __ldg(cell_start + base + xw);
+                        n1[r] = __ldg(cell_start + base + xw + 1) - b1[r];
+                    }
                 }
             }
-        }
 #pragma unroll
-        for (int r = 0; r < R; ++r)
-            for (int q = 0; q < n0[r] + n1[r]; q += 4) {
-                float4 pj[4];
+            for (int r = 0; r < R; ++r)
+                for (int q = 0; q < n0[r] + n1[r]; q += 4) {
+                    float4 pj[4];
 #pragma unroll
-                for (int u = 0; u < 4; ++u) {
-                    const int c = q + u < n0[r] + n1[r] ? q + u : q;
-                    pj[u] = __ldg(pos_sorted + (c < n0[r] ? b0[r] + c : b1[r] + c - n0[r]));
+                    for (int u = 0; u < 4; ++u) {
+                        const int c = q + u < n0[r] + n1[r] ? q + u : q;
+                        pj[u] = __ldg(pos_sorted + (c < n0[r] ? b0[r] + c : b1[r] + c - n0[r]));
+                    }
+#pragma unroll
+                    for (int u = 0; u < 4; ++u)
+                        if (q + u < n0[r] + n1[r]) test(pj[u]);
                 }
-#pragma unroll
-                for (int u = 0; u < 4; ++u)
-                    if (q + u < n0[r] + n1[r]) test(pj[u]);
-            }
-    }
-    __syncwarp(gmask);
-    int c = lcnt[grp];
-    if (c > P.maxnb) {
-        if (lane == 0) atomicOr(&ctrl->err, kErrNbrOverflow);
-        c = P.maxnb;
-    }
-    for (int s = lane; s < c; s += L) {
-        const int v = list[s];
-        int r = 0;
-        for (int q = 0; q < c; ++q) r += list[q] < v;
-        nbr[(size_t)r * P.n_pad + id] = v;
-    }
-    if (lane == 0) {
-        nbr_cnt[id] = c;
-        perm[k] = id;
-        disp_build[id] = disp[id];
-    }
-    __syncwarp(gmask);  // the scratch is read before the next particle's
+        }
+        __syncwarp(gmask);
+        int c = lcnt[grp];
+        if (c > P.maxnb) {
+            if (lane == 0) atomicOr(&ctrl->err, kErrNbrOverflow);
+            c = P.maxnb;
+        }
+        for (int s = lane; s < c; s += L) {
+            const int v = list[s];
+            int r = 0;
+            for (int q = 0; q < c; ++q) r += list[q] < v;
+            nbr[(size_t)r * P.n_pad + id] = v;
+        }
+        if (lane == 0) {
+            nbr_cnt[id] = c;
+            perm[k] = id;
+            disp_build[id] = disp[id];
+        }
+        __syncwarp(gmask);  // the scratch is read before the next particle's
     }
 }
 
@@ -2002,7 +2002,7 @@ cudaError_t launch_rebuild(const StepParams& P, const ParticleBuffers& B, cudaSt
     cudaError_t e = launch_cell_build(P, B, B.pos_next, B.ctrl->rebuild, st);
     if (e != cudaSuccess) return e;
     if (P.maxnb <= kNbrSortCap && P.n <= kNbrLanesMaxN)
-        return launch_nbr_lanes(nbr_lanes, std::min((P.n + kNbrGroups - 1) / kNbrGroups, 6 * 152), P.maxnb, st, P, B.ctrl, B.pos_sorted,
+        return launch_nbr_lanes(nbr_lanes, std::min((P.n + kNbrGroups - 1) / kNbrGroups, 6 * kChipSms), P.maxnb, st, P, B.ctrl, B.pos_sorted,
                                 B.cell_start, B.nbr, B.nbr_cnt, B.perm, B.disp, B.disp_build);
     nbr_build<<<(P.n + kThreads - 1) / kThreads, kThreads, 0, st>>>(P, B.ctrl, B.pos_sorted, B.cell_start, B.nbr,
                                                                      B.nbr_cnt, B.perm, B.disp, B.disp_build);

@@ -11,6 +11,8 @@
 
 namespace gld {
 
+constexpr int kChipSms = 152;  // SMs of a GB300, the one target: launch rules stated in threads per SM
+
 // History convolution (k_history.cu).  ctrl != nullptr: the step is read on
 // the device; otherwise `step` is used.  t >= 0: the step is number t of a
 // block of len steps whose parts launch_conv_pre has formed.
