@@ -209,15 +209,18 @@ def kernel_source_hash() -> str:
     return h.hexdigest()[:16]
 
 
-def measured_traffic(workload: str):
+def measured_traffic(workload: str, first: int, steps: int):
     """DRAM bytes per step of the history convolution from the committed ncu
-    summary, if it was taken on the current kernel sources."""
+    summary, if it was taken on the current kernel sources over the same steps
+    (what a step streams depends on its place in the ring)."""
     path = os.path.join(PROFILES, "hist_conv_traffic.json")
     try:
         d = json.load(open(path))
     except Exception:
         return None
-    if d.get("kernel_source_sha256_16") != kernel_source_hash() or d.get("workload") != workload:
+    if d.get("kernel_source_sha256_16") != kernel_source_hash():
+        return None
+    if (d.get("workload"), d.get("first_step"), d.get("steps")) != (workload, first, steps):
         return None
     return d.get("dram_bytes_per_step")
 
@@ -565,9 +568,11 @@ def main():
     prof = sim.profile_steps(args.profile_steps)
     h_ms, prof_steps = prof["hist_conv"][0], prof["cforce"][1]
     nacc, blocked = 2, sim.diag()
-    alg_bytes = conv_bytes(w.n, w.m_max, 2 if args.hist == "bf16" else 4, nacc, bool(args.kahan),
-                           sim.step_index - prof_steps, prof_steps, blocked["conv_ranges"], blocked["conv_block"])
-    kname, traffic = "history convolution (a step's sums and its share of the block's parts)", measured_traffic(args.workload)
+    first = sim.step_index - prof_steps
+    alg_bytes = conv_bytes(w.n, w.m_max, 2 if args.hist == "bf16" else 4, nacc, bool(args.kahan), first, prof_steps,
+                           blocked["conv_ranges"], blocked["conv_block"])
+    kname = "history convolution (a step's sums and its share of the block's parts)"
+    traffic = None if args.kahan or args.hist == "bf16" else measured_traffic(args.workload, first, prof_steps)
     if args.modes:  # per column: Y' of every mode read and written, two ring values, the projections
         nm = len(inputs.memory_modes(w)[0])
         elem = 2 if args.hist == "bf16" else 4
