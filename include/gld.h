@@ -195,8 +195,8 @@ gld_status gld_get_order(gld_ctx* ctx, int32_t* int2ext);
  * used in the last step's pair-correlated noise (gld_set_pair_noise_krylov;
  * 0 when off), steps taken inside one kernel (use_graphs = 1) so far,
  * ranges of slots that a memory sum is split into (0: m_max <= 32 or no
- * kernels), steps of a block whose parts the convolution forms at once (0: it
- * streams whole rings)}.
+ * kernels), steps of a block whose parts the step kernels form at once (0:
+ * they stream whole rings)}.
  * Synchronizes. */
 gld_status gld_get_diag(gld_ctx* ctx, int64_t* out, int32_t count);
 

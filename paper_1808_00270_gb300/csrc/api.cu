@@ -291,6 +291,9 @@ cudaError_t launch_noise(gld_ctx* c, cudaStream_t s)
     return e;
 }
 
+// Whether the step kernels form the convolution in blocks of steps.
+bool in_blocks(const gld_ctx* c) { return c->P.cblk && c->conv_alone; }
+
 // The convolution of step n, whose index the device holds in ctrl->step (or,
 // next, in ctrl->conv_step).  Blocks of conv_len steps start at `origin` and
 // every conv_len steps on: their first step forms the parts, the others resume
@@ -301,7 +304,7 @@ cudaError_t launch_conv(gld_ctx* c, long long n, long long origin, long long* pa
 {
     const StepParams& P = c->P;
     int t = -1;
-    if (P.cblk) {
+    if (in_blocks(c)) {
         const int rel = (int)((n - origin) % c->conv_len);
         if (rel == 0) {
             const cudaError_t e =
@@ -364,7 +367,7 @@ cudaError_t capture_fork_next(gld_ctx* c, int t, cudaStream_t s)
 {
     cudaError_t e = cudaEventRecord(c->ev_fork, s);
     if (e == cudaSuccess) e = cudaStreamWaitEvent(c->cap3, c->ev_fork, 0);
-    long long part_step = c->P.cblk ? (t + 1) / c->conv_len * c->conv_len : 0;  // by an earlier step of the block
+    long long part_step = in_blocks(c) ? (t + 1) / c->conv_len * c->conv_len : 0;  // by an earlier step of the block
     if (e == cudaSuccess) e = launch_conv(c, t + 1, 0, &part_step, true, c->cap3);
     if (e == cudaSuccess) e = cudaEventRecord(c->ev_join, c->cap3);
     return e;
@@ -374,7 +377,7 @@ cudaError_t capture_fork_next(gld_ctx* c, int t, cudaStream_t s)
 cudaError_t capture_memory(gld_ctx* c, int t, cudaStream_t s)
 {
     if (c->P.nmodes > 0) return launch_memory(c, s);
-    long long part_step = c->P.cblk ? t / c->conv_len * c->conv_len : 0;
+    long long part_step = in_blocks(c) ? t / c->conv_len * c->conv_len : 0;
     return launch_conv(c, t, 0, &part_step, false, s);
 }
 
@@ -742,12 +745,12 @@ gld_status step_cluster(gld_ctx* c, int64_t k, bool boundary)
 // starts from its first step's memory sums and the parts of their block.
 gld_status replay(gld_ctx* c, cudaGraphExec_t g, int steps, bool overlap)
 {
-    if (c->P.cblk && c->part_step != c->host_step) c->conv_valid_step = -1;
+    if (in_blocks(c) && c->part_step != c->host_step) c->conv_valid_step = -1;
     if (overlap) GLD_CUDA(c, launch_memory(c, c->st));
     GLD_CUDA(c, cudaGraphLaunch(g, c->st));
     c->host_step += steps;
     c->conv_valid_step = overlap ? c->host_step : -1;
-    c->part_step = overlap && c->P.cblk ? c->host_step : -1;
+    c->part_step = overlap && in_blocks(c) ? c->host_step : -1;
     return GLD_OK;
 }
 
@@ -798,7 +801,7 @@ constexpr int kConditionalMinN = 262144;
 // convolution.  A program that steps by fewer than 64 otherwise launches every
 // kernel by itself (37 us per step at 10000 particles where a graph takes 20);
 // the piece is captured once some 64 steps went that way.
-int segment_steps(const gld_ctx* c) { return c->P.cblk ? c->conv_len : 8; }
+int segment_steps(const gld_ctx* c) { return in_blocks(c) ? c->conv_len : 8; }
 
 bool capture_segment(gld_ctx* c)
 {
@@ -1255,6 +1258,7 @@ gld_status gld_set_kernels(gld_ctx* c, const double* Ks, int32_t Q, const double
         if (!c->B.part) cudaGetLastError();
         P.cblk = c->B.part ? 1 : 0;
     }
+    c->conv_alone = conv_blocks_alone(P.hist_bf16, P.n_pad, P.m_max, c->prm.kahan, c->conv_G);
     P.nmodes = 0;  // new kernels: back to the ring convolution until modes are set again
     P.pn_deg = 0;  // and to the self-kernel noise until the pair noise is set again
     P.perp = 0;    // and to parallel components only
@@ -1473,7 +1477,7 @@ gld_status gld_get_diag(gld_ctx* c, int64_t* out, int32_t count)
     long long rebuilds = 0;
     GLD_CUDA(c, cudaMemcpy(&rebuilds, &c->B.ctrl->rebuilds, sizeof(rebuilds), cudaMemcpyDeviceToHost));
     const int64_t v[8] = {c->graph_mode,      rebuilds,         c->P.maxnb, c->P.nc,
-                          c->kry.last_iters, c->cluster_steps, c->conv_G,  c->P.cblk ? c->conv_len : 0};
+                          c->kry.last_iters, c->cluster_steps, c->conv_G,  in_blocks(c) ? c->conv_len : 0};
     for (int k = 0; k < count; ++k) out[k] = k < 8 ? v[k] : 0;
     return GLD_OK;
 }
@@ -1607,7 +1611,7 @@ gld_status gld_profile_steps(gld_ctx* c, int64_t nsteps, double* ms, int64_t* la
         c->noise_end = c->host_step + T;
         c->noise_valid = true;
         for (int t = 0; t < T; ++t) {
-            const bool parts = c->P.cblk && c->P.nmodes == 0 && t % c->conv_len == 0;
+            const bool parts = in_blocks(c) && c->P.nmodes == 0 && t % c->conv_len == 0;
             timed(GLD_PROF_HIST, 1 + (parts ? conv_pre_launches(c->P.nacc) : 0), [&] { return launch_memory(c, c->st); });
             if (pnoise) timed(GLD_PROF_PNOISE, sweep_kernels, [&] { return launch_pair_noise(c->P, c->B, c->d_zblk, c->d_bvec, c->st); });
             timed(GLD_PROF_PAIR, 1, [&] { return launch_pair_force_integrate(c->P, c->B, c->st); });

@@ -28,6 +28,7 @@ struct gld_ctx {
     long long eager_steps = 0;       // steps launched kernel by kernel since the graphs were dropped
     bool cluster_graph = false;      // gexec holds a noise block and its steps in one kernel
     long long cluster_steps = 0;     // steps taken inside the cluster kernel so far
+    bool conv_alone = false;         // the step kernels take blocks (conv_blocks_alone)
     int conv_G = 0, conv_len = 0;    // split of a column's slots; steps of a block of the convolution
     long long part_step = -1;        // first step of the block whose parts B.part holds
     std::vector<void*> allocs;

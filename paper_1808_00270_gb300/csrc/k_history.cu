@@ -165,7 +165,7 @@ cudaError_t conv_block_shape(int bf16, int n_pad, int m_max, int nacc, int kahan
 {
     *G = *len = 0;
     *bytes = 0;
-    if (m_max - 1 < kMinBlockedSlots) return cudaSuccess;
+    if (m_max - 1 < (kahan ? 2 : 1) * kMinBlockedSlots) return cudaSuccess;
     Shape sh{};
     const cudaError_t e = by_nacc(nacc, kahan != 0, [&](auto na, auto ka) {
         return bf16 ? shape_of<decltype(na)::value, decltype(ka)::value, true>(n_pad, m_max, &sh)
@@ -177,6 +177,33 @@ cudaError_t conv_block_shape(int bf16, int n_pad, int m_max, int nacc, int kahan
     const int rows = std::max(sh.G * *len, pre_len(kahan, 1));  // alone, and in a batch (one range)
     *bytes = sizeof(float) * (size_t)rows * nacc * (kahan ? 2 : 1) * 3 * n_pad;
     return cudaSuccess;
+}
+
+// A system alone runs the convolution beside its list build and F^C, so blocks
+// have to save more than their parts' launch: the ring must be long, the longer
+// the fewer its columns.  Time per step with whole sums over time with blocks, at
+// H slots (one pair term, graphs):
+//   FP32           4097: 0.96 at 100, 0.98 at 160, 1.08 at 200   16384: 0.99 at 128, 1.09 at 160
+//                 40000: 0.99 at 80, 1.03 at 100, 1.08 at 128    65536: 1.00 at 64, 1.05 at 100, 1.15 at 128
+//                262144: 1.03 at 32, 1.11 at 64, 1.22 at 128    600000: 0.98 at 49, 1.06 at 64, 1.18 at 128
+//   BF16          16384: 0.96 at 100, 1.05 at 128   100000: 0.97 at 100, 1.02 at 128   160000: 0.99 at 80, 1.01 at 100
+//                262144: 1.00 at 49, 1.03 at 64     600000: 0.98 at 49, 1.03 at 64
+// Compensated sums have one range at every size and are bound by operations once
+// their columns fill the chip; blocks save loads, not operations.
+//   FP32          16384: 0.96 at 80, 1.05 at 100     40000: 0.97 at 100, 1.01 at 128   160000: 0.98 at 49, 1.02 at 64
+//   BF16          16384: 1.00 at 80, 1.16 at 100     65536: 0.95 at 80, 1.03 at 100    100000: 0.96 at 128, 1.00 at 160
+//                262144: 0.96 at 32, 0.93 at 160, 0.95 at 300
+bool conv_blocks_alone(int bf16, int n_pad, int m_max, int kahan, int G)
+{
+    const int H = m_max - 1;
+    const long long per_sm = 3LL * n_pad / (bf16 ? 8 : 4) / kChipSms;  // 16-byte columns
+    if (kahan) {
+        if (per_sm >= 512) return !bf16 && H >= 64;
+        return H >= (bf16 && per_sm >= 192 ? 160 : 96);
+    }
+    if (G == 1) return H >= 56;
+    if (G == 2) return H >= (bf16 ? 96 : 56);
+    return H >= (bf16 ? 128 : per_sm >= 160 ? 96 : 160);
 }
 
 cudaError_t launch_hist_conv(const void* ring, int bf16, int n_pad, int m_max, const Ctrl* ctrl,

@@ -56,7 +56,7 @@ def _result(g):
 
 # four ranges of slots, in FP32 and BF16; steps in a cluster and step kernels;
 # past the cluster kernel
-@pytest.mark.parametrize("n,m_max,kw", [(300, 100, {}), (1000, 131, dict(hist_dtype="bf16")), (6000, 70, {}), (500, 60, dict(kahan=True))])
+@pytest.mark.parametrize("n,m_max,kw", [(300, 100, {}), (1000, 131, dict(hist_dtype="bf16")), (6000, 70, {}), (500, 70, dict(kahan=True))])
 def test_alone(n, m_max, kw, monkeypatch):
     got = []
     for graphs, refuse in ((1, True), (2, True), (0, True), (1, False)):
