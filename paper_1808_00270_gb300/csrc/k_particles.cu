@@ -27,6 +27,7 @@
 // neighbours lie close in memory; ids never change, so the displacement
 // history is never permuted.
 #include <algorithm>
+#include <cmath>
 
 #include <cuda_bf16.h>
 
@@ -2073,9 +2074,21 @@ cudaError_t pn_sweeps_room(const StepParams& P, int* found)
     if (e != cudaSuccess) return e;
     const int grid = (P.n + kSweepThreads - 1) / kSweepThreads, per_sm = (grid + sms - 1) / sms;
     // pairs per thread: the list's capacity, or what the blocks of an SM share
-    // of 200 KB; lists hold about 1.7 times the pairs inside the cutoff
+    // of 200 KB
     const int room = std::min(P.maxnb, (int)(200 * 1024 / ((size_t)per_sm * 20 * kSweepThreads)));
-    if (!coop || per_sm > 8 || room < 8) return cudaSuccess;
+    // A launch each costs the same for every sweep; here the first pass costs
+    // more and a sweep less, the less the more blocks share an SM, and nothing is
+    // gained once many particles have more pairs than room.  us per step, a
+    // launch each / one launch, at the mean number of pairs inside the cutoff:
+    //   32768 particles (2 blocks per SM)  degree 2, 1.7 pairs: 34.9 / 33.1, 13 pairs: 69.6 / 63.1
+    //                                      degree 8, 1.7 pairs: 76.8 / 59.5, 13 pairs: 175.6 / 112.5
+    //   65536 (4, room for 20)  degree 2: 42.3 / 42.5, 86.4 / 88.7      degree 8: 88.1 / 77.2, 198 / 164
+    //                           17 pairs, degree 2: 107 / 118           degree 8: 244 / 229
+    //   90000 (5, 16)           degree 2: 49.2 / 51.0, 103 / 111        degree 8: 96.8 / 91.9, 231 / 216
+    //                           17 pairs                                degree 8: 280 / 303
+    //   110000 (6, 13)          degree 8: 102.6 / 102.9, 233 / 270     131072 (7, 11): 115 / 119, 267 / 323
+    const double pairs = P.n / ((double)P.box * P.box * P.box) * 4.18879020478639 * std::pow((double)P.rc2, 1.5);
+    if (!coop || room < 8 || pairs > 0.8 * room || per_sm > 5 || P.pn_deg < per_sm - 1) return cudaSuccess;
     const size_t smem = (size_t)20 * kSweepThreads * room;
     if ((e = allow_smem(pn_sweeps, smem)) != cudaSuccess) return e;
     int occ = 0;
