@@ -181,29 +181,32 @@ cudaError_t conv_block_shape(int bf16, int n_pad, int m_max, int nacc, int kahan
 
 // A system alone runs the convolution beside its list build and F^C, so blocks
 // have to save more than their parts' launch: the ring must be long, the longer
-// the fewer its columns.  Time per step with whole sums over time with blocks, at
-// H slots (one pair term, graphs):
-//   FP32           4097: 0.96 at 100, 0.98 at 160, 1.08 at 200   16384: 0.99 at 128, 1.09 at 160
-//                 40000: 0.99 at 80, 1.03 at 100, 1.08 at 128    65536: 1.00 at 64, 1.05 at 100, 1.15 at 128
-//                262144: 1.03 at 32, 1.11 at 64, 1.22 at 128    600000: 0.98 at 49, 1.06 at 64, 1.18 at 128
-//   BF16          16384: 0.96 at 100, 1.05 at 128   100000: 0.97 at 100, 1.02 at 128   160000: 0.99 at 80, 1.01 at 100
-//                262144: 1.00 at 49, 1.03 at 64     600000: 0.98 at 49, 1.03 at 64
+// the fewer its columns.  Time per step with whole sums over time with blocks at
+// H slots (one pair term, graphs; 3 and 11 neighbours in a list):
+//   FP32            4097: 0.95-0.98 at 160, 1.00-1.08 at 200    8192: 0.98-1.01 at 128, 1.05-1.08 at 160
+//                  16384: 0.96-1.07 at 100, 0.99-1.14 at 128   40000: 1.00-1.02 at 80, 1.03-1.07 at 100
+//                  65536: 1.00-1.09 at 64, 1.05-1.16 at 100   262144: 1.04 at 49, 1.11 at 64, 1.22 at 128
+//                 600000: 0.98 at 49, 1.06 at 64, 1.18 at 128
+//   BF16            8192: 0.98-1.00 at 128, 1.05-1.10 at 160   20000: 1.01 at 128, 1.11 at 160
+//                 100000: 1.02 at 128, 1.07-1.08 at 160       160000: 0.99 at 80, 1.01 at 100, 1.04 at 128
+//                 262144: 1.00 at 49, 1.03 at 64              600000: 0.98 at 49, 1.03 at 64
 // Compensated sums have one range at every size and are bound by operations once
 // their columns fill the chip; blocks save loads, not operations.
-//   FP32          16384: 0.96 at 80, 1.05 at 100     40000: 0.97 at 100, 1.01 at 128   160000: 0.98 at 49, 1.02 at 64
-//   BF16          16384: 1.00 at 80, 1.16 at 100     65536: 0.95 at 80, 1.03 at 100    100000: 0.96 at 128, 1.00 at 160
-//                262144: 0.96 at 32, 0.93 at 160, 0.95 at 300
+//   FP32            8192: 0.98 at 80, 1.04 at 100              20000: 1.01 at 128, 1.08 at 160
+//                  40000: 0.93-1.01 at 128, 0.98-1.09 at 160  160000: 0.98 at 49, 1.02 at 64, 1.09 at 128
+//   BF16           20000: 1.02 at 80, 1.16 at 100              40000: 0.96-1.04 at 80, 1.07-1.17 at 100
+//                 100000: 0.99-1.00 at 160, 1.06 at 200       262144: 0.96 at 32, 0.93 at 160, 0.95 at 300
 bool conv_blocks_alone(int bf16, int n_pad, int m_max, int kahan, int G)
 {
     const int H = m_max - 1;
     const long long per_sm = 3LL * n_pad / (bf16 ? 8 : 4) / kChipSms;  // 16-byte columns
     if (kahan) {
         if (per_sm >= 512) return !bf16 && H >= 64;
-        return H >= (bf16 && per_sm >= 192 ? 160 : 96);
+        return H >= (bf16 ? (per_sm >= 192 ? 192 : 96) : per_sm >= 64 ? 160 : 96);
     }
     if (G == 1) return H >= 56;
     if (G == 2) return H >= (bf16 ? 96 : 56);
-    return H >= (bf16 ? 128 : per_sm >= 160 ? 96 : 160);
+    return H >= (bf16 ? 144 : per_sm >= 64 ? 96 : per_sm >= 32 ? 144 : 192);
 }
 
 cudaError_t launch_hist_conv(const void* ring, int bf16, int n_pad, int m_max, const Ctrl* ctrl,

@@ -17,11 +17,11 @@ def _cuda():
     torch.cuda.set_device(0)
 
 
-# four ranges, few and many columns; two; one; BF16; compensated sums of few and
-# many columns
-LINES = [(5000, 160, "f32", False), (40001, 96, "f32", False), (90001, 56, "f32", False), (150001, 56, "f32", False),
-         (12001, 128, "bf16", False), (140001, 96, "bf16", False), (300001, 56, "bf16", False),
-         (5000, 96, "f32", True), (120001, 64, "f32", True), (12001, 96, "bf16", True), (100001, 160, "bf16", True)]
+# four ranges of few, more and many columns; two; one; BF16; compensated sums of
+# few and many columns
+LINES = [(5000, 192, "f32", False), (8193, 144, "f32", False), (40001, 96, "f32", False), (90001, 56, "f32", False), (150001, 56, "f32", False),
+         (12001, 144, "bf16", False), (140001, 96, "bf16", False), (300001, 56, "bf16", False),
+         (5000, 96, "f32", True), (30001, 160, "f32", True), (120001, 64, "f32", True), (12001, 96, "bf16", True), (100001, 192, "bf16", True)]
 
 
 @pytest.mark.parametrize("n,slots,hist,kahan", LINES)

@@ -23,7 +23,7 @@ def _workload(n, m_max):
 
 # blocks of 8 steps (a split into ranges) and of 16, memories too short for
 # blocks; lists built by one kernel and by four
-@pytest.mark.parametrize("n,m_max,block,lists", [(4097, 170, 8, 1), (8193, 170, 8, 4), (150001, 66, 16, 4), (5000, 100, 0, 1), (5000, 32, 0, 1)])
+@pytest.mark.parametrize("n,m_max,block,lists", [(4097, 200, 8, 1), (8193, 170, 8, 4), (150001, 66, 16, 4), (5000, 100, 0, 1), (5000, 32, 0, 1)])
 def test_launches_of_a_step(n, m_max, block, lists):
     g = make_gpu(_workload(n, m_max), psd_clamp=True)
     d = g.diag()
@@ -36,7 +36,7 @@ def test_launches_of_a_step(n, m_max, block, lists):
 
 
 def test_launches_of_three_accumulators():
-    w = _workload(4097, 170)
+    w = _workload(4097, 200)
     g = make_gpu(w)
     ks, gk, f, dr = kernels(w)
     g.set_kernels(ks, g=gk, f=f, dr=dr, gs=0.5 * gk, fs=0.3 * f)
