@@ -23,6 +23,7 @@
 // behind the cluster barrier (release / acquire), never through the read-only
 // path.
 #include <algorithm>
+#include <cmath>
 
 #include <cuda_bf16.h>
 
@@ -766,6 +767,10 @@ bool cluster_ok(const StepParams& P, int kahan)
     int ctas = 0;
     size_t smem = 0;
     const StepsKernel kern = steps_kernel(P, &ctas, &smem);
+    // long lists: the chip's other SMs win over the launches they cost (launch.h)
+    const double list = P.n / ((double)P.box * P.box * P.box) * 4.18879020478639 * std::pow((double)P.rl2, 1.5);
+    const int lanes = cluster_lanes(P.n, ctas);
+    if (lanes < 8 && list > (lanes == 4 ? 24.0 : 8.0)) return false;
     return cluster_fits(kern, ctas, smem);
 }
 

@@ -208,6 +208,10 @@ cudaError_t launch_batch_noise(const BatchPlan& bp, cudaStream_t st);     // k_n
 // 4096, and 27.5, 23.3 / 27.3 there with m_max = 400.  Calls of eight steps and more
 // take the cluster too; replayed pieces of a block are faster for those above
 // kClusterBlockMaxN: 12.7 / 11.7 at 256, 16.3 / 12.4 at 2048, 19.2 / 13.5 at 4096.
+// With fewer than eight lanes per particle long lists keep the 16 SMs too busy:
+// time of the step kernels over the cluster's, single steps at 3, 12, 23 and 35
+// entries (m_max = 100): 1.34, 1.15, 1.03, 0.78 at 2048 particles, 1.31, 0.90, 0.67,
+// 0.48 at 4096 (1.05 at 6), but 1.39, 1.29, 1.17, 1.02 with eight lanes at 1024.
 constexpr int kClusterMaxN = 4096;
 constexpr int kClusterBlockMaxN = 192;
 bool cluster_ok(const StepParams& P, int kahan);
