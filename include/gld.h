@@ -434,7 +434,7 @@ gld_status gld_get_bytes(gld_ctx* ctx, int64_t* bytes);
  * device (the VACF partial sums scale with its SM count); no device memory
  * is touched.  The history ring is (m_max-1)*3*n_pad*{4,2} bytes of it, the
  * white-noise window (64 + 2(m_max-1))*3*n_pad*4 bytes, the parts of a block of
- * steps (m_max > 32) 16 or, for small systems, 32 times (1+Q+Qs)*3*n_pad*4. */
+ * steps (m_max > 32, with compensated sums > 64) 16 or, for small systems, 32 times (1+Q+Qs)*3*n_pad*4. */
 gld_status gld_bytes_needed(const gld_params* params, int32_t Q, int32_t Qs, int32_t nr, int64_t* bytes);
 
 const char* gld_last_error(const gld_ctx* ctx);
