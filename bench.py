@@ -51,7 +51,7 @@ def parse():
     ap.add_argument("--serve-requests", type=int, default=60,
                     help="requests of the serving trace summarised in the headline line (0: none)")
     ap.add_argument("--graph-form", default="conditional", choices=["conditional", "gated"],
-                    help="gated: rebuild kernels gated on the device at every size, no cluster kernels "
+                    help="gated: rebuild kernels gated on the device instead of a conditional graph node "
                          "(every graph node a plain kernel, which per-kernel profilers can capture)")
     ap.add_argument("--modes", action="store_true",
                     help="memory sums in auxiliary-variable form (the workload's kernels are sums of damped modes) "

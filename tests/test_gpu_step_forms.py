@@ -17,7 +17,7 @@ def _cuda():
     torch.cuda.set_device(0)
 
 
-def _three_forms(n, m_max, calls, history=True):
+def _three_forms(n, m_max, calls):
     from paper_1808_00270_gb300 import ARR_DISP, ARR_FC, ARR_FD, ARR_FR, ARR_HIST, inputs
     w = inputs.Workload("form", n=n, box=inputs.box_for_density(n, 0.1), m_max=m_max, dt=0.01, r_c=2.0, tau_s=0.2,
                         tau_p=0.1, steps=1, seed=7)
@@ -27,8 +27,7 @@ def _three_forms(n, m_max, calls, history=True):
         for k in calls:
             g.step(k)
         diag.append(g.diag())
-        arrays = (ARR_DISP, ARR_FC, ARR_FD, ARR_FR) + ((ARR_HIST,) if history else ())
-        got.append([*g.get_state()] + [g.get(a) for a in arrays])
+        got.append([*g.get_state()] + [g.get(a) for a in (ARR_DISP, ARR_FC, ARR_FD, ARR_FR, ARR_HIST)])
         g.close()
     for other in got[1:]:
         for x, y in zip(got[0], other):
@@ -47,5 +46,5 @@ def test_small_systems(n):
 
 def test_rebuild_in_a_conditional_node():
     """Blocks, single steps until pieces of a block are replayed, pieces, a block."""
-    d0, d1, d2 = _three_forms(2000000, 40, [64, 64] + [1] * 70 + [10, 32, 16, 64], history=False)
+    d0, d1, d2 = _three_forms(262144, 40, [64, 64] + [1] * 70 + [10, 32, 16, 64])
     assert (d0["graph_mode"], d1["graph_mode"], d2["graph_mode"]) == (0, 2, 1)
