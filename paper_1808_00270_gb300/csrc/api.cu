@@ -793,8 +793,11 @@ bool capture_graph_mode(gld_ctx* c, bool conditional, int steps, bool noise, cud
 
 // Particles from which the rebuild goes into a conditional node: the node costs
 // about 7 us per step, the gated kernels that find nothing to do less than that
-// below (32768: 40.4 against 32.8 us per step, 131072: 98.8 against 92.9,
-// 262144: 185.5 against 185.7).
+// below (us per step, node / gated: 32768: 40.4 / 32.8, 131072: 98.8 / 92.9).  Here
+// it depends: behind the long convolution of the suspension (262144, m_max = 400)
+// and with lists that last the node costs nothing, 190.7 / 191.9 over 4096 steps,
+// but 198 / 190 in its first 500; with m_max = 100 83.2 / 74.7; 500000: 147.6 /
+// 143.1, 1000000: 291.1 / 283.5, 2000000: 555.1 / 555.3, 3000000: 812.4 / 819.1.
 constexpr int kConditionalMinN = 262144;
 
 // Steps of a piece of a noise block that is replayed as a graph: a block of the
