@@ -1261,7 +1261,7 @@ gld_status gld_set_kernels(gld_ctx* c, const double* Ks, int32_t Q, const double
         if (!c->B.part) cudaGetLastError();
         P.cblk = c->B.part ? 1 : 0;
     }
-    c->conv_alone = conv_blocks_alone(P.hist_bf16, P.n_pad, P.m_max, c->prm.kahan, c->conv_G);
+    c->conv_alone = conv_blocks_alone(P.hist_bf16, P.n_pad, P.m_max, P.nacc, c->prm.kahan);
     P.nmodes = 0;  // new kernels: back to the ring convolution until modes are set again
     P.pn_deg = 0;  // and to the self-kernel noise until the pair noise is set again
     P.perp = 0;    // and to parallel components only

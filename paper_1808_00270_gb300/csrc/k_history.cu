@@ -159,6 +159,14 @@ cudaError_t dispatch(int nacc, int kahan, const void* ring, int bf16, int n_pad,
     });
 }
 
+cudaError_t shape_for(int bf16, int n_pad, int m_max, int nacc, int kahan, Shape* sh)
+{
+    return by_nacc(nacc, kahan != 0, [&](auto na, auto ka) {
+        return bf16 ? shape_of<decltype(na)::value, decltype(ka)::value, true>(n_pad, m_max, sh)
+                    : shape_of<decltype(na)::value, decltype(ka)::value, false>(n_pad, m_max, sh);
+    });
+}
+
 }  // namespace
 
 cudaError_t conv_block_shape(int bf16, int n_pad, int m_max, int nacc, int kahan, int* G, int* len, size_t* bytes)
@@ -167,10 +175,7 @@ cudaError_t conv_block_shape(int bf16, int n_pad, int m_max, int nacc, int kahan
     *bytes = 0;
     if (m_max - 1 < (kahan ? 2 : 1) * kMinBlockedSlots) return cudaSuccess;
     Shape sh{};
-    const cudaError_t e = by_nacc(nacc, kahan != 0, [&](auto na, auto ka) {
-        return bf16 ? shape_of<decltype(na)::value, decltype(ka)::value, true>(n_pad, m_max, &sh)
-                    : shape_of<decltype(na)::value, decltype(ka)::value, false>(n_pad, m_max, &sh);
-    });
+    const cudaError_t e = shape_for(bf16, n_pad, m_max, nacc, kahan, &sh);
     if (e != cudaSuccess) return e;
     *G = sh.G;
     *len = pre_len(kahan, sh.G);
@@ -185,7 +190,7 @@ cudaError_t conv_block_shape(int bf16, int n_pad, int m_max, int nacc, int kahan
 // H slots (one pair term, graphs; 3 and 11 neighbours in a list):
 //   FP32            4097: 0.95-0.98 at 160, 1.00-1.08 at 200    8192: 0.98-1.01 at 128, 1.05-1.08 at 160
 //                  16384: 0.96-1.07 at 100, 0.99-1.14 at 128   40000: 1.00-1.02 at 80, 1.03-1.07 at 100
-//                  65536: 1.00-1.09 at 64, 1.05-1.16 at 100   262144: 1.04 at 49, 1.11 at 64, 1.22 at 128
+//                  65536: 1.00-1.09 at 64, 1.05-1.16 at 100   262144: 1.03 at 32, 1.11 at 64, 1.22 at 128
 //                 600000: 0.98 at 49, 1.06 at 64, 1.18 at 128
 //   BF16            8192: 0.98-1.00 at 128, 1.05-1.10 at 160   20000: 1.01 at 128, 1.11 at 160
 //                 100000: 1.02 at 128, 1.07-1.08 at 160       160000: 0.99 at 80, 1.01 at 100, 1.04 at 128
@@ -196,17 +201,20 @@ cudaError_t conv_block_shape(int bf16, int n_pad, int m_max, int nacc, int kahan
 //                  40000: 0.93-1.01 at 128, 0.98-1.09 at 160  160000: 0.98 at 49, 1.02 at 64, 1.09 at 128
 //   BF16           20000: 1.02 at 80, 1.16 at 100              40000: 0.96-1.04 at 80, 1.07-1.17 at 100
 //                 100000: 0.99-1.00 at 160, 1.06 at 200       262144: 0.96 at 32, 0.93 at 160, 0.95 at 300
-bool conv_blocks_alone(int bf16, int n_pad, int m_max, int kahan, int G)
+bool conv_blocks_alone(int bf16, int n_pad, int m_max, int nacc, int kahan)
 {
     const int H = m_max - 1;
+    if (H < kMinBlockedSlots) return false;
+    Shape sh{};
+    if (shape_for(bf16, n_pad, m_max, nacc, kahan, &sh) != cudaSuccess) return false;
     const long long per_sm = 3LL * n_pad / (bf16 ? 8 : 4) / kChipSms;  // 16-byte columns
     if (kahan) {
         if (per_sm >= 512) return !bf16 && H >= 64;
         return H >= (bf16 ? (per_sm >= 192 ? 192 : 96) : per_sm >= 64 ? 160 : 96);
     }
-    if (G == 1) return H >= 56;
-    if (G == 2) return H >= (bf16 ? 96 : 56);
-    return H >= (bf16 ? 144 : per_sm >= 64 ? 96 : per_sm >= 32 ? 144 : 192);
+    if (sh.G == 1) return H >= (sh.kind == 0 ? 32 : 56);  // (columns of one wave, or more)
+    if (sh.G == 2) return H >= (bf16 ? 96 : 56);
+    return H >= (bf16 ? 144 : per_sm >= 56 ? 96 : per_sm >= 32 ? 144 : 192);
 }
 
 cudaError_t launch_hist_conv(const void* ring, int bf16, int n_pad, int m_max, const Ctrl* ctrl,

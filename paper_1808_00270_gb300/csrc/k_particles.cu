@@ -2088,7 +2088,7 @@ cudaError_t pn_sweeps_room(const StepParams& P, int* found)
     //                           17 pairs                                degree 8: 280 / 303
     //   110000 (6, 13)          degree 8: 102.6 / 102.9, 233 / 270     131072 (7, 11): 115 / 119, 267 / 323
     const double pairs = P.n / ((double)P.box * P.box * P.box) * 4.18879020478639 * std::pow((double)P.rc2, 1.5);
-    if (!coop || room < 8 || pairs > 0.8 * room || per_sm > 5 || P.pn_deg < per_sm - 1) return cudaSuccess;
+    if (!coop || room < 8 || pairs > 0.85 * room || per_sm > 5 || P.pn_deg < per_sm - 1) return cudaSuccess;
     const size_t smem = (size_t)20 * kSweepThreads * room;
     if ((e = allow_smem(pn_sweeps, smem)) != cudaSuccess) return e;
     int occ = 0;

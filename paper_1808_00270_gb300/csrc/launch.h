@@ -38,7 +38,7 @@ cudaError_t launch_hist_conv_next(const void* ring, int bf16, int n_pad, int m_m
 constexpr int kMinBlockedSlots = 32;
 cudaError_t conv_block_shape(int bf16, int n_pad, int m_max, int nacc, int kahan, int* G, int* len, size_t* bytes);
 // Whether the step kernels of a system alone take blocks, whose parts it has.
-bool conv_blocks_alone(int bf16, int n_pad, int m_max, int kahan, int G);
+bool conv_blocks_alone(int bf16, int n_pad, int m_max, int nacc, int kahan);
 cudaError_t launch_conv_pre(const void* ring, int bf16, int n_pad, int m_max, const long long* nstep, const float* coef,
                             int nacc, float* part, int G, int len, int kahan, cudaStream_t st);
 int conv_pre_launches(int nacc);

@@ -28,7 +28,7 @@ def _launches(g, degree):
 @pytest.mark.parametrize("n,rho,degree,one", [
     (38912, 0.05, 2, True), (58368, 0.05, 2, True), (58369, 0.05, 2, False), (77824, 0.05, 3, True),
     (77825, 0.05, 3, False), (97280, 0.05, 4, True), (97281, 0.05, 8, False),
-    (60000, 0.47, 4, True), (60000, 0.49, 4, False)])
+    (60000, 0.50, 4, True), (60000, 0.52, 4, False)])
 def test_where_one_launch_takes_all_sweeps(n, rho, degree, one):
     g = _system(n, rho, degree=degree)
     assert (_launches(g, degree) == 1) == one
@@ -36,11 +36,11 @@ def test_where_one_launch_takes_all_sweeps(n, rho, degree, one):
 
 
 def test_more_pairs_than_a_thread_keeps():
-    """15 pairs on average and room for 20: against a launch per sweep (a vanishing
+    """17 pairs on average and room for 20: against a launch per sweep (a vanishing
     perpendicular factor), which adds nothing but roundings, at most 2 K (pairs + 4)
     of 6e-8 each, adding up at random."""
     from paper_1808_00270_gb300 import ARR_FR
-    a, b = _system(60000, 0.47, degree=4), _system(60000, 0.47, degree=4, perp0=True)
+    a, b = _system(60000, 0.50, degree=4), _system(60000, 0.50, degree=4, perp0=True)
     a.step(1)
     b.step(1)
     assert rel_l2(a.get(ARR_FR), b.get(ARR_FR)) < 1e-5
