@@ -90,9 +90,9 @@ typedef struct gld_params {
     int32_t psd_clamp;   /* 1: clamp negative noise modes to 0 instead of failing    */
     int32_t use_graphs;  /* 1 (default): replay steps from captured CUDA graphs,
                           * list rebuilds gated on the device, from 262144 particles
-                          * on in a conditional node; up to 4096 particles the
-                          * steps of a part of a noise block (up to 192: of any)
-                          * run inside one kernel; 2: graphs of the step
+                          * on in a conditional node; up to 4096 particles (dense
+                          * systems up to 1024) the steps of a part of a noise
+                          * block (up to 192: of any) run inside one kernel; 2: graphs of the step
                           * kernels with gated rebuilds at every size (e.g. for
                           * per-kernel profilers); 0: launch every kernel from the
                           * host.  The bits are the same                       */
